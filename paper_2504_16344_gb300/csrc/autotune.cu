@@ -121,17 +121,22 @@ tw_status autotune_lane(tw_ctx *c, tw_lane &L) {
     const int k = tw_autotune_pick((int)ms.size(), ms.data());
     if (k >= 0) { t.adj_tile = cand[k]; t.adj_tile_ms = ms[k]; }
   }
-  // 2) FP64-class adjoint: right-hand sides per warp
+  // 2) FP64-class adjoint: on the tensor cores (0), or right-hand sides per warp
   if (c->op[TW_MAP_F][TW_PREC_FP64]) {
     const void *A = c->opG[0] ? c->opG[0] : c->op[TW_MAP_F][0];
-    const int cand[3] = {4, 2, 1};
-    double ms[3];
-    for (int k = 0; k < 3; ++k)
-      ms[k] = time_ms([&] {
+    const int8_t *ea = c->opG[0] ? c->eaG[0] : c->ea[TW_MAP_F][0];
+    const bool tc = ea && L.sl64_ws;
+    const int cand[4] = {0, 4, 2, 1};
+    double ms[4];
+    for (int k = 0; k < 4; ++k)
+      ms[k] = k == 0 && !tc ? -1.0 : time_ms([&] {
+        if (k == 0)
+          return launch_gemm_adj_sl64(A, ea, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm, Nf,
+                                      Nd, Nm, B, L.sl64_ws, L.sl64_ws_n, L.sl64_eb, L.sl64_eb_n, c->d_err, 0);
         return launch_gemm_adj_dd(A, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm, Nf, Nd, Nm,
                                   B, 0, cand[k]);
       });
-    const int k = tw_autotune_pick(3, ms);
+    const int k = tw_autotune_pick(4, ms);
     if (k >= 0) { t.adj_rw = cand[k]; t.adj_rw_ms = ms[k]; }
   }
   // 3) forward products (the forecast's F_q X): lanes per right-hand side

@@ -26,12 +26,16 @@ struct tw_lane {
   void *bsl_ws = nullptr;
   int *bsl_eb = nullptr;
   size_t bsl_ws_n = 0, bsl_eb_n = 0;
+  // the same for the FP64-class adjoint (gemm_sl64.cu); null: its SIMT form runs
+  void *sl64_ws = nullptr;
+  int *sl64_eb = nullptr;
+  size_t sl64_ws_n = 0, sl64_eb_n = 0;
   // tiles of the batched products (tw_batch_tiles): right-hand sides per
   // tensor-core tile (mixed adjoint) and per warp (FP64-class adjoint), lanes
   // per right-hand side (forward products); chosen by measurement at
   // tw_reserve_batch, the same for every lane of a context
   int sl_tile = 0;
-  int adj_rw = 0;
+  int adj_rw = 0;                    // 0: the FP64-class adjoint runs on the tensor cores
   int fwd_lpb = 1;
   size_t bytes = 0;                  // device bytes of the lane
 };
@@ -46,8 +50,9 @@ struct tw_ctx {
   // G^ = F^ C per frequency (the paper's G* = Gamma_pr F* of Phase 2), per kept
   // format, when TW_KEEP_G: the adjoint applies of tw_infer then need no prior filter
   void *opG[3] = {nullptr, nullptr, nullptr};
-  // row exponents of the FP32 storages for the batched adjoint on the tensor
-  // cores: ea[which][fmt][w][m] (fmt 1, 2), eaG[fmt] for G^ (gemm_sl.cu)
+  // row exponents of the stored operators for the batched adjoint on the tensor
+  // cores: ea[which][fmt][w][m], eaG[fmt] for G^ (gemm_sl.cu; fmt 0, F only:
+  // gemm_sl64.cu, null if they did not fit)
   int8_t *ea[2][3] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};
   int8_t *eaG[3] = {nullptr, nullptr, nullptr};
   std::vector<char> loaded[2];     // per row: loaded?

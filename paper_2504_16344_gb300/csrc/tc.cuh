@@ -1,0 +1,213 @@
+// tc.cuh -- building blocks of the tensor-core (tcgen05) kernels whose
+// operands are cut into exact fixed-point bf16 slices: mbarrier waits with a
+// time limit, bulk copies, MMA issue, shared-memory descriptors and the
+// slicing arithmetic.
+#pragma once
+#include <stdint.h>
+
+#include <type_traits>
+#include <utility>
+
+#include "df64.cuh"
+
+namespace tw {
+
+// ------------------------------------------------------------ addresses
+__device__ __forceinline__ uint32_t tc_su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// byte offset of the 16-byte chunk q (0..3) of row r in a K-major tile of 32
+// bf16 per row with the 64-byte swizzle (chunk index XOR bits 1-2 of the row)
+__host__ __device__ __forceinline__ uint32_t tc_swz64(int r, int q) {
+  return (uint32_t)r * 64u + ((uint32_t)(q ^ ((r >> 1) & 3)) << 4);
+}
+// shared-memory matrix descriptor: K-major, 64-byte swizzle, 8-row groups 512
+// bytes apart; bits 46-48 = 0b001 (descriptor version), bits 61-63 = 4 (64B)
+__device__ __forceinline__ uint64_t tc_sdesc64(uint32_t saddr) {
+  uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(512 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)4 << 61;
+  return d;
+}
+// instruction descriptor, kind::f16: D F32, A and B BF16, both K-major
+__host__ __device__ __forceinline__ uint32_t tc_idesc_bf16(int M, int N) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// ------------------------------------------------------------ mbarriers
+__device__ __forceinline__ void tc_mbar_init(uint32_t bar, unsigned count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void tc_mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tc_mbar_arrive_tx(uint32_t bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool tc_mbar_try(uint32_t bar, unsigned parity) {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\t"
+               "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+               "selp.b32 %0, 1, 0, p;\n\t}"
+               : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ unsigned long long tc_time() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+constexpr unsigned long long TC_WAIT_NS = 4000000000ull;   // bound of every wait (4 s)
+// true once the phase of this parity has completed; false after TC_WAIT_NS or
+// (fail != nullptr) once another role of the CTA has failed
+__device__ __forceinline__ bool tc_mbar_wait(uint32_t bar, unsigned parity, volatile int *fail) {
+  unsigned long long t0 = 0;
+  for (unsigned it = 1;; ++it) {
+    if (tc_mbar_try(bar, parity)) return true;
+    if ((it & 255u) == 0) {
+      if (fail && *fail) return false;
+      const unsigned long long t = tc_time();
+      if (t0 == 0) t0 = t;
+      else if (t - t0 > TC_WAIT_NS) return false;
+    }
+  }
+}
+
+// ------------------------------------------------------ copies and MMAs
+__device__ __forceinline__ void tc_bulk_g2s(uint32_t dst, const void *src, unsigned bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+// D (TMEM) (+)= A (TMEM) B (shared memory): bf16 operands, FP32 accumulators
+__device__ __forceinline__ void tc_mma_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile("{\n\t.reg .pred p;\n\t"
+               "setp.ne.b32 p, %4, 0;\n\t"
+               "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+               ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
+}
+__device__ __forceinline__ void tc_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+               ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+// one lane of a converged warp.  MMAs and commits are issued by a warp whose 32
+// lanes run the issuing loop together, one elected lane doing the work of each
+// unrolled group: 15 cycles per 128 x 16 x 16 MMA; issued inside a branch taken by lane 0 alone
+// they took 45 (operands moved to uniform registers one MMA at a time)
+__device__ __forceinline__ bool tc_elect() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.b32 %0, 1, 0, P;\n\t}" : "=r"(p));
+  return p != 0;
+}
+// TMEM stores: 4 consecutive columns of the warp's 32 lanes
+__device__ __forceinline__ void tc_st4(uint32_t addr, const uint32_t *v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};"
+               ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tc_ld4(uint32_t *v, uint32_t addr) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr));
+}
+__device__ __forceinline__ void tc_ld2(uint32_t *v, uint32_t addr) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(addr));
+}
+__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// ------------------------------------------------------------ slicing
+// 2^e as a float, e in [-126, 127]
+__device__ __forceinline__ float tc_pow2f(int e) { return __int_as_float((e + 127) << 23); }
+// bf16 bits of two floats of at most 8 significant bits (exact): upper halves
+__device__ __forceinline__ uint32_t tc_pack_bf16(float lo, float hi) {
+  return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
+}
+// smallest e in [-100, 127] with |hi + lo| < 2^e for every float pair whose
+// |hi| <= mx (the low half may lift the sum past mx by one unit in the last
+// place); the upper clamp keeps e in 8 bits and costs one bit of headroom
+__device__ __forceinline__ int tc_exp_above(float mx) {
+  mx *= 1.0f + 1.0f / 1048576.0f;
+  if (!(mx > 0.f)) return -100;
+  const int e = (int)((__float_as_uint(mx) >> 23) & 0xffu) - 126;
+  return e < -100 ? -100 : (e > 127 ? 127 : e);
+}
+
+// Seven 8-bit slices of a float pair scaled to |hi + lo| < 2^7: step s rounds
+// what is left to a multiple of 2^-8s (adding and subtracting 1.5 2^(23-8s)),
+//   hi + lo = s0 + s1 + ... + s6 + r,  |s_p| <= 2^(7-8p) (s2: 129/128 of it), |r| <= 2^-49,
+// every s_p an integer of at most 8 significant bits times 2^-8p: exact in
+// bf16.  The first two steps act on hi alone (exact); what is left of it is
+// then joined with lo (TwoSum, its error added back before slice 4).
+struct Slicer7 {
+  float r, e;
+  __device__ __forceinline__ void init(float hi, float lo) { r = hi; e = lo; }
+  template <int S> __device__ __forceinline__ float next() {
+    if (S == 2) two_sum(r, e, r, e);
+    if (S == 4) r = __fadd_rn(r, e);
+    const float M = 1.5f * (float)(1 << 23) / (float)(1ull << (8 * S));
+    const float s = __fsub_rn(__fadd_rn(r, M), M);
+    r = __fsub_rn(r, s);
+    return s;
+  }
+};
+
+// f(integral_constant<int, S>) for S = 0..6, in order
+template <class F> __device__ __forceinline__ void for_slices7(F &f) {
+  f(std::integral_constant<int, 0>{});
+  f(std::integral_constant<int, 1>{});
+  f(std::integral_constant<int, 2>{});
+  f(std::integral_constant<int, 3>{});
+  f(std::integral_constant<int, 4>{});
+  f(std::integral_constant<int, 5>{});
+  f(std::integral_constant<int, 6>{});
+}
+
+// ------------------------------------------- products of seven slices
+constexpr int TC_NSL = 7;                // slices per operand
+constexpr int TC_NACC = 6;               // accumulators: levels 0..4, and 5..6
+constexpr int TC_NPAIR = 28;             // slice pairs of levels 0..6
+// level of slice pair p = 0..27 (levels in order, pair (i, L - i) of level L)
+__host__ __device__ constexpr int tc_pair_level(int p) {
+  int l = 0, first = 0;
+  while (p >= first + l + 1) { first += l + 1; ++l; }
+  return l;
+}
+// the MMA of slice pair PR: operand addresses are compile-time selections of
+// the precomputed ones, so the issuing thread spends a few instructions on it
+// (computing the pair's descriptors in the loop cost about 50 cycles an MMA)
+template <bool FIRST, int PR>
+__device__ __forceinline__ void tc_issue_pair(const uint32_t *d, uint32_t a, const uint64_t *b, uint32_t idesc) {
+  constexpr int L = tc_pair_level(PR), si = PR - L * (L + 1) / 2, sj = L - si;
+  constexpr int ac = L < 5 ? L : 5;
+  // the first MMA of a chunk into each accumulator overwrites it
+  tc_mma_ts(d[ac], a + 8u * si, b[sj], idesc, FIRST && si == 0 && L < 6 ? 0u : 1u);
+}
+template <bool FIRST, int P0, int... PR>
+__device__ __forceinline__ void tc_issue_pairs(std::integer_sequence<int, PR...>, const uint32_t *d, uint32_t a,
+                                            const uint64_t *b, uint32_t idesc) {
+  (tc_issue_pair<FIRST, P0 + PR>(d, a, b, idesc), ...);
+}
+// half H of a stage's pairs (14 each)
+template <int H>
+__device__ __forceinline__ void tc_issue_half(bool first, const uint32_t *d, uint32_t a, const uint64_t *b,
+                                           uint32_t idesc) {
+  if (first)
+    tc_issue_pairs<true, H * TC_NPAIR / 2>(std::make_integer_sequence<int, TC_NPAIR / 2>{}, d, a, b, idesc);
+  else
+    tc_issue_pairs<false, H * TC_NPAIR / 2>(std::make_integer_sequence<int, TC_NPAIR / 2>{}, d, a, b, idesc);
+}
+
+// D0 + .. + D4 + D56 as a float pair.  D_L is a multiple of 2^-8L of at most
+// (L+1) 204 2^(14-8L): a running sum below 2^22 leaves a TwoSum error of at
+// most 2^-3, and adding that to D2 (below 2^7.4, multiples of 2^-16), then to
+// D3 (below 0.8, multiples of 2^-24), is exact in 24 bits; from D4 on the
+// rounding is that of the pair's low half.
+__device__ __forceinline__ dd tc_join_levels(const float *d) {
+  float s, e;
+  two_sum(d[0], d[1], s, e);
+  two_sum(s, __fadd_rn(e, d[2]), s, e);
+  two_sum(s, __fadd_rn(e, d[3]), s, e);
+  return dd_make(s, __fadd_rn(e, __fadd_rn(d[4], d[5])));
+}
+
+}  // namespace tw

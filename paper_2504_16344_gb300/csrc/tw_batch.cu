@@ -121,8 +121,16 @@ tw_status infer_core(tw_ctx *c, tw_lane &L, tw_prec prec, int B, const int *win,
     { twh::Phase p(c, TW_PH_RFFT_DATA, s);
       TW_CUDA(c, launch_rfft_time_dd(by, 1, Nd, Nt, (cdd *)L.byh, Nd, Nd, c->plT, c->twT, c->twL, s, ba_y)); }
     { twh::Phase p(c, TW_PH_GEMV_ADJ, s);
-      TW_CUDA(c, launch_gemm_adj_dd(A, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm,
-                                    Nf, Nd, Nm, B, s, L.adj_rw)); }
+      // tensor cores unless a SIMT tile was chosen (tw_batch_tiles) or their
+      // exponents or workspace did not fit
+      const int8_t *ea = useG ? c->eaG[0] : c->ea[TW_MAP_F][0];
+      if (L.adj_rw == 0 && ea && L.sl64_ws)
+        TW_CUDA(c, launch_gemm_adj_sl64(A, ea, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm,
+                                        Nf, Nd, Nm, B, L.sl64_ws, L.sl64_ws_n, L.sl64_eb, L.sl64_eb_n,
+                                        c->d_err, s));
+      else
+        TW_CUDA(c, launch_gemm_adj_dd(A, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm,
+                                      Nf, Nd, Nm, B, s, L.adj_rw)); }
     { twh::Phase p(c, TW_PH_IRFFT_PARAM, s);
       if (fuse)   // m, then m's spectrum in place of x^ (each CTA owns its columns)
         TW_CUDA(c, launch_irfft_rfft_time_dd((const cdd *)L.bxh, Nm, m, 0, Nm, (cdd *)L.bxh, Nm, Nm, Nt,
@@ -227,13 +235,14 @@ size_t lane_bytes(const tw_ctx *c, int bmax) {
     const int cols = (bmax + 7) / 8 * 8 + 80;
     b += 2 * B * np * sizeof(dd) + sl_ws_bytes(c->Nf, c->Rmax, cols) + sl_eb_bytes(c->Nf, cols);
   }
+  if (c->ea[TW_MAP_F][0]) b += sl64_ws_bytes(c->Nf, c->Nd, bmax) + sl64_eb_bytes(c->Nf, bmax);
   return b;
 }
 
 void free_lane(tw_ctx *c, tw_lane &L) {
   void **bufs[] = {(void **)&L.win_dev, (void **)&L.trsm_prog, (void **)&L.bz, (void **)&L.by,
                    (void **)&L.bzd, (void **)&L.byd, (void **)&L.brd, &L.byh, &L.bxh, &L.bpart,
-                   &L.bsl_ws, (void **)&L.bsl_eb};
+                   &L.bsl_ws, (void **)&L.bsl_eb, &L.sl64_ws, (void **)&L.sl64_eb};
   for (void **b : bufs) { twh::dfree(c, *b); *b = nullptr; }
   L.bmax = 0;
   L.bytes = 0;
@@ -268,6 +277,12 @@ tw_status alloc_lane(tw_ctx *c, tw_lane &L, int bmax) {
     L.bsl_eb_n = sl_eb_bytes(c->Nf, cols);
     L.bsl_ws = take(L.bsl_ws_n);
     L.bsl_eb = (int *)take(L.bsl_eb_n);
+  }
+  if (ok && c->ea[TW_MAP_F][0]) {     // optional: null leaves the SIMT product
+    L.sl64_ws_n = sl64_ws_bytes(c->Nf, c->Nd, bmax);
+    L.sl64_eb_n = sl64_eb_bytes(c->Nf, bmax);
+    L.sl64_eb = (int *)twh::dalloc(c, L.sl64_eb_n);
+    if (L.sl64_eb) L.sl64_ws = twh::dalloc(c, L.sl64_ws_n);
   }
   if (!ok) {
     free_lane(c, L);
