@@ -30,12 +30,13 @@ struct tw_lane {
   void *sl64_ws = nullptr;
   int *sl64_eb = nullptr;
   size_t sl64_ws_n = 0, sl64_eb_n = 0;
+  int8_t *sl64_ex = nullptr;         // [Nf][bmax] exponents of x^ (gemm_fwd_sl64.cu)
   // tiles of the batched products (tw_batch_tiles): right-hand sides per
   // tensor-core tile (mixed adjoint) and per warp (FP64-class adjoint), lanes
   // per right-hand side (forward products); chosen by measurement at
   // tw_reserve_batch, the same for every lane of a context
   int sl_tile = 0;
-  int adj_rw = 0;                    // 0: the FP64-class adjoint runs on the tensor cores
+  int adj_rw = 0;                    // 0: the FP64-class products run on the tensor cores
   int fwd_lpb = 1;
   size_t bytes = 0;                  // device bytes of the lane
 };
@@ -55,6 +56,9 @@ struct tw_ctx {
   // gemm_sl64.cu, null if they did not fit)
   int8_t *ea[2][3] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};
   int8_t *eaG[3] = {nullptr, nullptr, nullptr};
+  // exponents of each row of the FP64-class operators over the grid, ef[which][w][r]
+  // (gemm_fwd_sl64.cu; null if they did not fit)
+  int8_t *ef[2] = {nullptr, nullptr};
   std::vector<char> loaded[2];     // per row: loaded?
   std::vector<unsigned long long> col_hash;   // per row of F: fingerprint of its block column
   // FFT plans and twiddle tables (df64 and float)

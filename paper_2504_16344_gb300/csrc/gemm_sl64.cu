@@ -33,7 +33,7 @@
 // two to four 16-wide A' stages of 7 x 8 columns; for P <= 16 the accumulators
 // are double-buffered as well.
 // Measured (64 right-hand sides, 100 rows, 50,000 grid points, 401 frequencies):
-// 28.2 ms, against 246 ms for the SIMT product and 4.8 ms to read the operator;
+// 25.1 ms (28.2 ms with scalar instead of packed slicing), against 246 ms for the SIMT product and 4.8 ms to read the operator;
 // a stage takes 2,100 cycles where its MMAs need 900 (the accumulators are
 // single-buffered at N = 64, so the MMAs of a tile wait for the drain of the
 // one before).  Issuing the MMAs from one lane's branch instead of an elected
@@ -121,8 +121,9 @@ k_bsl64_build(const cdd *__restrict__ Y, long y_bstride, int Nr, int B, int P, i
   for (int t = threadIdx.x; t < natoms * N * 4; t += blockDim.x) {
     const int a = t / (N * 4), n = (t >> 2) % N, q = t & 3;
     const int part = n >= P, bl = n - part * P, b = nt * P + bl;
-    const float sc = tc_pow2f(7 - e_sh[bl]);
-    Slicer7 sl[8];
+    const float sc1 = tc_pow2f(7 - e_sh[bl]);
+    const f2 sc = f2_make(sc1, sc1);
+    Slicer7 sl[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int s = 16 * a + 4 * q + u;
@@ -130,17 +131,13 @@ k_bsl64_build(const cdd *__restrict__ Y, long y_bstride, int Nr, int B, int P, i
       if (b < B && s < Nr) y = ld_cdd(Y + (size_t)b * y_bstride + (size_t)w * Nr + s);
       // the two reals of this row: (yr, yi) for the real-part column, (yi, -yr) for the imaginary
       const dd v0 = part ? y.im : y.re, v1 = part ? dd_neg(y.re) : y.im;
-      sl[2 * u].init(v0.hi * sc, v0.lo * sc);
-      sl[2 * u + 1].init(v1.hi * sc, v1.lo * sc);
+      sl[u].init(v0.hi, v0.lo, v1.hi, v1.lo, sc);
     }
     uint8_t *at = base + (size_t)a * NSL * slice_bytes + tc_swz64(n, q);
     auto put = [&](auto S) {
       uint32_t wd[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float s0 = sl[2 * u].template next<S.value>(), s1 = sl[2 * u + 1].template next<S.value>();
-        wd[u] = tc_pack_bf16(s0, s1);
-      }
+      for (int u = 0; u < 4; ++u) wd[u] = sl[u].template next<S.value>();
       *reinterpret_cast<uint4 *>(at + S.value * slice_bytes) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
     };
     for_slices7(put);
@@ -285,16 +282,16 @@ k_gemm_adj_sl64(const float4 *__restrict__ A, const int8_t *__restrict__ ea, con
       while (st >= SA) { st -= SA; ++use; }
     };
     for (int i = 0; i < my_tiles && ok; ++i) {
-      const float sc = tc_pow2f(7 - e_next);
+      const float sc1 = tc_pow2f(7 - e_next);
+      const f2 sc = f2_make(sc1, sc1);
       e_next = row_scale_exp(i + 1);
       for (int a = 0; a < natoms; ++a) {
         asm volatile("cp.async.wait_group %0;" ::"n"(RAW_D - 2) : "memory");
-        Slicer7 sl[8];
+        Slicer7 sl[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const float4 v = *reinterpret_cast<const float4 *>(rawp + slot * RAW_SLOT + u * NPROD * 16);
-          sl[2 * u].init(v.x * sc, v.y * sc);
-          sl[2 * u + 1].init(v.z * sc, v.w * sc);
+          sl[u].init(v.x, v.y, v.z, v.w, sc);
         }
         if (++slot == RAW_D) slot = 0;
         load();
@@ -315,10 +312,7 @@ k_gemm_adj_sl64(const float4 *__restrict__ A, const int8_t *__restrict__ ea, con
         auto put = [&](auto S) {
           uint32_t wd[4];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const float s0 = sl[2 * u].template next<S.value>(), s1 = sl[2 * u + 1].template next<S.value>();
-            wd[u] = tc_pack_bf16(s0, s1);
-          }
+          for (int u = 0; u < 4; ++u) wd[u] = sl[u].template next<S.value>();
           tc_st4(at + 8u * S.value, wd);
         };
         for_slices7(put);
@@ -368,19 +362,22 @@ k_gemm_adj_sl64(const float4 *__restrict__ A, const int8_t *__restrict__ ea, con
             tc_fence_before();
             tc_mbar_arrive(tempty(bf));
           }
+          f2 v[NACC], rh, rl, ih, il;                // both columns at once
+#pragma unroll
+          for (int L = 0; L < NACC; ++L) v[L] = f2_make(__uint_as_float(dr[L][0]), __uint_as_float(dr[L][1]));
+          tc_join_levels(v, rh, rl);
+#pragma unroll
+          for (int L = 0; L < NACC; ++L) v[L] = f2_make(__uint_as_float(di[L][0]), __uint_as_float(di[L][1]));
+          tc_join_levels(v, ih, il);
+          const float2 arh = f2_split(rh), arl = f2_split(rl), aih = f2_split(ih), ail = f2_split(il);
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
             if (m >= Nm || b0 + c0 + j >= B) continue;
             const float sb = tc_pow2f(ebw[c0 + j] - 7);
-            float vr[NACC], vi[NACC];
-#pragma unroll
-            for (int L = 0; L < NACC; ++L) {
-              vr[L] = __uint_as_float(dr[L][j]);
-              vi[L] = __uint_as_float(di[L][j]);
-            }
             cdd x;
-            x.re = dd_scale2(dd_scale2(tc_join_levels(vr), sa), sb);
-            x.im = dd_scale2(dd_scale2(tc_join_levels(vi), sa), sb);
+            x.re = dd_make_raw(j ? arh.y : arh.x, j ? arl.y : arl.x);
+            x.im = dd_make_raw(j ? aih.y : aih.x, j ? ail.y : ail.x);
+            x = cdd_scale2(cdd_scale2(x, sa), sb);
             cdd *xo = xp + (size_t)(c0 + j) * x_bstride;
             if (c > 0) x = cdd_add(ld_cdd(xo), x);     // this thread stored the earlier chunks
             st_cdd(xo, x);

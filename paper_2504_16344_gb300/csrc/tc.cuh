@@ -138,16 +138,28 @@ __device__ __forceinline__ int tc_exp_above(float mx) {
 // every s_p an integer of at most 8 significant bits times 2^-8p: exact in
 // bf16.  The first two steps act on hi alone (exact); what is left of it is
 // then joined with lo (TwoSum, its error added back before slice 4).
+// Two pairs at a time in packed f32x2 instructions: each lane rounds like the
+// scalar one, in half the issue slots, which is what the slicing warps of a
+// product kernel compete for.
 struct Slicer7 {
-  float r, e;
-  __device__ __forceinline__ void init(float hi, float lo) { r = hi; e = lo; }
-  template <int S> __device__ __forceinline__ float next() {
-    if (S == 2) two_sum(r, e, r, e);
-    if (S == 4) r = __fadd_rn(r, e);
-    const float M = 1.5f * (float)(1 << 23) / (float)(1ull << (8 * S));
-    const float s = __fsub_rn(__fadd_rn(r, M), M);
-    r = __fsub_rn(r, s);
-    return s;
+  f2 r, e;
+  __device__ __forceinline__ void init(float hi0, float lo0, float hi1, float lo1, f2 scale) {
+    r = mul2(f2_make(hi0, hi1), scale);
+    e = mul2(f2_make(lo0, lo1), scale);
+  }
+  // slice S of both pairs as two bf16 (the first in the low half); S = 0 .. 6 in order
+  template <int S> __device__ __forceinline__ uint32_t next() {
+    if (S == 2) {
+      const f2 s = add2(r, e), bb = sub2(s, r);
+      e = add2(sub2(r, sub2(s, bb)), sub2(e, bb));
+      r = s;
+    }
+    if (S == 4) r = add2(r, e);
+    constexpr float m = 1.5f * (float)(1 << 23) / (float)(1ull << (8 * S));
+    const f2 M = f2_make(m, m), s = sub2(add2(r, M), M);
+    r = sub2(r, s);
+    const float2 v = f2_split(s);
+    return tc_pack_bf16(v.x, v.y);
   }
 };
 
@@ -202,12 +214,20 @@ __device__ __forceinline__ void tc_issue_half(bool first, const uint32_t *d, uin
 // most 2^-3, and adding that to D2 (below 2^7.4, multiples of 2^-16), then to
 // D3 (below 0.8, multiples of 2^-24), is exact in 24 bits; from D4 on the
 // rounding is that of the pair's low half.
-__device__ __forceinline__ dd tc_join_levels(const float *d) {
-  float s, e;
-  two_sum(d[0], d[1], s, e);
-  two_sum(s, __fadd_rn(e, d[2]), s, e);
-  two_sum(s, __fadd_rn(e, d[3]), s, e);
-  return dd_make(s, __fadd_rn(e, __fadd_rn(d[4], d[5])));
+// Two values at a time (packed f32x2).
+__device__ __forceinline__ void tc_two_sum2(f2 a, f2 b, f2 &s, f2 &e) {
+  s = add2(a, b);
+  const f2 bb = sub2(s, a);
+  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+}
+__device__ __forceinline__ void tc_join_levels(const f2 *d, f2 &hi, f2 &lo) {
+  f2 s, e;
+  tc_two_sum2(d[0], d[1], s, e);
+  tc_two_sum2(s, add2(e, d[2]), s, e);
+  tc_two_sum2(s, add2(e, d[3]), s, e);
+  e = add2(e, add2(d[4], d[5]));
+  hi = add2(s, e);
+  lo = sub2(e, sub2(hi, s));
 }
 
 }  // namespace tw

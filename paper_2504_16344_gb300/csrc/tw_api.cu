@@ -287,8 +287,12 @@ tw_status tw_create(tw_ctx **out, int Nd, int Nq, int Nx, int Ny, int Nt, double
         }
   }
   // the FP64-class operator's are optional: without them its batched adjoint
-  // runs on the FP32 pipes
-  if (st == TW_OK && c->op[TW_MAP_F][0]) c->ea[TW_MAP_F][0] = (int8_t *)twh::dalloc(c, Nf * Nm);
+  // and forward product run on the FP32 pipes
+  if (st == TW_OK && c->op[TW_MAP_F][0]) {
+    c->ea[TW_MAP_F][0] = (int8_t *)twh::dalloc(c, Nf * Nm);
+    for (int which = 0; which < 2; ++which)
+      c->ef[which] = (int8_t *)twh::dalloc(c, Nf * (size_t)rows_of(c, which));
+  }
   if (st != TW_OK) {
     // keep the message for the caller: report via stderr since ctx is freed
     fprintf(stderr, "tw_create: %s\n", c->err.c_str());
@@ -366,6 +370,8 @@ tw_status tw_set_block_column(tw_ctx *c, tw_map which, int row0, int nrows, cons
       TW_CUDA(c, launch_row_exp(c->op[which][fmt], fmt, c->ea[which][fmt], c->Nf, R, c->Nm, s));
   if (all && c->ea[which][0])
     TW_CUDA(c, launch_row_exp64(c->op[which][0], c->ea[which][0], c->Nf, R, c->Nm, s));
+  if (all && c->ef[which])
+    TW_CUDA(c, launch_fwd_exp64(c->op[which][0], c->ef[which], c->Nf, R, c->Nm, s));
   // with the prior known, keep G = Phi C^{1/2} of these rows for tw_factor_K,
   // computed in FP64 from the caller's FP64 column
   if (which == TW_MAP_F && c->prior_set) {

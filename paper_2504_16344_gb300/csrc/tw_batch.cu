@@ -57,6 +57,22 @@ tw_status check_batch(tw_ctx *c, tw_prec prec, int nrhs, const int *win) {
 
 namespace twb {
 
+// y^ = F^ x^ of a map in the FP64 class (x^ in L.bxh, y^ to L.byh): on the
+// tensor cores unless SIMT tiles were chosen or their tables did not fit
+static cudaError_t forward_dd(tw_ctx *c, tw_lane &L, int which, int B, cudaStream_t s) {
+  const int Nf = c->Nf, Nr = which == TW_MAP_F ? c->Nd : c->Nq, Nm = c->Nm;
+  const void *A = c->op[which][TW_PREC_FP64];
+  const cdd *x = (const cdd *)L.bxh;
+  if (L.adj_rw != 0 || !c->ef[which] || !L.sl64_ex)
+    return launch_gemm_fwd_dd(A, x, (long)Nf * Nm, (cdd *)L.bpart, (cdd *)L.byh, (long)Nf * Nr, Nf, Nr, Nm, B, s,
+                              fwd_lpb(L));
+  cudaError_t e = launch_gemm_fwd_sl64(A, c->ef[which], x, (long)Nf * Nm, L.sl64_ex, (cdd *)L.bpart, Nf, Nr, Nm, B,
+                                       L.bmax, c->d_err, s);
+  if (e != cudaSuccess) return e;
+  return launch_gemm_fwd_reduce_dd((const cdd *)L.bpart, (cdd *)L.byh, (long)Nf * Nr, gemm_fwd_sl64_nrange(Nm), Nf,
+                                   Nr, B, s);
+}
+
 // q = F_q m for B right-hand sides; rows t >= win[b] of m are taken as zero
 // spec_ready: m's spectrum is already in L.bxh (the fused transform of infer_core)
 tw_status forecast_core(tw_ctx *c, tw_lane &L, tw_prec prec, int B, const int *win, const double *m,
@@ -71,8 +87,7 @@ tw_status forecast_core(tw_ctx *c, tw_lane &L, tw_prec prec, int B, const int *w
       TW_CUDA(c, launch_rfft_time_dd(m, 0, Nm, Nt, (cdd *)L.bxh, Nm, Nm, c->plT, c->twT, c->twL, s, ba_m));
     }
     { twh::Phase p(c, TW_PH_GEMV_FWD, s);
-      TW_CUDA(c, launch_gemm_fwd_dd(Aq, (const cdd *)L.bxh, (long)Nf * Nm, (cdd *)L.bpart,
-                                    (cdd *)L.byh, (long)Nf * Nq, Nf, Nq, Nm, B, s, fwd_lpb(L))); }
+      TW_CUDA(c, forward_dd(c, L, TW_MAP_FQ, B, s)); }
     { twh::Phase p(c, TW_PH_IRFFT_DATA, s);
       TW_CUDA(c, launch_irfft_time_dd((const cdd *)L.byh, Nq, q, 0, Nq, Nq, Nt, c->plT, c->twT, c->twL, s, ba_q)); }
   } else {
@@ -197,8 +212,7 @@ tw_status sample_core(tw_ctx *c, tw_lane &L, tw_prec prec, int B, const int *win
     { twh::Phase p(c, TW_PH_RFFT_PARAM, s);
       TW_CUDA(c, launch_rfft_time_dd(samples, 0, Nm, Nt, (cdd *)L.bxh, Nm, Nm, c->plT, c->twT, c->twL, s, ba_m)); }
     { twh::Phase p(c, TW_PH_GEMV_FWD, s);
-      TW_CUDA(c, launch_gemm_fwd_dd(A, (const cdd *)L.bxh, (long)Nf * Nm, (cdd *)L.bpart, (cdd *)L.byh,
-                                    (long)Nf * Nd, Nf, Nd, Nm, B, s, fwd_lpb(L))); }
+      TW_CUDA(c, forward_dd(c, L, TW_MAP_F, B, s)); }
     { twh::Phase p(c, TW_PH_IRFFT_DATA, s);
       TW_CUDA(c, launch_irfft_time_dd((const cdd *)L.byh, Nd, L.brd, 0, Nd, Nd, Nt, c->plT, c->twT, c->twL, s, ba_d)); }
   } else {
@@ -235,14 +249,14 @@ size_t lane_bytes(const tw_ctx *c, int bmax) {
     const int cols = (bmax + 7) / 8 * 8 + 80;
     b += 2 * B * np * sizeof(dd) + sl_ws_bytes(c->Nf, c->Rmax, cols) + sl_eb_bytes(c->Nf, cols);
   }
-  if (c->ea[TW_MAP_F][0]) b += sl64_ws_bytes(c->Nf, c->Nd, bmax) + sl64_eb_bytes(c->Nf, bmax);
+  if (c->ea[TW_MAP_F][0]) b += sl64_ws_bytes(c->Nf, c->Nd, bmax) + sl64_eb_bytes(c->Nf, bmax) + (size_t)c->Nf * bmax;
   return b;
 }
 
 void free_lane(tw_ctx *c, tw_lane &L) {
   void **bufs[] = {(void **)&L.win_dev, (void **)&L.trsm_prog, (void **)&L.bz, (void **)&L.by,
                    (void **)&L.bzd, (void **)&L.byd, (void **)&L.brd, &L.byh, &L.bxh, &L.bpart,
-                   &L.bsl_ws, (void **)&L.bsl_eb, &L.sl64_ws, (void **)&L.sl64_eb};
+                   &L.bsl_ws, (void **)&L.bsl_eb, &L.sl64_ws, (void **)&L.sl64_eb, (void **)&L.sl64_ex};
   for (void **b : bufs) { twh::dfree(c, *b); *b = nullptr; }
   L.bmax = 0;
   L.bytes = 0;
@@ -283,6 +297,7 @@ tw_status alloc_lane(tw_ctx *c, tw_lane &L, int bmax) {
     L.sl64_eb_n = sl64_eb_bytes(c->Nf, bmax);
     L.sl64_eb = (int *)twh::dalloc(c, L.sl64_eb_n);
     if (L.sl64_eb) L.sl64_ws = twh::dalloc(c, L.sl64_ws_n);
+    if (L.sl64_ws) L.sl64_ex = (int8_t *)twh::dalloc(c, (size_t)c->Nf * bmax);
   }
   if (!ok) {
     free_lane(c, L);
