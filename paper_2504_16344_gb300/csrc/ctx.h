@@ -31,6 +31,10 @@ struct tw_lane {
   int *sl64_eb = nullptr;
   size_t sl64_ws_n = 0, sl64_eb_n = 0;
   int8_t *sl64_ex = nullptr;         // [Nf][bmax] exponents of x^ (gemm_fwd_sl64.cu)
+  // z slices of the solves' panel updates (trsm_tc.cu); null: the sweeps run
+  // as one SIMT launch
+  void *trsm_ws = nullptr;
+  size_t trsm_ws_n = 0;
   // tiles of the batched products (tw_batch_tiles): right-hand sides per
   // tensor-core tile (mixed adjoint) and per warp (FP64-class adjoint), lanes
   // per right-hand side (forward products); chosen by measurement at
@@ -118,6 +122,7 @@ struct tw_ctx {
   // tiles chosen for its products
   tw_lane lane;
   tw_tiles tiles{};
+  int8_t *trsm_ef = nullptr, *trsm_eb = nullptr;   // row exponents of Lfs, Lbs (trsm_tc.cu; null: not kept)
   tw::dd *inv_dd = nullptr;   // float-pair diagonal-block inverses of the FP64 factor (batched solves)
   // Phase 3 QoI precomputations (tw_qoi_build): rows indexed by QoI entry t*Nq + i
   double *Qmap = nullptr, *Wmap = nullptr;   // [Nq Nt][Nd Nt]: Q = F_q Gamma_pr F^T K^-1, W = (F Gamma_pr F_q^T)^T

@@ -79,12 +79,32 @@ cudaError_t launch_trsm_d(const double *Lp, const double *Linv, const double *Lc
                           const void *rhs, int rhs_kind, long rhs_bstride, double *out,
                           long out_bstride, const int *win, int Nd, int Nt, int B, int NB,
                           int *prog, bool fwd, int *err, int *abort_flag, cudaStream_t s);
+// split: two right-hand sides per column slice, a row's sum split over four
+// threads (faster hand-offs, other rounding)
 // the same sweeps with the single-vector solve's pre-multiplied blocks: Lx =
 // Lf (Linv_I L_IJ, forward) or Lb (L_IJ Linv_J, backward), packed like L
 cudaError_t launch_trsm_dd_scaled(const dd *Lx, const dd *Linv, const void *rhs, int rhs_kind,
                                   long rhs_bstride, dd *out, long out_bstride, const int *win, int Nd,
-                                  int Nt, int B, int NB, int *prog, bool fwd, int *err, int *abort_flag,
-                                  cudaStream_t s);
+                                  int Nt, int B, int NB, int *prog, bool fwd, bool split, int *err,
+                                  int *abort_flag, cudaStream_t s);
+// block rows I0 .. I1-1 of that sweep (a panel), whose rows of out hold the
+// products with the panels before; prog as the panels before left it (zeroed
+// before the first), *tbase the tickets they drew (advanced)
+cudaError_t launch_trsm_dd_panel(const dd *Lx, const dd *Linv, const void *rhs, int rhs_kind, long rhs_bstride,
+                                 dd *out, long out_bstride, const int *win, int Nd, int Nt, int B, int NB, int I0,
+                                 int I1, int *tbase, int *prog, bool fwd, int *err, int *abort_flag,
+                                 cudaStream_t s);
+// the whole sweep in panels, the products between panels on the tensor cores
+// (trsm_tc.cu); ea: row exponents of Lx (launch_trsm_tc_exp, trsm_tc_exp_bytes
+// each); ws: trsm_tc_ws_bytes(B)
+bool trsm_tc_applies(int NB, int bmax);
+size_t trsm_tc_exp_bytes(int NB);
+size_t trsm_tc_ws_bytes(int B);
+cudaError_t launch_trsm_tc_exp(const dd *Lf, const dd *Lb, int8_t *ef, int8_t *eb, int NB, cudaStream_t s);
+cudaError_t launch_trsm_dd_tc(const dd *Lx, const int8_t *ea, const dd *Linv, const void *rhs, int rhs_kind,
+                              long rhs_bstride, dd *out, long out_bstride, const int *win, int Nd, int Nt, int B,
+                              int NB, int *prog, bool fwd, void *ws, size_t ws_bytes, int *err, int *abort_flag,
+                              cudaStream_t s);
 cudaError_t launch_chain_blocks_d(const double *Lp, const double *Linv, double *Mf, double *Cb,
                                   int NB, cudaStream_t s);
 cudaError_t launch_chain_blocks_f(const float *Lp, const float *Linv, float *Mf, float *Cb, int NB,

@@ -57,6 +57,24 @@ tw_status check_batch(tw_ctx *c, tw_prec prec, int nrhs, const int *win) {
 
 namespace twb {
 
+// one batched sweep with K's factor in double-float.  FP64-class results: in
+// panels with the products between them on the tensor cores where their tables
+// are kept, else split over threads.  The reduced paths keep the plain sweep: a
+// last-bit change of y moves the FP32 roundings after it, and with them their
+// results by a few of FP32's last bits.
+static cudaError_t sweep(tw_ctx *c, tw_lane &L, tw_prec prec, bool fwd, const void *rhs, int rhs_kind,
+                         long rhs_bstride, dd *out, const int *win, int B, cudaStream_t s) {
+  const dd *Lx = fwd ? c->Lfs : c->Lbs;
+  int *prog = L.trsm_prog + (fwd ? 0 : trsm_prog_ints(L.bmax));
+  const bool f64 = prec == TW_PREC_FP64, panels = trsm_tc_applies(c->NB, c->lane.bmax);
+  if (f64 && panels && c->trsm_eb && L.trsm_ws)
+    return launch_trsm_dd_tc(Lx, fwd ? c->trsm_ef : c->trsm_eb, c->inv_dd, rhs, rhs_kind, rhs_bstride, out,
+                             c->n_pad, win, c->Nd, c->Nt, B, c->NB, prog, fwd, L.trsm_ws, L.trsm_ws_n, c->d_err,
+                             c->abort_flag, s);
+  return launch_trsm_dd_scaled(Lx, c->inv_dd, rhs, rhs_kind, rhs_bstride, out, c->n_pad, win, c->Nd, c->Nt, B,
+                               c->NB, prog, fwd, f64 && !panels, c->d_err, c->abort_flag, s);
+}
+
 // y^ = F^ x^ of a map in the FP64 class (x^ in L.bxh, y^ to L.byh): on the
 // tensor cores unless SIMT tiles were chosen or their tables did not fit
 static cudaError_t forward_dd(tw_ctx *c, tw_lane &L, int which, int B, cudaStream_t s) {
@@ -113,7 +131,6 @@ tw_status infer_core(tw_ctx *c, tw_lane &L, tw_prec prec, int B, const int *win,
   // with G^ = F^ C kept the adjoint gives m directly (no prior filter)
   const bool useG = c->opG[prec] != nullptr;
   const void *A = useG ? c->opG[prec] : c->op[TW_MAP_F][prec];
-  int *prog_f = L.trsm_prog, *prog_b = L.trsm_prog + trsm_prog_ints(L.bmax);
   const BatchArg ba_y{B, np, (long)Nf * Nd, 0, win};
   const BatchArg ba_x{B, (long)Nf * Nm, (long)Nt * Nm, 0, win};
   // with G^ (no prior after the inverse transform) and a forecast requested,
@@ -128,11 +145,9 @@ tw_status infer_core(tw_ctx *c, tw_lane &L, tw_prec prec, int B, const int *win,
     // lane's 8-byte solve buffers
     dd *bz = reinterpret_cast<dd *>(L.bz), *by = reinterpret_cast<dd *>(L.by);
     { twh::Phase p(c, TW_PH_TRSV_FWD, s);
-      TW_CUDA(c, launch_trsm_dd_scaled(c->Lfs, c->inv_dd, rhs, 0, rhs_bstride, bz, np, win, Nd, Nt, B,
-                                       c->NB, prog_f, true, c->d_err, c->abort_flag, s)); }
+      TW_CUDA(c, sweep(c, L, prec, true, rhs, 0, rhs_bstride, bz, win, B, s)); }
     { twh::Phase p(c, TW_PH_TRSV_BWD, s);
-      TW_CUDA(c, launch_trsm_dd_scaled(c->Lbs, c->inv_dd, bz, 1, np, by, np, win, Nd, Nt, B, c->NB,
-                                       prog_b, false, c->d_err, c->abort_flag, s)); }
+      TW_CUDA(c, sweep(c, L, prec, false, bz, 1, np, by, win, B, s)); }
     { twh::Phase p(c, TW_PH_RFFT_DATA, s);
       TW_CUDA(c, launch_rfft_time_dd(by, 1, Nd, Nt, (cdd *)L.byh, Nd, Nd, c->plT, c->twT, c->twL, s, ba_y)); }
     { twh::Phase p(c, TW_PH_GEMV_ADJ, s);
@@ -160,11 +175,9 @@ tw_status infer_core(tw_ctx *c, tw_lane &L, tw_prec prec, int B, const int *win,
   } else {
     // the same double-float sweeps as the FP64 path
     { twh::Phase p(c, TW_PH_TRSV_FWD, s);
-      TW_CUDA(c, launch_trsm_dd_scaled(c->Lfs, c->inv_dd, rhs, 0, rhs_bstride, L.bzd, np, win, Nd, Nt, B,
-                                       c->NB, prog_f, true, c->d_err, c->abort_flag, s)); }
+      TW_CUDA(c, sweep(c, L, prec, true, rhs, 0, rhs_bstride, L.bzd, win, B, s)); }
     { twh::Phase p(c, TW_PH_TRSV_BWD, s);
-      TW_CUDA(c, launch_trsm_dd_scaled(c->Lbs, c->inv_dd, L.bzd, 1, np, L.byd, np, win, Nd, Nt, B, c->NB,
-                                       prog_b, false, c->d_err, c->abort_flag, s)); }
+      TW_CUDA(c, sweep(c, L, prec, false, L.bzd, 1, np, L.byd, win, B, s)); }
     // double-float data spectra; the product on the tensor cores with both
     // sides cut into exact fixed-point slices: F^T y cancels (y is large
     // against m), so its sum has to be formed far below FP32 rounding
@@ -249,6 +262,7 @@ size_t lane_bytes(const tw_ctx *c, int bmax) {
     const int cols = (bmax + 7) / 8 * 8 + 80;
     b += 2 * B * np * sizeof(dd) + sl_ws_bytes(c->Nf, c->Rmax, cols) + sl_eb_bytes(c->Nf, cols);
   }
+  if (c->trsm_eb) b += trsm_tc_ws_bytes(bmax);
   if (c->ea[TW_MAP_F][0]) b += sl64_ws_bytes(c->Nf, c->Nd, bmax) + sl64_eb_bytes(c->Nf, bmax) + (size_t)c->Nf * bmax;
   return b;
 }
@@ -256,7 +270,7 @@ size_t lane_bytes(const tw_ctx *c, int bmax) {
 void free_lane(tw_ctx *c, tw_lane &L) {
   void **bufs[] = {(void **)&L.win_dev, (void **)&L.trsm_prog, (void **)&L.bz, (void **)&L.by,
                    (void **)&L.bzd, (void **)&L.byd, (void **)&L.brd, &L.byh, &L.bxh, &L.bpart,
-                   &L.bsl_ws, (void **)&L.bsl_eb, &L.sl64_ws, (void **)&L.sl64_eb, (void **)&L.sl64_ex};
+                   &L.bsl_ws, (void **)&L.bsl_eb, &L.sl64_ws, (void **)&L.sl64_eb, &L.trsm_ws, (void **)&L.sl64_ex};
   for (void **b : bufs) { twh::dfree(c, *b); *b = nullptr; }
   L.bmax = 0;
   L.bytes = 0;
@@ -292,6 +306,10 @@ tw_status alloc_lane(tw_ctx *c, tw_lane &L, int bmax) {
     L.bsl_ws = take(L.bsl_ws_n);
     L.bsl_eb = (int *)take(L.bsl_eb_n);
   }
+  if (ok && c->trsm_eb) {             // optional: null leaves the sweeps in one launch
+    L.trsm_ws_n = trsm_tc_ws_bytes(bmax);
+    L.trsm_ws = twh::dalloc(c, L.trsm_ws_n);
+  }
   if (ok && c->ea[TW_MAP_F][0]) {     // optional: null leaves the SIMT product
     L.sl64_ws_n = sl64_ws_bytes(c->Nf, c->Nd, bmax);
     L.sl64_eb_n = sl64_eb_bytes(c->Nf, bmax);
@@ -318,7 +336,10 @@ namespace {
 void free_batch(tw_ctx *c) {
   twb::free_lane(c, c->lane);
   twh::dfree(c, c->inv_dd);
+  twh::dfree(c, c->trsm_ef);
+  twh::dfree(c, c->trsm_eb);
   c->inv_dd = nullptr;
+  c->trsm_ef = c->trsm_eb = nullptr;
 }
 
 }  // namespace
@@ -326,6 +347,7 @@ void free_batch(tw_ctx *c) {
 tw_status twh::refresh_dd_factor(tw_ctx *c, cudaStream_t s) {
   if (!c->have64) return TW_OK;
   if (c->inv_dd) TW_CUDA(c, launch_double_to_dd(c->inv64, c->inv_dd, (size_t)c->NB * NB_ * NB_, s));
+  if (c->trsm_eb) TW_CUDA(c, launch_trsm_tc_exp(c->Lfs, c->Lbs, c->trsm_ef, c->trsm_eb, c->NB, s));
   TW_CUDA(c, cudaStreamSynchronize(s));
   return TW_OK;
 }
@@ -346,6 +368,10 @@ tw_status tw_reserve_batch(tw_ctx *c, int bmax) {
   if (!c->inv_dd) {
     free_batch(c);
     return twh::fail(c, TW_ERR_OOM, "batch workspaces");
+  }
+  if (trsm_tc_applies(c->NB, bmax) && c->op[TW_MAP_F][TW_PREC_FP64]) {       // optional: without both the sweeps stay on the FP32 pipes
+    c->trsm_ef = (int8_t *)twh::dalloc(c, trsm_tc_exp_bytes(c->NB));
+    if (c->trsm_ef) c->trsm_eb = (int8_t *)twh::dalloc(c, trsm_tc_exp_bytes(c->NB));
   }
   tw_status st = twb::alloc_lane(c, c->lane, bmax);
   if (st != TW_OK) {

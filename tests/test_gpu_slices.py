@@ -58,3 +58,38 @@ def test_products_on_tensor_cores(Nd, Nx, Ny, B, keep_g):
             e = (out[0][k][b] - out[4][k][b]).norm() / out[4][k][b].norm()
             tol = 2.0 ** -46 * n + (2.0 ** -51 * s0[b].norm() / out[4][k][b].norm() if k == 2 else 0.0)
             assert e < tol, (k, b, float(e))
+
+
+# one sweep with narrow slices (1 right-hand side, an odd number of them, one
+# and several block rows), then panels: 132 block rows (11 full panels), 172 and
+# 260 (part panels, odd pairs of blocks), right-hand sides that take tiles of 64,
+# 48 and 32 columns (and 16, one alone), windows that end inside the panels
+@pytest.mark.parametrize("Nd,Nt,B", [(7, 9, 1), (50, 33, 17), (49, 33, 40), (200, 42, 64), (200, 42, 65),
+                                     (199, 55, 48), (200, 83, 32)])
+def test_batched_solves(Nd, Nt, B):
+    import torch
+    from paper_2504_16344_gb300 import tw
+    Nx, Ny = 6, 5
+    ctx = tw.Context(Nd, 2, Nx, Ny, Nt, keep=tw.KEEP_FP64)
+    ctx.set_prior(1.0, 0.1, 1.0)
+    g = torch.Generator(device="cuda").manual_seed(Nd + Nt + B)
+    ctx.set_block_column(tw.MAP_F, 0, torch.randn((Nt, Nd, Nx * Ny), generator=g, dtype=torch.float64,
+                                                  device="cuda"))
+    ctx.set_block_column(tw.MAP_FQ, 0, torch.randn((Nt, 2, Nx * Ny), generator=g, dtype=torch.float64,
+                                                   device="cuda"))
+    ctx.factor_K(1.0 * Nx * Ny * Nt)       # K's condition stays below a few hundred
+    d = torch.randn((B, Nt, Nd), generator=g, dtype=torch.float64, device="cuda")
+    win = [1 + (7 * b + Nt - 1) % Nt for b in range(B)]
+    ref = ctx.infer(tw.PREC_FP64, d, windows=win)          # single-vector solves: no batch is reserved
+    ctx.reserve_batch(B)
+    m, _ = ctx.infer_batch(tw.PREC_FP64, d, torch.tensor(win, dtype=torch.int32, device="cuda"))
+    # the same right-hand sides one at a time: bitwise the same (no batch mates)
+    one, _ = ctx.infer_batch(tw.PREC_FP64, d[B - 1:], torch.tensor(win[-1:], dtype=torch.int32, device="cuda"))
+    ctx.check()
+    assert torch.equal(one[0], m[B - 1])
+    # two backward-stable solves in 48-bit arithmetic: condition x 2^-46 x a
+    # modest growth, below 1e-11 as the library's FP64 bound
+    for b in range(B):
+        e = (m[b] - ref[b]).norm() / ref[b].norm()
+        assert e < 1e-11, (b, float(e))
+    ctx.close()
