@@ -182,34 +182,20 @@ __device__ __forceinline__ cf cf_mul(cf a, cf b) {
 // --------------------------------------------- precision policies
 // Each policy names a complex type, a real type and the operations the FFT
 // engine needs, so one engine serves the df64 path and the FP32 path.
-struct PolDD {
-  typedef cdd cx;
-  typedef dd re;
-  static constexpr int occ = 3;   // CTAs of 256 threads per SM the FFT kernels aim for
-  static constexpr int smem = 72 * 1024;   // shared-memory budget of one FFT CTA
-  static __device__ __forceinline__ cx zero() { return cdd_zero(); }
-  static __device__ __forceinline__ cx add(cx a, cx b) { return cdd_add(a, b); }
-  static __device__ __forceinline__ cx sub(cx a, cx b) { return cdd_sub(a, b); }
-  static __device__ __forceinline__ cx mul(cx a, cx b) { return cdd_mul(a, b); }
-  static __device__ __forceinline__ cx conj(cx a) { return cdd_conj(a); }
-  static __device__ __forceinline__ cx mul_mi(cx a) { return cdd_mul_mi(a); }
-  static __device__ __forceinline__ cx mul_i(cx a) { return cdd_mul_i(a); }
-  static __device__ __forceinline__ cx scale_re(cx a, re s) { return cdd_scale(a, s); }
-  static __device__ __forceinline__ cx scale2(cx a, float p2) { return cdd_scale2(a, p2); }
-  static __device__ __forceinline__ re re_add(re a, re b) { return dd_add(a, b); }
-  static __device__ __forceinline__ re re_sub(re a, re b) { return dd_sub(a, b); }
-  static __device__ __forceinline__ re re_neg(re a) { return dd_neg(a); }
-  static __device__ __forceinline__ re re_mul(re a, re b) { return dd_mul(a, b); }
-  static __device__ __forceinline__ re re_zero() { return dd_zero(); }
-  static __device__ __forceinline__ cx make(re r, re i) { cx z; z.re = r; z.im = i; return z; }
-  static __device__ __forceinline__ re real(cx a) { return a.re; }
-  static __device__ __forceinline__ re imag(cx a) { return a.im; }
-};
 struct PolF {
   typedef cf cx;
   typedef float re;
-  static constexpr int occ = 4;
+  static constexpr bool fused = true;   // fused passes (fft_engine.cuh)
+  // 4 CTAs a SM, 3 where the 25-point pass may run (64 registers spill it): the
+  // 400-step transforms of 64 right-hand sides take 15.6 ms with it at 3 CTAs
+  // against 17.5 ms without it at 4, the 60-step ones of 16 (no such pass) 1.23
+  // ms at 4 against 1.42 ms at 3
+  static constexpr int occ = 4, occ_big = 3;
+  static constexpr int occ_prior = 4;   // ... of the prior filter
   static constexpr int smem = 64 * 1024;
+  typedef cf mem;
+  static __device__ __forceinline__ cx from_mem(mem a) { return a; }
+  static __device__ __forceinline__ mem to_mem(cx a) { return a; }
   static __device__ __forceinline__ cx zero() { return cf_zero(); }
   static __device__ __forceinline__ cx add(cx a, cx b) { return cf_add(a, b); }
   static __device__ __forceinline__ cx sub(cx a, cx b) { return cf_sub(a, b); }
@@ -233,8 +219,13 @@ struct PolF {
 struct PolD {
   typedef cd cx;
   typedef double re;
-  static constexpr int occ = 2;
+  static constexpr bool fused = false;   // fused passes (fft_engine.cuh)
+  static constexpr int occ = 2, occ_big = 2;
+  static constexpr int occ_prior = 2;   // ... of the prior filter
   static constexpr int smem = 64 * 1024;
+  typedef cd mem;
+  static __device__ __forceinline__ cx from_mem(mem a) { return a; }
+  static __device__ __forceinline__ mem to_mem(cx a) { return a; }
   static __device__ __forceinline__ cx make(re r, re i) { cx z; z.re = r; z.im = i; return z; }
   static __device__ __forceinline__ cx zero() { return make(0.0, 0.0); }
   static __device__ __forceinline__ cx add(cx a, cx b) { return make(a.re + b.re, a.im + b.im); }
@@ -318,4 +309,94 @@ __device__ __forceinline__ void dd_add2(f2 &ah, f2 &al, f2 bh, f2 bl) {
   ah = add2(s, e);
   al = sub2(e, sub2(ah, s));
 }
+
+// ------------------------------------- complex double-float in packed pairs
+// hi = (Re, Im) high parts, lo = (Re, Im) low parts: a complex operation runs
+// both parts in one packed instruction, with the bits of the cdd functions
+// above in half the issue slots, which is what the FFT kernels are short of
+// (their FMA pipe was 52% busy at 68% issue).  The double-float transform of 64 x
+// 50,000 series of 400 steps, there and back: 59.5 -> 57.8 ms; the prior filter of
+// 32 x 400 fields of 200 x 250, twice: 64.8 -> 60.0 ms.
+struct __align__(16) cdp { f2 hi, lo; };
+__device__ __forceinline__ f2 f2_neg(f2 a) { a.v ^= 0x8000000080000000ull; return a; }
+__device__ __forceinline__ f2 f2_neg_hi(f2 a) { a.v ^= 0x8000000000000000ull; return a; }   // lane 1
+__device__ __forceinline__ f2 f2_bcast(float x) { return f2_make(x, x); }
+__device__ __forceinline__ cdp cdp_add(cdp a, cdp b) { dd_add2(a.hi, a.lo, b.hi, b.lo); return a; }
+__device__ __forceinline__ cdp cdp_sub(cdp a, cdp b) {
+  const f2 s = sub2(a.hi, b.hi);
+  const f2 bb = sub2(s, a.hi);
+  f2 e = sub2(sub2(a.hi, sub2(s, bb)), add2(b.hi, bb));
+  e = add2(e, sub2(a.lo, b.lo));
+  cdp r;
+  r.hi = add2(s, e);
+  r.lo = sub2(e, sub2(r.hi, s));
+  return r;
+}
+// (x, y) -> (-y, x) and (y, -x)
+__device__ __forceinline__ f2 f2_mul_i(f2 a) { const float2 v = f2_split(a); return f2_make(-v.y, v.x); }
+__device__ __forceinline__ f2 f2_mul_mi(f2 a) { const float2 v = f2_split(a); return f2_make(v.y, -v.x); }
+__device__ __forceinline__ cdp cdp_mul(cdp a, cdp b) {
+  // (re, im) = a.re (b.re, b.im) + a.im (-b.im, b.re), as dd_dot2 in each lane
+  const float2 ah = f2_split(a.hi), al = f2_split(a.lo);
+  const f2 xh = f2_bcast(ah.x), xl = f2_bcast(al.x), yh = f2_bcast(ah.y), yl = f2_bcast(al.y);
+  const f2 ch = f2_mul_i(b.hi), cl = f2_mul_i(b.lo);
+  const f2 p = mul2(xh, b.hi);
+  f2 e = fma2(xh, b.hi, f2_neg(p));
+  e = fma2(xh, b.lo, e);
+  e = fma2(xl, b.hi, e);
+  const f2 q = mul2(yh, ch);
+  f2 f = fma2(yh, ch, f2_neg(q));
+  f = fma2(yh, cl, f);
+  f = fma2(yl, ch, f);
+  const f2 s = add2(p, q);
+  const f2 bb = sub2(s, p);
+  f2 r = add2(sub2(p, sub2(s, bb)), sub2(q, bb));
+  r = add2(r, add2(e, f));
+  cdp o;
+  o.hi = add2(s, r);
+  o.lo = sub2(r, sub2(o.hi, s));
+  return o;
+}
+__device__ __forceinline__ cdp cdp_scale(cdp a, dd s) {
+  const f2 sh = f2_bcast(s.hi), sl = f2_bcast(s.lo);
+  const f2 p = mul2(a.hi, sh);
+  f2 e = fma2(a.hi, sh, f2_neg(p));
+  e = fma2(a.hi, sl, e);
+  e = fma2(a.lo, sh, e);
+  cdp o;
+  o.hi = add2(p, e);
+  o.lo = sub2(e, sub2(o.hi, p));
+  return o;
+}
+
+// double-float FFTs: cdp in registers and shared memory, cdd in the spectra
+struct PolDD {
+  typedef cdp cx;
+  typedef cdd mem;
+  typedef dd re;
+  static constexpr bool fused = false;   // fused passes (fft_engine.cuh)
+  static constexpr int occ = 3, occ_big = 3;   // CTAs of 256 threads per SM the FFT kernels aim for
+  static constexpr int occ_prior = 3;   // ... of the prior filter
+  static constexpr int smem = 72 * 1024;   // shared-memory budget of one FFT CTA
+  static __device__ __forceinline__ cx from_mem(mem a) { return make(a.re, a.im); }
+  static __device__ __forceinline__ mem to_mem(cx a) { mem z; z.re = real(a); z.im = imag(a); return z; }
+  static __device__ __forceinline__ cx zero() { return make(dd_zero(), dd_zero()); }
+  static __device__ __forceinline__ cx add(cx a, cx b) { return cdp_add(a, b); }
+  static __device__ __forceinline__ cx sub(cx a, cx b) { return cdp_sub(a, b); }
+  static __device__ __forceinline__ cx mul(cx a, cx b) { return cdp_mul(a, b); }
+  static __device__ __forceinline__ cx conj(cx a) { a.hi = f2_neg_hi(a.hi); a.lo = f2_neg_hi(a.lo); return a; }
+  static __device__ __forceinline__ cx mul_mi(cx a) { a.hi = f2_mul_mi(a.hi); a.lo = f2_mul_mi(a.lo); return a; }
+  static __device__ __forceinline__ cx mul_i(cx a) { a.hi = f2_mul_i(a.hi); a.lo = f2_mul_i(a.lo); return a; }
+  static __device__ __forceinline__ cx scale_re(cx a, re s) { return cdp_scale(a, s); }
+  static __device__ __forceinline__ cx scale2(cx a, float p2) { const f2 p = f2_bcast(p2); a.hi = mul2(a.hi, p); a.lo = mul2(a.lo, p); return a; }
+  static __device__ __forceinline__ re re_add(re a, re b) { return dd_add(a, b); }
+  static __device__ __forceinline__ re re_sub(re a, re b) { return dd_sub(a, b); }
+  static __device__ __forceinline__ re re_neg(re a) { return dd_neg(a); }
+  static __device__ __forceinline__ re re_mul(re a, re b) { return dd_mul(a, b); }
+  static __device__ __forceinline__ re re_zero() { return dd_zero(); }
+  static __device__ __forceinline__ cx make(re r, re i) { cx z; z.hi = f2_make(r.hi, i.hi); z.lo = f2_make(r.lo, i.lo); return z; }
+  static __device__ __forceinline__ re real(cx a) { dd r; r.hi = f2_split(a.hi).x; r.lo = f2_split(a.lo).x; return r; }
+  static __device__ __forceinline__ re imag(cx a) { dd r; r.hi = f2_split(a.hi).y; r.lo = f2_split(a.lo).y; return r; }
+};
+
 }  // namespace tw

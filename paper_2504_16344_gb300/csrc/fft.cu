@@ -100,15 +100,16 @@ __device__ __forceinline__ void add_out<PolD>(void *base, int kind, long off, do
 // a thread's loads are all in flight at once; the caller's __syncthreads()
 // after this makes the tile visible to the CTA
 template <class P>
-__device__ __forceinline__ void stage_cols(typename P::cx *buf, const typename P::cx *in, long ld,
+__device__ __forceinline__ void stage_cols(typename P::mem *buf, const typename P::mem *in, long ld,
                                            long n0, long N, int nk, int B) {
-  constexpr int SZ = (int)sizeof(typename P::cx);
+  constexpr int SZ = (int)sizeof(typename P::mem);
+  const int lgB = __ffs(B) - 1;   // B is a power of two
   static_assert(SZ == 8 || SZ == 16, "cp.async copies 8 or 16 bytes");
   for (int idx = threadIdx.x; idx < nk * B; idx += blockDim.x) {
-    const int b = idx % B, k = idx / B;
+    const int b = idx & (B - 1), k = idx >> lgB;
     const long n = n0 + b;
     const bool ok = n < N;
-    const typename P::cx *src = ok ? in + (long)k * ld + n : in;
+    const typename P::mem *src = ok ? in + (long)k * ld + n : in;
     const uint32_t dst = (uint32_t)__cvta_generic_to_shared(buf + idx);
     if (SZ == 16)
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
@@ -118,16 +119,16 @@ __device__ __forceinline__ void stage_cols(typename P::cx *buf, const typename P
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
 }
 
-template <class P>
-__global__ void __launch_bounds__(256, P::occ)
+template <class P, bool BIG>
+__global__ void __launch_bounds__(256, BIG ? P::occ_big : P::occ)
 k_rfft_time(const void *__restrict__ in, int in_kind, long in_ld, int n_in,
-            typename P::cx *__restrict__ out, long out_ld, int N, FftPlan pl,
+            typename P::mem *__restrict__ out, long out_ld, int N, FftPlan pl,
             const typename P::cx *__restrict__ twM, const typename P::cx *__restrict__ twL,
             int B, BatchArg ba) {
   typedef typename P::cx cx;
   typedef typename P::re re;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int M = pl.M;
+  const int M = pl.M, lgB = __ffs(B) - 1;   // B is a power of two
   cx *buf0 = reinterpret_cast<cx *>(smem_raw);
   cx *buf1 = buf0 + (M + 1) * B;
   const long n0 = (long)blockIdx.x * B;
@@ -137,7 +138,7 @@ k_rfft_time(const void *__restrict__ in, int in_kind, long in_ld, int n_in,
   out += bz * ba.out_stride;
   // pack z_j = x_{2j} + i x_{2j+1}; x_t = 0 for t >= nin
   for (int idx = threadIdx.x; idx < M * B; idx += blockDim.x) {
-    const int b = idx % B, j = idx / B;
+    const int b = idx & (B - 1), j = idx >> lgB;
     const long n = n0 + b;
     re r = P::re_zero(), im = P::re_zero();
     if (n < N) {
@@ -148,31 +149,31 @@ k_rfft_time(const void *__restrict__ in, int in_kind, long in_ld, int n_in,
     buf0[j * B + b] = P::make(r, im);
   }
   __syncthreads();
-  cx *Z = fft_run<P, false>(buf0, buf1, twM, pl, B, B, 1, true);
+  cx *Z = fft_run<P, false, BIG>(buf0, buf1, twM, pl, B, B, 1, true);
   // X_k = (Z_k + conj Z_{M-k})/2 + W_L^k (Z_k - conj Z_{M-k})/(2i)
   for (int idx = threadIdx.x; idx < (M + 1) * B; idx += blockDim.x) {
-    const int b = idx % B, k = idx / B;
+    const int b = idx & (B - 1), k = idx >> lgB;
     const long n = n0 + b;
     if (n >= N) continue;
-    cx zk = Z[(k % M) * B + b];
-    cx zc = P::conj(Z[((M - k) % M) * B + b]);
+    cx zk = Z[(k == M ? 0 : k) * B + b];
+    cx zc = P::conj(Z[(k == 0 ? 0 : M - k) * B + b]);
     cx E = P::scale2(P::add(zk, zc), 0.5f);
     cx O = P::scale2(P::mul_mi(P::sub(zk, zc)), 0.5f);
     cx X = P::add(E, P::mul(ld_cx<P>(twL + k), O));
-    out[(long)k * out_ld + n] = X;
+    out[(long)k * out_ld + n] = P::to_mem(X);
   }
 }
 
-template <class P>
-__global__ void __launch_bounds__(256, P::occ)
-k_irfft_time(const typename P::cx *__restrict__ in, long in_ld, void *__restrict__ out,
+template <class P, bool BIG>
+__global__ void __launch_bounds__(256, BIG ? P::occ_big : P::occ)
+k_irfft_time(const typename P::mem *__restrict__ in, long in_ld, void *__restrict__ out,
              int out_kind, long out_ld, int N, int n_keep, FftPlan pl,
              const typename P::cx *__restrict__ twM, const typename P::cx *__restrict__ twL,
              typename P::re invM, int B, BatchArg ba) {
   typedef typename P::cx cx;
   typedef typename P::re re;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int M = pl.M;
+  const int M = pl.M, lgB = __ffs(B) - 1;   // B is a power of two
   cx *buf0 = reinterpret_cast<cx *>(smem_raw);
   cx *buf1 = buf0 + (M + 1) * B;
   const long n0 = (long)blockIdx.x * B;
@@ -180,21 +181,22 @@ k_irfft_time(const typename P::cx *__restrict__ in, long in_ld, void *__restrict
   in += bz * ba.in_stride;
   const long ooff = bz * ba.out_stride;
   const int nkeep = ba.window(bz, n_keep);
-  stage_cols<P>(buf0, in, in_ld, n0, N, M + 1, B);
+  typename P::mem *raw = reinterpret_cast<typename P::mem *>(buf0);
+  stage_cols<P>(raw, in, in_ld, n0, N, M + 1, B);
   __syncthreads();
   // Z_k = E_k + i O_k, E_k = (X_k + conj X_{M-k})/2, O_k = (X_k - conj X_{M-k}) W_L^{-k} / 2
   for (int idx = threadIdx.x; idx < M * B; idx += blockDim.x) {
-    const int b = idx % B, k = idx / B;
-    cx xk = buf0[k * B + b];
-    cx xc = P::conj(buf0[(M - k) * B + b]);
+    const int b = idx & (B - 1), k = idx >> lgB;
+    cx xk = P::from_mem(raw[k * B + b]);
+    cx xc = P::conj(P::from_mem(raw[(M - k) * B + b]));
     cx E = P::scale2(P::add(xk, xc), 0.5f);
     cx O = P::scale2(P::mul(P::sub(xk, xc), P::conj(ld_cx<P>(twL + k))), 0.5f);
     buf1[k * B + b] = P::add(E, P::mul_i(O));
   }
   __syncthreads();
-  cx *z = fft_run<P, true>(buf1, buf0, twM, pl, B, B, 1, true);
+  cx *z = fft_run<P, true, BIG>(buf1, buf0, twM, pl, B, B, 1, true);
   for (int idx = threadIdx.x; idx < M * B; idx += blockDim.x) {
-    const int b = idx % B, t = idx / B;
+    const int b = idx & (B - 1), t = idx >> lgB;
     const long n = n0 + b;
     if (n >= N) continue;
     re v = P::re_zero();
@@ -211,10 +213,10 @@ k_irfft_time(const typename P::cx *__restrict__ in, long in_ld, void *__restrict
 // transform of m (-> m^ into `spec`, which may be `in`: a CTA reads all of its
 // columns before it writes them).  The forecast's time FFT of m then needs no
 // second pass over m in HBM and no conversion of m back from its stored type.
-template <class P>
-__global__ void __launch_bounds__(256, P::occ)
-k_irfft_rfft_time(const typename P::cx *in, long in_ld, void *__restrict__ out, int out_kind,
-                  long out_ld, typename P::cx *spec, long spec_ld, int N, int n_keep_all, FftPlan pl,
+template <class P, bool BIG>
+__global__ void __launch_bounds__(256, BIG ? P::occ_big : P::occ)
+k_irfft_rfft_time(const typename P::mem *in, long in_ld, void *__restrict__ out, int out_kind,
+                  long out_ld, typename P::mem *spec, long spec_ld, int N, int n_keep_all, FftPlan pl,
                   const typename P::cx *__restrict__ twM, const typename P::cx *__restrict__ twL,
                   typename P::re invM, int B, BatchArg ba) {
   typedef typename P::cx cx;
@@ -227,28 +229,29 @@ k_irfft_rfft_time(const typename P::cx *in, long in_ld, void *__restrict__ out, 
   spec += bz * ba.work_stride;
   const long ooff = bz * ba.out_stride;
   const int n_keep = ba.window(bz, n_keep_all);
-  const int M = pl.M;
+  const int M = pl.M, lgB = __ffs(B) - 1;   // B is a power of two
   cx *buf0 = reinterpret_cast<cx *>(smem_raw);
   cx *buf1 = buf0 + (M + 1) * B;
   const long n0 = (long)blockIdx.x * B;
-  stage_cols<P>(buf0, in, in_ld, n0, N, M + 1, B);
+  typename P::mem *raw = reinterpret_cast<typename P::mem *>(buf0);
+  stage_cols<P>(raw, in, in_ld, n0, N, M + 1, B);
   __syncthreads();
   // inverse: Z_k = E_k + i O_k (as in k_irfft_time)
   for (int idx = threadIdx.x; idx < M * B; idx += blockDim.x) {
-    const int b = idx % B, k = idx / B;
-    cx xk = buf0[k * B + b];
-    cx xc = P::conj(buf0[(M - k) * B + b]);
+    const int b = idx & (B - 1), k = idx >> lgB;
+    cx xk = P::from_mem(raw[k * B + b]);
+    cx xc = P::conj(P::from_mem(raw[(M - k) * B + b]));
     cx E = P::scale2(P::add(xk, xc), 0.5f);
     cx O = P::scale2(P::mul(P::sub(xk, xc), P::conj(ld_cx<P>(twL + k))), 0.5f);
     buf1[k * B + b] = P::add(E, P::mul_i(O));
   }
   __syncthreads();
-  cx *z = fft_run<P, true>(buf1, buf0, twM, pl, B, B, 1, true);
+  cx *z = fft_run<P, true, BIG>(buf1, buf0, twM, pl, B, B, 1, true);
   cx *w = z == buf0 ? buf1 : buf0;
   // m_t = invM (Re, Im) z_{t/2} for t < n_keep, else 0: written out, and
   // packed again as the forward transform's input m_{2j} + i m_{2j+1}
   for (int idx = threadIdx.x; idx < M * B; idx += blockDim.x) {
-    const int b = idx % B, j = idx / B;
+    const int b = idx & (B - 1), j = idx >> lgB;
     const long n = n0 + b;
     const cx zz = z[j * B + b];
     const int t0 = 2 * j, t1 = 2 * j + 1;
@@ -263,17 +266,17 @@ k_irfft_rfft_time(const typename P::cx *in, long in_ld, void *__restrict__ out, 
     w[j * B + b] = P::make(t0 < M ? r0 : P::re_zero(), t1 < M ? r1 : P::re_zero());
   }
   __syncthreads();
-  cx *Z = fft_run<P, false>(w, z, twM, pl, B, B, 1, true);
+  cx *Z = fft_run<P, false, BIG>(w, z, twM, pl, B, B, 1, true);
   // X_k = (Z_k + conj Z_{M-k})/2 + W_L^k (Z_k - conj Z_{M-k})/(2i)  (as in k_rfft_time)
   for (int idx = threadIdx.x; idx < (M + 1) * B; idx += blockDim.x) {
-    const int b = idx % B, k = idx / B;
+    const int b = idx & (B - 1), k = idx >> lgB;
     const long n = n0 + b;
     if (n >= N) continue;
-    cx zk = Z[(k % M) * B + b];
-    cx zc = P::conj(Z[((M - k) % M) * B + b]);
+    cx zk = Z[(k == M ? 0 : k) * B + b];
+    cx zc = P::conj(Z[(k == 0 ? 0 : M - k) * B + b]);
     cx E = P::scale2(P::add(zk, zc), 0.5f);
     cx O = P::scale2(P::mul_mi(P::sub(zk, zc)), 0.5f);
-    spec[(long)k * spec_ld + n] = P::add(E, P::mul(ld_cx<P>(twL + k), O));
+    spec[(long)k * spec_ld + n] = P::to_mem(P::add(E, P::mul(ld_cx<P>(twL + k), O)));
   }
 }
 
@@ -288,7 +291,7 @@ struct FieldMap {
 
 // rows pass: pair tp holds z = x_{2tp} + i x_{2tp+1}; FFT along b (length Ny)
 template <class P, bool INV>
-__global__ void __launch_bounds__(256, P::occ)
+__global__ void __launch_bounds__(256, P::occ_prior)
 k_prior_rows(const void *__restrict__ x, int in_kind, void *__restrict__ y, int out_kind,
              typename P::cx *__restrict__ work, int nt, int Nx, int Ny, FftPlan ply,
              const typename P::cx *__restrict__ twy, int BR, FieldMap fm, BatchArg ba, int accum) {
@@ -301,6 +304,7 @@ k_prior_rows(const void *__restrict__ x, int in_kind, void *__restrict__ y, int 
   const int a0 = blockIdx.x * BR;
   const int t0 = 2 * tp, t1 = 2 * tp + 1;
   const int bz = blockIdx.z;
+  const unsigned mag = fdiv_mag((unsigned)Ny);   // idx / Ny below without a division
   // fields t >= ntb of this batch entry are zero (input) / written as zero
   const int ntb = ba.window(bz, nt);
   const long xoff = bz * ba.in_stride, yoff = bz * ba.out_stride;
@@ -308,7 +312,9 @@ k_prior_rows(const void *__restrict__ x, int in_kind, void *__restrict__ y, int 
   if (t0 >= ntb) {
     if (INV && !accum) {
       for (int idx = threadIdx.x; idx < BR * Ny; idx += blockDim.x) {
-        const int j = idx % Ny, b = idx / Ny, a = a0 + b;
+        unsigned jq, jr;
+        fdivmod((unsigned)idx, (unsigned)Ny, mag, jq, jr);
+        const int j = (int)jr, b = (int)jq, a = a0 + b;
         if (a >= Nx) continue;
         st_out<P>(y, out_kind, yoff + ((long)fm(t0) * Nx + a) * Ny + j, P::re_zero());
         if (t1 < nt) st_out<P>(y, out_kind, yoff + ((long)fm(t1) * Nx + a) * Ny + j, P::re_zero());
@@ -317,7 +323,9 @@ k_prior_rows(const void *__restrict__ x, int in_kind, void *__restrict__ y, int 
     return;
   }
   for (int idx = threadIdx.x; idx < BR * Ny; idx += blockDim.x) {
-    const int j = idx % Ny, b = idx / Ny, a = a0 + b;
+    unsigned jq, jr;
+    fdivmod((unsigned)idx, (unsigned)Ny, mag, jq, jr);
+    const int j = (int)jr, b = (int)jq, a = a0 + b;
     cx v = P::zero();
     if (a < Nx) {
       if (!INV) {
@@ -331,9 +339,11 @@ k_prior_rows(const void *__restrict__ x, int in_kind, void *__restrict__ y, int 
     buf0[b * Ny + j] = v;
   }
   __syncthreads();
-  cx *Z = fft_run<P, INV>(buf0, buf1, twy, ply, BR, 1, Ny, false);
+  cx *Z = fft_run<P, INV, true>(buf0, buf1, twy, ply, BR, 1, Ny, false);
   for (int idx = threadIdx.x; idx < BR * Ny; idx += blockDim.x) {
-    const int j = idx % Ny, b = idx / Ny, a = a0 + b;
+    unsigned jq, jr;
+    fdivmod((unsigned)idx, (unsigned)Ny, mag, jq, jr);
+    const int j = (int)jr, b = (int)jq, a = a0 + b;
     if (a >= Nx) continue;
     cx v = Z[b * Ny + j];
     if (!INV) {
@@ -355,7 +365,7 @@ k_prior_rows(const void *__restrict__ x, int in_kind, void *__restrict__ y, int 
 // columns pass: forward FFT along a (length Nx, stride Ny), scale by lambda,
 // inverse FFT along a, in place in `work`.
 template <class P>
-__global__ void __launch_bounds__(256, P::occ)
+__global__ void __launch_bounds__(256, P::occ_prior)
 k_prior_cols(typename P::cx *__restrict__ work, const typename P::re *__restrict__ lam, int Nx,
              int Ny, FftPlan plx, const typename P::cx *__restrict__ twx, int BC, int nt,
              BatchArg ba) {
@@ -363,26 +373,27 @@ k_prior_cols(typename P::cx *__restrict__ work, const typename P::re *__restrict
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx *buf0 = reinterpret_cast<cx *>(smem_raw);
   cx *buf1 = buf0 + Nx * BC;
+  const int lgB = __ffs(BC) - 1;   // BC is a power of two
   const int tp = blockIdx.y;
   const int j0 = blockIdx.x * BC;
   const int bz = blockIdx.z;
   if (2 * tp >= ba.window(bz, nt)) return;
   cx *wp = work + bz * ba.work_stride + (long)tp * Nx * Ny;
   for (int idx = threadIdx.x; idx < Nx * BC; idx += blockDim.x) {
-    const int b = idx % BC, a = idx / BC, j = j0 + b;
+    const int b = idx & (BC - 1), a = idx >> lgB, j = j0 + b;
     buf0[a * BC + b] = (j < Ny) ? wp[(long)a * Ny + j] : P::zero();
   }
   __syncthreads();
-  cx *Z = fft_run<P, false>(buf0, buf1, twx, plx, BC, BC, 1, true);
+  cx *Z = fft_run<P, false, true>(buf0, buf1, twx, plx, BC, BC, 1, true);
   cx *O = (Z == buf0) ? buf1 : buf0;
   for (int idx = threadIdx.x; idx < Nx * BC; idx += blockDim.x) {
-    const int b = idx % BC, p = idx / BC, j = j0 + b;
+    const int b = idx & (BC - 1), p = idx >> lgB, j = j0 + b;
     if (j < Ny) Z[p * BC + b] = P::scale_re(Z[p * BC + b], lam[(long)p * Ny + j]);
   }
   __syncthreads();
-  cx *Y = fft_run<P, true>(Z, O, twx, plx, BC, BC, 1, true);
+  cx *Y = fft_run<P, true, true>(Z, O, twx, plx, BC, BC, 1, true);
   for (int idx = threadIdx.x; idx < Nx * BC; idx += blockDim.x) {
-    const int b = idx % BC, a = idx / BC, j = j0 + b;
+    const int b = idx & (BC - 1), a = idx >> lgB, j = j0 + b;
     if (j < Ny) wp[(long)a * Ny + j] = Y[a * BC + b];
   }
 }
@@ -396,11 +407,14 @@ k_cfield_rows(cdd *__restrict__ x, cd *__restrict__ work, int Nx, int Ny, FftPla
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cd *buf0 = reinterpret_cast<cd *>(smem_raw);
   cd *buf1 = buf0 + BR * Ny;
+  const unsigned mag = fdiv_mag((unsigned)Ny);
   const int f = blockIdx.y, a0 = blockIdx.x * BR;
   cdd *xf = x + (long)f * Nx * Ny;
   cd *wf = work + (long)f * Nx * Ny;
   for (int idx = threadIdx.x; idx < BR * Ny; idx += blockDim.x) {
-    const int j = idx % Ny, b = idx / Ny, a = a0 + b;
+    unsigned jq, jr;
+    fdivmod((unsigned)idx, (unsigned)Ny, mag, jq, jr);
+    const int j = (int)jr, b = (int)jq, a = a0 + b;
     cd v = PolD::zero();
     if (a < Nx) {
       if (!INV) {
@@ -413,9 +427,11 @@ k_cfield_rows(cdd *__restrict__ x, cd *__restrict__ work, int Nx, int Ny, FftPla
     buf0[b * Ny + j] = v;
   }
   __syncthreads();
-  cd *Z = fft_run<PolD, INV>(buf0, buf1, twy, ply, BR, 1, Ny, false);
+  cd *Z = fft_run<PolD, INV, true>(buf0, buf1, twy, ply, BR, 1, Ny, false);
   for (int idx = threadIdx.x; idx < BR * Ny; idx += blockDim.x) {
-    const int j = idx % Ny, b = idx / Ny, a = a0 + b;
+    unsigned jq, jr;
+    fdivmod((unsigned)idx, (unsigned)Ny, mag, jq, jr);
+    const int j = (int)jr, b = (int)jq, a = a0 + b;
     if (a >= Nx) continue;
     const cd v = Z[b * Ny + j];
     if (!INV) {
@@ -442,32 +458,52 @@ int pick_batch(int len, size_t elem, int cap, size_t budget) {
 }
 
 template <class P>
-cudaError_t rfft_time(const void *in, int in_kind, long in_ld, int n_in, typename P::cx *out,
+cudaError_t rfft_time(const void *in, int in_kind, long in_ld, int n_in, typename P::mem *out,
                       long out_ld, int N, const FftPlan &pl, const typename P::cx *twM,
                       const typename P::cx *twL, cudaStream_t s, BatchArg ba = BatchArg{}) {
   if (N <= 0 || ba.count <= 0) return cudaSuccess;
   const int B = pick_batch(pl.M + 1, sizeof(typename P::cx), 32, P::smem);
   const size_t sm = (size_t)2 * (pl.M + 1) * B * sizeof(typename P::cx);
-  ensure_smem(k_rfft_time<P>, sm);
   const dim3 grid((unsigned)((N + B - 1) / B), (unsigned)ba.count);
-  k_rfft_time<P><<<grid, 256, sm, s>>>(in, in_kind, in_ld, n_in, out, out_ld, N, pl, twM, twL, B,
+  const bool big = P::fused && fft_big(pl);
+  if constexpr (P::fused) {
+    if (big) {
+      ensure_smem(k_rfft_time<P, true>, sm);
+      k_rfft_time<P, true><<<grid, 256, sm, s>>>(in, in_kind, in_ld, n_in, out, out_ld, N, pl, twM, twL, B,
                                        ba);
+    }
+  }
+  if (!big) {
+    ensure_smem(k_rfft_time<P, false>, sm);
+    k_rfft_time<P, false><<<grid, 256, sm, s>>>(in, in_kind, in_ld, n_in, out, out_ld, N, pl, twM, twL, B,
+                                       ba);
+  }
   count_launches(1);
   return cudaGetLastError();
 }
 
 template <class P>
-cudaError_t irfft_time(const typename P::cx *in, long in_ld, void *out, int out_kind, long out_ld,
+cudaError_t irfft_time(const typename P::mem *in, long in_ld, void *out, int out_kind, long out_ld,
                        int N, int n_keep, const FftPlan &pl, const typename P::cx *twM,
                        const typename P::cx *twL, typename P::re invM, cudaStream_t s,
                        BatchArg ba = BatchArg{}) {
   if (N <= 0 || ba.count <= 0) return cudaSuccess;
   const int B = pick_batch(pl.M + 1, sizeof(typename P::cx), 32, P::smem);
   const size_t sm = (size_t)2 * (pl.M + 1) * B * sizeof(typename P::cx);
-  ensure_smem(k_irfft_time<P>, sm);
   const dim3 grid((unsigned)((N + B - 1) / B), (unsigned)ba.count);
-  k_irfft_time<P><<<grid, 256, sm, s>>>(in, in_ld, out, out_kind, out_ld, N, n_keep, pl, twM, twL,
+  const bool big = P::fused && fft_big(pl);
+  if constexpr (P::fused) {
+    if (big) {
+      ensure_smem(k_irfft_time<P, true>, sm);
+      k_irfft_time<P, true><<<grid, 256, sm, s>>>(in, in_ld, out, out_kind, out_ld, N, n_keep, pl, twM, twL,
                                         invM, B, ba);
+    }
+  }
+  if (!big) {
+    ensure_smem(k_irfft_time<P, false>, sm);
+    k_irfft_time<P, false><<<grid, 256, sm, s>>>(in, in_ld, out, out_kind, out_ld, N, n_keep, pl, twM, twL,
+                                        invM, B, ba);
+  }
   count_launches(1);
   return cudaGetLastError();
 }
@@ -502,12 +538,15 @@ cudaError_t prior(const void *x, int in_kind, void *y, int out_kind, int nt, int
   return cudaGetLastError();
 }
 
+// the double-float twiddle tables are stored as packed pairs (upload_twiddles)
+const cdp *packed(const cdd *t) { return reinterpret_cast<const cdp *>(t); }
+
 }  // namespace
 
 cudaError_t launch_rfft_time_dd(const void *in, int in_kind, long in_ld, int n_in, cdd *out,
                                 long out_ld, int N, const FftPlan &pl, const cdd *twM,
                                 const cdd *twL, cudaStream_t s, const BatchArg &ba) {
-  return rfft_time<PolDD>(in, in_kind, in_ld, n_in, out, out_ld, N, pl, twM, twL, s, ba);
+  return rfft_time<PolDD>(in, in_kind, in_ld, n_in, out, out_ld, N, pl, packed(twM), packed(twL), s, ba);
 }
 cudaError_t launch_rfft_time_f(const void *in, int in_kind, long in_ld, int n_in, cf *out,
                                long out_ld, int N, const FftPlan &pl, const cf *twM,
@@ -515,17 +554,27 @@ cudaError_t launch_rfft_time_f(const void *in, int in_kind, long in_ld, int n_in
   return rfft_time<PolF>(in, in_kind, in_ld, n_in, out, out_ld, N, pl, twM, twL, s, ba);
 }
 template <class P>
-cudaError_t irfft_rfft_time(const typename P::cx *in, long in_ld, void *out, int out_kind, long out_ld,
-                            typename P::cx *spec, long spec_ld, int N, int n_keep, const FftPlan &pl,
+cudaError_t irfft_rfft_time(const typename P::mem *in, long in_ld, void *out, int out_kind, long out_ld,
+                            typename P::mem *spec, long spec_ld, int N, int n_keep, const FftPlan &pl,
                             const typename P::cx *twM, const typename P::cx *twL, typename P::re invM,
                             cudaStream_t s, const BatchArg &ba) {
   if (N <= 0 || ba.count <= 0) return cudaSuccess;
   const int B = pick_batch(pl.M + 1, sizeof(typename P::cx), 32, P::smem);
   const size_t sm = (size_t)2 * (pl.M + 1) * B * sizeof(typename P::cx);
-  ensure_smem(k_irfft_rfft_time<P>, sm);
   const dim3 grid((unsigned)((N + B - 1) / B), (unsigned)ba.count);
-  k_irfft_rfft_time<P><<<grid, 256, sm, s>>>(in, in_ld, out, out_kind, out_ld, spec, spec_ld, N, n_keep, pl,
+  const bool big = P::fused && fft_big(pl);
+  if constexpr (P::fused) {
+    if (big) {
+      ensure_smem(k_irfft_rfft_time<P, true>, sm);
+      k_irfft_rfft_time<P, true><<<grid, 256, sm, s>>>(in, in_ld, out, out_kind, out_ld, spec, spec_ld, N, n_keep, pl,
                                              twM, twL, invM, B, ba);
+    }
+  }
+  if (!big) {
+    ensure_smem(k_irfft_rfft_time<P, false>, sm);
+    k_irfft_rfft_time<P, false><<<grid, 256, sm, s>>>(in, in_ld, out, out_kind, out_ld, spec, spec_ld, N, n_keep, pl,
+                                             twM, twL, invM, B, ba);
+  }
   count_launches(1);
   return cudaGetLastError();
 }
@@ -537,8 +586,8 @@ cudaError_t launch_irfft_rfft_time_dd(const cdd *in, long in_ld, void *out, int 
   dd invM;
   invM.hi = (float)inv;
   invM.lo = (float)(inv - (double)invM.hi);
-  return irfft_rfft_time<PolDD>(in, in_ld, out, out_kind, out_ld, spec, spec_ld, N, n_keep, pl, twM, twL,
-                                invM, s, ba);
+  return irfft_rfft_time<PolDD>(in, in_ld, out, out_kind, out_ld, spec, spec_ld, N, n_keep, pl,
+                                packed(twM), packed(twL), invM, s, ba);
 }
 cudaError_t launch_irfft_rfft_time_f(const cf *in, long in_ld, void *out, int out_kind, long out_ld,
                                      cf *spec, long spec_ld, int N, int n_keep, const FftPlan &pl,
@@ -554,7 +603,8 @@ cudaError_t launch_irfft_time_dd(const cdd *in, long in_ld, void *out, int out_k
   dd invM;
   invM.hi = (float)inv;
   invM.lo = (float)(inv - (double)invM.hi);
-  return irfft_time<PolDD>(in, in_ld, out, out_kind, out_ld, N, n_keep, pl, twM, twL, invM, s, ba);
+  return irfft_time<PolDD>(in, in_ld, out, out_kind, out_ld, N, n_keep, pl, packed(twM), packed(twL), invM, s,
+                           ba);
 }
 cudaError_t launch_irfft_time_f(const cf *in, long in_ld, void *out, int out_kind, long out_ld,
                                 int N, int n_keep, const FftPlan &pl, const cf *twM,
@@ -566,7 +616,8 @@ cudaError_t launch_prior_dd(const void *x, int in_kind, void *y, int out_kind, i
                             int Ny, cdd *work, const dd *lam, const FftPlan &plx,
                             const FftPlan &ply, const cdd *twx, const cdd *twy, cudaStream_t s,
                             const BatchArg &ba, int accum) {
-  return prior<PolDD>(x, in_kind, y, out_kind, nt, Nx, Ny, work, lam, plx, ply, twx, twy, s,
+  return prior<PolDD>(x, in_kind, y, out_kind, nt, Nx, Ny, reinterpret_cast<cdp *>(work), lam, plx, ply,
+                      packed(twx), packed(twy), s,
                       FieldMap{1 << 30, 0, 0}, ba, accum);
 }
 cudaError_t launch_prior_d(const void *x, int in_kind, void *y, int out_kind, int nt, int Nx,

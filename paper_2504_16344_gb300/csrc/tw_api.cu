@@ -94,18 +94,45 @@ FftPlan make_plan(int M) {
   int m = M, n = 0;
   const int small[5] = {4, 2, 3, 5, 7};
   for (int r : small)
-    while (m % r == 0 && n < TW_FFT_MAX_STAGES) { p.R[n++] = r; m /= r; }
+    while (m % r == 0 && n < TW_FFT_MAX_STAGES) { p.st.R[n++] = r; m /= r; }
   for (int q = 11; m > 1 && n < TW_FFT_MAX_STAGES; q += 2)
-    while (m % q == 0 && n < TW_FFT_MAX_STAGES) { p.R[n++] = q; m /= q; }
-  if (m > 1) p.R[n++] = m;  // remaining factor (only for absurd lengths)
-  p.nst = n;
+    while (m % q == 0 && n < TW_FFT_MAX_STAGES) { p.st.R[n++] = q; m /= q; }
+  if (m > 1) p.st.R[n++] = m;  // remaining factor (only for absurd lengths)
+  p.st.nst = n;
+  for (int i = 0; i < n; ++i) p.st.R2[i] = 1;
+  // neighbours fused: the fewest passes, and of those the smallest largest
+  // radix (fewer registers, more butterflies); best[i]: from stage i on
+  auto fusable = [](int a, int b) {
+#define TW_FFT_PAIR(A, C) || (a == A && b == C)
+    return (a == 5 && b == 5) TW_FFT_PAIRS(TW_FFT_PAIR);
+#undef TW_FFT_PAIR
+  };
+  struct Tail { int passes, largest; bool pair; };
+  std::vector<Tail> best(n + 2, Tail{0, 0, false});
+  for (int i = n - 1; i >= 0; --i) {
+    const int *R = p.st.R;
+    best[i] = Tail{1 + best[i + 1].passes, std::max(R[i] <= 7 ? R[i] : 0, best[i + 1].largest), false};
+    if (i + 1 < n && fusable(R[i], R[i + 1])) {
+      const Tail two{1 + best[i + 2].passes, std::max(R[i] * R[i + 1], best[i + 2].largest), true};
+      if (two.passes < best[i].passes || (two.passes == best[i].passes && two.largest < best[i].largest)) best[i] = two;
+    }
+  }
+  int nc = 0;
+  for (int i = 0; i < n; ++nc) {
+    p.fst.R[nc] = p.st.R[i];
+    p.fst.R2[nc] = best[i].pair ? p.st.R[i + 1] : 1;
+    i += best[i].pair ? 2 : 1;
+  }
+  p.fst.nst = nc;
   // magic multipliers for the engine's divisions by p and by S = M / R
   auto mag = [](unsigned x) -> unsigned { return x <= 1 ? 0u : (unsigned)((1ull << 32) / x); };
-  int prod = 1;
-  for (int st = 0; st < n; ++st) {
-    p.pmag[st] = mag((unsigned)prod);
-    p.smag[st] = mag((unsigned)(M / p.R[st]));
-    prod *= p.R[st];
+  for (FftStages *f : {&p.st, &p.fst}) {
+    int prod = 1;
+    for (int st = 0; st < f->nst; ++st) {
+      f->pmag[st] = mag((unsigned)prod);
+      f->smag[st] = mag((unsigned)(M / (f->R[st] * f->R2[st])));
+      prod *= f->R[st] * f->R2[st];
+    }
   }
   return p;
 }
@@ -134,8 +161,12 @@ tw_status upload_twiddles(tw_ctx *c, int n, double denom, cdd **out_dd, cf **out
   for (int t = 0; t < n; ++t) {
     const double a = -2.0 * kPi * (double)t / denom;
     const double cr = cos(a), ci = sin(a);
-    split_dd(cr, h[t].re);
-    split_dd(ci, h[t].im);
+    dd re, im;
+    split_dd(cr, re);
+    split_dd(ci, im);
+    // in the order of the FFT engine's packed pairs: both high parts, both low parts
+    h[t].re.hi = re.hi; h[t].re.lo = im.hi;
+    h[t].im.hi = re.lo; h[t].im.lo = im.lo;
     hf[t].re = (float)cr;
     hf[t].im = (float)ci;
   }
