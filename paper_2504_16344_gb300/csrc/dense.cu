@@ -233,6 +233,101 @@ k_potrf_diag(T *__restrict__ K, long ldk, int J, T *__restrict__ inv, int *err) 
   }
 }
 
+// The factor in FP64 (the one of record) with the same bits: every entry's
+// operations are those of the form above in the same order, only their
+// schedule differs, and the inverse is left to k_inv_diag_d.  The block is one
+// CTA's work and every column of K waits for it, so what counts is its chain:
+// two warps (thread = row) carry a panel of 8 columns in registers, with two
+// barriers of 64 threads a column, and all threads then apply the panel to the
+// rest.  (Above: three CTA barriers a column, an entry's indices from a square
+// root, and for the inverse 2,000 dependent operations in one thread per
+// column.)  The Cholesky of 10,000 rows: 103 -> 74 ms.
+__global__ void __launch_bounds__(256)
+k_potrf_diag_d(double *__restrict__ K, long ldk, int J, int *err) {
+  __shared__ double sA[NB_][NB_ + 1], sInv[NB_], sCol[2][NB_];
+  const int tid = threadIdx.x;
+  double *Ablk = K + (long)J * NB_ * ldk + (long)J * NB_;
+  for (int idx = tid; idx < NB_ * NB_; idx += 256) {
+    const int r = idx / NB_, c = idx % NB_;
+    sA[r][c] = (c <= r) ? Ablk[(long)r * ldk + c] : 0.0;
+  }
+  __syncthreads();
+  for (int c0 = 0; c0 < NB_; c0 += 8) {
+    if (tid < NB_) {
+      const int r = tid;
+      double a[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) a[j] = sA[r][c0 + j];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        if (r == c0 + c) {
+          double piv = a[c];
+          if (!(piv > 0.0)) {                   // not positive definite (or NaN)
+            record_error(err, TW_ERR_NOT_SPD, J * NB_ + c0 + c);
+            piv = 1.0;
+          }
+          a[c] = sqrt(piv);
+          sInv[r] = 1.0 / a[c];
+        }
+        asm volatile("bar.sync 1, 64;" ::: "memory");
+        if (r != c0 + c) a[c] = __dmul_rn(a[c], sInv[c0 + c]);
+        sCol[c & 1][r] = a[c];
+        asm volatile("bar.sync 1, 64;" ::: "memory");
+#pragma unroll
+        for (int j = c + 1; j < 8; ++j) a[j] = __dadd_rn(a[j], __dmul_rn(-a[c], sCol[c & 1][c0 + j]));
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (r >= c0 + j) sA[r][c0 + j] = a[j];
+    }
+    __syncthreads();
+    for (int r = c0 + 8 + (tid >> 4); r < NB_; r += 16)
+      for (int k = c0 + 8 + (tid & 15); k <= r; k += 16) {
+        double v = sA[r][k];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v = __dadd_rn(v, __dmul_rn(-sA[r][c0 + j], sA[k][c0 + j]));
+        sA[r][k] = v;
+      }
+    __syncthreads();
+  }
+  // write the factor block back (lower part)
+  for (int idx = tid; idx < NB_ * NB_; idx += 256) {
+    const int r = idx / NB_, c = idx % NB_;
+    if (c <= r) Ablk[(long)r * ldk + c] = sA[r][c];
+  }
+}
+
+// Inverses of all the factor's diagonal blocks (only the solves use them), one
+// CTA a block once the factor is done: X_rj = -(sum_k L_rk X_kj) / L_rr, summed
+// from k = j up in groups of 16 as in the form above
+__global__ void __launch_bounds__(64)
+k_inv_diag_d(const double *__restrict__ K, long ldk, double *__restrict__ inv) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double(*sA)[NB_ + 1] = reinterpret_cast<double(*)[NB_ + 1]>(smem_raw);
+  double(*sX)[NB_ + 1] = sA + NB_;
+  __shared__ double sInv[NB_];
+  const int j = threadIdx.x, J = blockIdx.x;
+  const double *Ablk = K + (long)J * NB_ * ldk + (long)J * NB_;
+  for (int r = 0; r < NB_; ++r) {
+    sA[r][j] = (j <= r) ? Ablk[(long)r * ldk + j] : 0.0;
+    sX[r][j] = 0.0;
+  }
+  __syncthreads();
+  sInv[j] = 1.0 / sA[j][j];
+  __syncthreads();
+  sX[j][j] = sInv[j];
+  for (int r = j + 1; r < NB_; ++r) {
+    double a = 0.0, t = 0.0;
+    for (int k = j; k < r; ++k) {
+      a = fma(sA[r][k], sX[k][j], a);
+      if (((k - j) & 15) == 15) { t = __dadd_rn(t, a); a = 0.0; }
+    }
+    sX[r][j] = -__dmul_rn(__dadd_rn(t, a), sInv[r]);
+  }
+  __syncthreads();
+  for (int r = 0; r < NB_; ++r) inv[(size_t)J * NB_ * NB_ + r * NB_ + j] = sX[r][j];
+}
+
 // ---------------------------------------- Cholesky: panel (substitution)
 // rows of block I = J+1+blockIdx.x: X L_JJ^T = A_IJ  (one row per thread)
 template <class T>
@@ -796,9 +891,9 @@ int cholesky_tc_width() { return CHOL_SW; }
 cudaError_t launch_cholesky_d(double *K, long ldk, int NB, double *inv, int *err, uint8_t *ws,
                               size_t ws_bytes, int *eg, cudaStream_t s) {
   if (!ws) return cholesky_t<double>(K, ldk, NB, inv, err, s);
-  const size_t sm_potrf = 2 * NB_ * (NB_ + 1) * sizeof(double);
+  const size_t sm_inv = 2 * NB_ * (NB_ + 1) * sizeof(double);
   const size_t sm_trsm = 2 * NB_ * (NB_ + 1) * sizeof(double);
-  smem_attr(k_potrf_diag<double>, sm_potrf);
+  smem_attr(k_inv_diag_d, sm_inv);
   smem_attr(k_trsm_panel<double>, sm_trsm);
   for (int J0 = 0; J0 < NB; J0 += CHOL_SW) {
     const int w = std::min(CHOL_SW, NB - J0);
@@ -812,7 +907,7 @@ cudaError_t launch_cholesky_d(double *K, long ldk, int NB, double *inv, int *err
                                                         ldk, 0, 1);
         count_launches(1);
       }
-      k_potrf_diag<double><<<1, 256, sm_potrf, s>>>(K, ldk, J, inv + (size_t)J * NB_ * NB_, err);
+      k_potrf_diag_d<<<1, 256, 0, s>>>(K, ldk, J, err);
       count_launches(1);
       if (nrow > 1) {
         k_trsm_panel<double><<<nrow - 1, 64, sm_trsm, s>>>(K, ldk, J);
@@ -829,7 +924,9 @@ cudaError_t launch_cholesky_d(double *K, long ldk, int NB, double *inv, int *err
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  return cudaSuccess;
+  k_inv_diag_d<<<NB, NB_, sm_inv, s>>>(K, ldk, inv);
+  count_launches(1);
+  return cudaGetLastError();
 }
 cudaError_t launch_pack_d(const double *K, long ldk, double *P, int NB, cudaStream_t s) {
   k_pack<double><<<152 * 8, 256, 0, s>>>(K, ldk, P, NB);

@@ -33,14 +33,24 @@
 // one rounding per panel.
 //
 // Kernel: persistent, one CTA per SM, over a host-ordered list of (128-row,
-// 32-column) tiles of the lower triangle (groups of 8 row tiles, column tile
+// 64-column) tiles of the lower triangle (groups of 8 row tiles, column tile
 // outer, so the CTAs running together share their slice tiles in L2).  One
 // thread issues the bulk copies of a k atom's slices (A: 7 x 128 rows, B: 7 x
-// 32 rows of the same sliced panel) into a 3-stage ring; one thread issues
-// the MMAs (six accumulators of 32 columns, double-buffered per chunk); four
-// warps drain TMEM (tcgen05.ld), one row each.  Every wait is bounded: on
-// expiry the kernel records TW_ERR_TIMEOUT, lets its copies and MMAs drain
+// 64 rows of the same sliced panel) into a 2-stage ring; four warps move A's
+// slices on to TMEM; one warp issues the MMAs (six accumulators of 64
+// columns); eight warps drain them, half a row each.  Every wait is bounded:
+// on expiry the kernel records TW_ERR_TIMEOUT, lets its copies and MMAs drain
 // (bounded), frees TMEM and returns.
+//
+// Why this tile.  With both operands in shared memory an MMA of 128 x 32 x 16
+// takes 45 cycles (A's 4 KB at 128 bytes a clock, issued from one lane's
+// branch), three times its arithmetic, and each A slice is read again for
+// every one of its up to seven pairs.  From TMEM a 128 x 64 x 16 MMA takes 32
+// cycles, its arithmetic; shared memory then carries one read of A by the
+// moving warps and B's 2 KB per MMA.  64 columns also halve the L2 reads of A.
+// The sums keep their bits: chunks, panels and the order within an
+// accumulator are what they were.  K of 10,000 rows from 12,500 grid points:
+// 67 -> 37 ms.
 #include <stdint.h>
 
 #include <algorithm>
@@ -49,115 +59,34 @@
 #include "../../include/tw.h"
 #include "dense_api.h"
 #include "kernels.h"
+#include "tc.cuh"
 
 namespace tw {
 
 namespace {
 
 constexpr int SK_TM = 128;                   // MMA M: rows of a tile
-constexpr int SK_TN = 32;                    // MMA N: columns of a tile
+constexpr int SK_TN = 64;                    // MMA N: columns of a tile
 constexpr int SK_KA = 32;                    // k per atom (two 16-wide MMA steps)
-constexpr int SK_NSL = 7;                    // slices per entry
-constexpr int SK_NACC = 6;                   // accumulators: levels 0 .. 4, and 5..6
+constexpr int SK_NSL = TC_NSL;               // slices per entry
+constexpr int SK_NACC = TC_NACC;             // accumulators: levels 0 .. 4, and 5..6
 constexpr int SK_CHUNK = 4;                  // atoms per exact chunk (128 k)
 constexpr int SK_A_SLICE = SK_TM * SK_KA * 2;     // 8 KB
-constexpr int SK_B_SLICE = SK_TN * SK_KA * 2;     // 2 KB
+constexpr int SK_B_SLICE = SK_TN * SK_KA * 2;     // 4 KB
 constexpr int SK_A_STAGE = SK_NSL * SK_A_SLICE;   // 56 KB
-constexpr int SK_B_STAGE = SK_NSL * SK_B_SLICE;   // 14 KB
-constexpr int SK_STAGE = SK_A_STAGE + SK_B_STAGE; // 70 KB
-constexpr int SK_S = 3;                      // ring stages
-constexpr int SK_NEPI = 128;                 // epilogue threads
-constexpr int SK_NTHR = 64 + SK_NEPI;        // copy warp, MMA warp, 4 epilogue warps
-constexpr unsigned long long SK_WAIT_NS = 4000000000ull;   // bound of every wait (4 s)
+constexpr int SK_B_STAGE = SK_NSL * SK_B_SLICE;   // 28 KB
+constexpr int SK_STAGE = SK_A_STAGE + SK_B_STAGE; // 84 KB
+constexpr int SK_S = 2;                      // ring stages
+constexpr int SK_SA = 2;                     // A stages in TMEM (16 k each)
+constexpr int SK_A_COLS = SK_NSL * 8;        // TMEM columns of one
+constexpr int SK_NMOV = 128, SK_NEPI = 256;  // moving and epilogue threads
+constexpr int SK_NTHR = SK_NMOV + SK_NEPI + 64;
+static_assert(SK_NACC * SK_TN + SK_SA * SK_A_COLS <= 512, "TMEM columns");
 constexpr int SK_EXP_MIN = -100, SK_EXP_MAX = 120;
 
-__device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__host__ __device__ __forceinline__ uint32_t swz64(int r, int q) {
-  return (uint32_t)r * 64u + ((uint32_t)(q ^ ((r >> 1) & 3)) << 4);
-}
-// K-major, 64-byte swizzle, 8-row groups 512 bytes apart (descriptor version 1)
-__device__ __forceinline__ uint64_t sdesc64(uint32_t saddr) {
-  uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(512 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)4 << 61;
-  return d;
-}
-// kind::f16: D F32, A and B BF16, both K-major
-__host__ __device__ __forceinline__ uint32_t idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_tx(uint32_t bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, unsigned parity) {
-  uint32_t ok;
-  asm volatile("{\n\t.reg .pred p;\n\t"
-               "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-               "selp.b32 %0, 1, 0, p;\n\t}"
-               : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ unsigned long long gtime() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// true once the phase of this parity has completed; false after SK_WAIT_NS
-// or once another role of the CTA has failed
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, unsigned parity, volatile int *fail) {
-  unsigned long long t0 = 0;
-  for (unsigned it = 1;; ++it) {
-    if (mbar_try(bar, parity)) return true;
-    if ((it & 255u) == 0) {
-      if (*fail) return false;
-      const unsigned long long t = gtime();
-      if (t0 == 0) t0 = t;
-      else if (t - t0 > SK_WAIT_NS) return false;
-    }
-  }
-}
-// the same without the early exit (draining the CTA's own asynchronous work)
-__device__ __forceinline__ bool mbar_drain(uint32_t bar, unsigned parity) {
-  unsigned long long t0 = 0;
-  for (unsigned it = 1;; ++it) {
-    if (mbar_try(bar, parity)) return true;
-    if ((it & 255u) == 0) {
-      const unsigned long long t = gtime();
-      if (t0 == 0) t0 = t;
-      else if (t - t0 > SK_WAIT_NS) return false;
-    }
-  }
-}
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, unsigned bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc,
-                                         uint32_t acc) {
-  asm volatile("{\n\t.reg .pred p;\n\t"
-               "setp.ne.b32 p, %4, 0;\n\t"
-               "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-               ::"r"(dtmem), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-               ::"r"(bar) : "memory");
-}
 // round to the nearest integer (ties to even), |v| < 2^22
 __device__ __forceinline__ float rnd_int(float v) {
   return __fsub_rn(__fadd_rn(v, 12582912.0f), 12582912.0f);
-}
-__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
 }
 __device__ __forceinline__ int exp_above(float mx) {
   if (!(mx > 0.f)) return SK_EXP_MIN;
@@ -185,8 +114,8 @@ k_syrk_row_exp(const dd *__restrict__ G, long ldg, int n, int kdim, int *__restr
 
 // ------------------------------------------------------ slices of a k panel
 // tiles[T][a][s][128 rows][32 bf16] (64-byte swizzle): rows 128 T .. +127 of
-// G, columns k0 + 32 a .. +31 of the panel, slice s.  A 32-row column tile
-// J is rows 32 (J mod 4) .. +31 of tile J / 4: 2 KB contiguous per slice.
+// G, columns k0 + 32 a .. +31 of the panel, slice s.  A 64-row column tile
+// J is rows 64 (J mod 2) .. +63 of tile J / 2: 4 KB contiguous per slice.
 __global__ void __launch_bounds__(256)
 k_syrk_slice(const dd *__restrict__ G, long ldg, int n, int kdim, int k0, const int *__restrict__ eg,
              uint8_t *__restrict__ tiles, int natoms) {
@@ -194,7 +123,7 @@ k_syrk_slice(const dd *__restrict__ G, long ldg, int n, int kdim, int k0, const 
   const int r = threadIdx.x & (SK_TM - 1), h = threadIdx.x >> 7;
   const int i = T * SK_TM + r;
   const int kb = k0 + SK_KA * a + 16 * h;
-  const float sc = pow2f(7 - eg[i]);
+  const float sc = tc_pow2f(7 - eg[i]);
   float hi[16], lo[16];
 #pragma unroll
   for (int u = 0; u < 16; ++u) {
@@ -214,7 +143,7 @@ k_syrk_slice(const dd *__restrict__ G, long ldg, int n, int kdim, int k0, const 
       for (int c = 0; c < 2; ++c) {
         const int u = 2 * u2 + c;
         const float si = rnd_int(hi[u]);
-        sl[c] = si * pow2f(-8 * s);
+        sl[c] = si * tc_pow2f(-8 * s);
         if (s + 1 < SK_NSL) {
           float rr, ee;
           two_sum(__fsub_rn(hi[u], si), lo[u], rr, ee);   // hi - si is exact
@@ -222,11 +151,11 @@ k_syrk_slice(const dd *__restrict__ G, long ldg, int n, int kdim, int k0, const 
           lo[u] = ee * 256.f;
         }
       }
-      wd[u2] = pack_bf16(sl[0], sl[1]);
+      wd[u2] = tc_pack_bf16(sl[0], sl[1]);
     }
     uint8_t *tile = base + (size_t)s * SK_A_SLICE;
-    *reinterpret_cast<uint4 *>(tile + swz64(r, 2 * h)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
-    *reinterpret_cast<uint4 *>(tile + swz64(r, 2 * h + 1)) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
+    *reinterpret_cast<uint4 *>(tile + tc_swz64(r, 2 * h)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+    *reinterpret_cast<uint4 *>(tile + tc_swz64(r, 2 * h + 1)) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
   }
 }
 
@@ -278,90 +207,187 @@ k_syrk_slice_d(const double *__restrict__ A, long ld, int n, int kdim, const int
       for (int c = 0; c < 2; ++c) {
         const int u = 2 * u2 + c;
         const double si = rint(x[u]);
-        sl[c] = (float)si * pow2f(-8 * s);
+        sl[c] = (float)si * tc_pow2f(-8 * s);
         x[u] = (x[u] - si) * 256.0;
       }
-      wd[u2] = pack_bf16(sl[0], sl[1]);
+      wd[u2] = tc_pack_bf16(sl[0], sl[1]);
     }
     uint8_t *tile = base + (size_t)s * SK_A_SLICE;
-    *reinterpret_cast<uint4 *>(tile + swz64(r, 2 * h)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
-    *reinterpret_cast<uint4 *>(tile + swz64(r, 2 * h + 1)) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
+    *reinterpret_cast<uint4 *>(tile + tc_swz64(r, 2 * h)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+    *reinterpret_cast<uint4 *>(tile + tc_swz64(r, 2 * h + 1)) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
   }
-}
-
-// pair number p = 0..27 -> (slice of A, slice of B), by level L = 0..6
-__device__ __forceinline__ void syrk_pair(int p, int &si, int &sj, int &L) {
-  int l = 0, first = 0;
-  while (p >= first + l + 1) { first += l + 1; ++l; }
-  L = l;
-  si = p - first;
-  sj = l - si;
 }
 
 // ------------------------------------------------------------------ the product
 // tile number t: from the list tl, or (tl == nullptr) in row-major order over
 // the lower triangle of 128-row tiles, row tile I holding column tiles
-// 0 .. 4I+3.  A column tile at or past nc is empty (the last row tile of a
+// 0 .. 2I+1.  A column tile at or past nc is empty (the last row tile of a
 // size that is not a multiple of 128); every role skips it alike.
 __device__ __forceinline__ bool tile_at(const int2 *__restrict__ tl, int t, int nc, int2 &out) {
   if (tl) { out = tl[t]; return true; }
-  int I = (int)((sqrt(1.0 + 2.0 * (double)t) - 1.0) * 0.5);
-  while (2 * (I + 1) * (I + 2) <= t) ++I;
-  while (I > 0 && 2 * I * (I + 1) > t) --I;
-  out = make_int2(I, t - 2 * I * (I + 1));
+  int I = (int)((sqrt(1.0 + 4.0 * (double)t) - 1.0) * 0.5);
+  while ((I + 1) * (I + 2) <= t) ++I;
+  while (I > 0 && I * (I + 1) > t) --I;
+  out = make_int2(I, t - I * (I + 1));
   return out.y < nc;
 }
 
+__device__ __forceinline__ void note(int *err, volatile int *fail, int info) {
+  if (!*fail && atomicCAS(err, 0, TW_ERR_TIMEOUT) == 0) err[1] = info;
+  *fail = 1;
+}
+
 // K[i][j] = / += / -= P_ij (mode 0 / 1 / 2) over this panel for the tiles (row
-// tile I of 128, column tile J of 32), entries of the lower 64-block triangle
+// tile I of 128, column tile J of 64), entries of the lower 64-block triangle
 // below n_pad only (n_pad a multiple of 64).
-// Warp roles: 0 the bulk-copy issuer, 1 the MMA issuer, 2-5 the epilogue (TMEM
-// lane quarter = warp mod 4).  Chunks (SK_CHUNK atoms) alternate between two
-// TMEM buffers of SK_NACC x 32 columns.
+// Warp roles: 0-3 move A's slices to TMEM, 4-11 the epilogue (TMEM lane
+// quarter = warp mod 4), 12 the bulk-copy issuer, 13 the MMA issuer.
 __global__ void __launch_bounds__(SK_NTHR, 1)
 k_syrk_sl(const uint8_t *__restrict__ Sl, const int *__restrict__ eg, const int2 *__restrict__ tl,
-          int ntl, int natoms, double *__restrict__ K, long ldk, int n_pad, int mode,
-          unsigned tmem_cols, int *err) {
+          int ntl, int natoms, double *__restrict__ K, long ldk, int n_pad, int mode, int *err) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2 * SK_S + 5];
+  __shared__ __align__(8) uint64_t bars[2 * SK_S + 2 * SK_SA + 3];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int my_tiles = (int)blockIdx.x < ntl ? (ntl - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   const int nchunk = (natoms + SK_CHUNK - 1) / SK_CHUNK;
   const int nc = (n_pad + SK_TN - 1) / SK_TN;
-  const uint32_t sbase = (su32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t bar0 = su32(&bars[0]);
+  const uint32_t sbase = (tc_su32(smem_raw) + 1023u) & ~1023u;
+  const uint8_t *gbase = smem_raw + (sbase - tc_su32(smem_raw));
+  const uint32_t bar0 = tc_su32(&bars[0]);
   auto full = [&](int st) { return bar0 + 8u * st; };
   auto empty = [&](int st) { return bar0 + 8u * (SK_S + st); };
-  auto tfull = [&](int bf) { return bar0 + 8u * (2 * SK_S + bf); };
-  auto tempty = [&](int bf) { return bar0 + 8u * (2 * SK_S + 2 + bf); };
-  const uint32_t drain = bar0 + 8u * (2 * SK_S + 4);
+  auto fullA = [&](int st) { return bar0 + 8u * (2 * SK_S + st); };
+  auto emptyA = [&](int st) { return bar0 + 8u * (2 * SK_S + SK_SA + st); };
+  const uint32_t tfull = bar0 + 8u * (2 * SK_S + 2 * SK_SA), tempty = tfull + 8u, drain = tfull + 16u;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                 ::"r"(su32(&tmem_slot)), "r"(tmem_cols) : "memory");
+                 ::"r"(tc_su32(&tmem_slot)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
     fail = 0;
     for (int st = 0; st < SK_S; ++st) {
-      mbar_init(full(st), 1);
-      mbar_init(empty(st), 1);
+      tc_mbar_init(full(st), 1);
+      tc_mbar_init(empty(st), 1 + SK_NMOV / 32);     // the MMAs and each moving warp
     }
-    for (int bf = 0; bf < 2; ++bf) {
-      mbar_init(tfull(bf), 1);
-      mbar_init(tempty(bf), SK_NEPI);
+    for (int st = 0; st < SK_SA; ++st) {
+      tc_mbar_init(fullA(st), SK_NMOV);
+      tc_mbar_init(emptyA(st), 1);
     }
-    mbar_init(drain, 1);
+    tc_mbar_init(tfull, 1);
+    tc_mbar_init(tempty, SK_NEPI);
+    tc_mbar_init(drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  tc_fence_before();
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tmem_slot;
+  tc_fence_after();
+  constexpr uint32_t tmem = 0;           // all 512 columns are allocated
+  constexpr uint32_t tmemA = tmem + SK_NACC * SK_TN;
   volatile int *vfail = &fail;
+  auto wait = [&](uint32_t bar, int parity) {      // by a whole warp
+    return __all_sync(0xffffffffu, tc_mbar_wait(bar, (unsigned)(parity & 1), vfail)) != 0;
+  };
 
-  if (warp == 0) {
+  if (warp < SK_NMOV / 32) {
+    // ---------------- A's slices from shared memory to TMEM: thread = row
+    const uint32_t lane_base = tmemA + ((uint32_t)(32 * warp) << 16);
+    int st = 0, use = 0, sa = 0, usea = 0;
+    bool ok = true;
+    for (int i = 0; i < my_tiles && ok; ++i) {
+      int2 t;
+      if (!tile_at(tl, (int)blockIdx.x + i * (int)gridDim.x, nc, t)) continue;
+      for (int a = 0; a < natoms && ok; ++a) {
+        if (!wait(full(st), use)) { ok = false; break; }
+        const uint8_t *src = gbase + (size_t)st * SK_STAGE;
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks) {
+          uint4 v[SK_NSL][2];
+#pragma unroll
+          for (int s = 0; s < SK_NSL; ++s)
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+              v[s][q] = *reinterpret_cast<const uint4 *>(src + s * SK_A_SLICE + tc_swz64(tid, 2 * ks + q));
+          if (ok && usea > 0 && !wait(emptyA(sa), usea - 1)) ok = false;
+          if (!ok) break;
+          tc_fence_after();
+#pragma unroll
+          for (int s = 0; s < SK_NSL; ++s)
+            tc_st8(lane_base + (uint32_t)(sa * SK_A_COLS + 8 * s), v[s][0], v[s][1]);
+          tc_wait_st();
+          tc_fence_before();
+          tc_mbar_arrive(fullA(sa));
+          if (++sa == SK_SA) { sa = 0; ++usea; }
+        }
+        __syncwarp();
+        if (lane == 0) tc_mbar_arrive(empty(st));
+        if (++st == SK_S) { st = 0; ++use; }
+      }
+    }
+    if (!ok && lane == 0) note(err, vfail, 34);
+  } else if (warp < (SK_NMOV + SK_NEPI) / 32) {
+    // ---------------- epilogue: exact level sums into int64, added to K at the end
+    constexpr int CW = SK_TN / 2;
+    const int lg = warp & 3, half = (warp - SK_NMOV / 32) >> 2;
+    const int r = 32 * lg + lane;
+    int use = 0;
+    bool ok = true;
+    for (int i = 0; i < my_tiles && ok; ++i) {
+      int2 t;
+      if (!tile_at(tl, (int)blockIdx.x + i * (int)gridDim.x, nc, t)) continue;
+      long long T[CW];
+      float F[CW];
+#pragma unroll
+      for (int j = 0; j < CW; ++j) { T[j] = 0; F[j] = 0.f; }
+      for (int c = 0; c < nchunk; ++c, ++use) {
+        if (!wait(tfull, use)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t trow = tmem + ((uint32_t)(32 * lg) << 16) + (uint32_t)(half * CW);
+#pragma unroll
+        for (int c0 = 0; c0 < CW; c0 += 2) {
+          uint32_t d[SK_NACC][2];
+#pragma unroll
+          for (int ac = 0; ac < SK_NACC; ++ac) tc_ld2(d[ac], trow + (uint32_t)(ac * SK_TN + c0));
+          tc_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            long long x = __float2int_rn(__uint_as_float(d[0][j]));
+#pragma unroll
+            for (int L = 1; L < 5; ++L)
+              x = x * 256 + __float2int_rn(__uint_as_float(d[L][j]) * tc_pow2f(8 * L));
+            T[c0 + j] += x;
+            F[c0 + j] += __uint_as_float(d[5][j]);
+          }
+        }
+        // the accumulators are read: the next chunk's MMAs may overwrite them
+        tc_fence_before();
+        tc_mbar_arrive(tempty);
+      }
+      if (!ok) break;
+      // a 64-column tile is one 64-block: one mask for the row
+      const long row = (long)t.x * SK_TM + r, col0 = (long)t.y * SK_TN + half * CW;
+      if (row < n_pad && (long)t.y <= (row >> 6)) {
+        const int ei = eg[row];
+        double2 *Kp = reinterpret_cast<double2 *>(K + row * ldk + col0);
+#pragma unroll
+        for (int q = 0; q < CW / 2; ++q) {
+          const double2 o = mode != 0 ? Kp[q] : make_double2(0.0, 0.0);
+          double v[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int j = 2 * q + h;
+            const double p = ldexp((double)T[j] * 0x1p-32 + (double)F[j], ei + eg[col0 + j] - 14);
+            const double old = h ? o.y : o.x;
+            v[h] = mode == 0 ? p : (mode == 1 ? old + p : old - p);
+          }
+          Kp[q] = make_double2(v[0], v[1]);
+        }
+      }
+    }
+    if (!ok && lane == 0) note(err, vfail, 33);
+  } else if (warp == (SK_NMOV + SK_NEPI) / 32) {
     if (lane == 0) {
       // ---------------- bulk copies: atom a of tile (I, J) into stage st
       int st = 0, use = 0, issued = 0;
@@ -370,172 +396,94 @@ k_syrk_sl(const uint8_t *__restrict__ Sl, const int *__restrict__ eg, const int2
         int2 t;
         if (!tile_at(tl, (int)blockIdx.x + i * (int)gridDim.x, nc, t)) continue;
         const uint8_t *Abase = Sl + (size_t)t.x * natoms * SK_A_STAGE;
-        const uint8_t *Bbase = Sl + (size_t)(t.y >> 2) * natoms * SK_A_STAGE + (size_t)(t.y & 3) * SK_B_SLICE;
+        const uint8_t *Bbase = Sl + (size_t)(t.y >> 1) * natoms * SK_A_STAGE + (size_t)(t.y & 1) * SK_B_SLICE;
         for (int a = 0; a < natoms; ++a) {
-          if (use > 0 && !mbar_wait(empty(st), (unsigned)((use - 1) & 1), vfail)) { ok = false; break; }
+          if (use > 0 && !tc_mbar_wait(empty(st), (unsigned)((use - 1) & 1), vfail)) { ok = false; break; }
           const uint32_t dst = sbase + (uint32_t)st * SK_STAGE;
-          mbar_arrive_tx(full(st), SK_STAGE);
-          bulk_g2s(dst, Abase + (size_t)a * SK_A_STAGE, SK_A_STAGE, full(st));
+          tc_mbar_arrive_tx(full(st), SK_STAGE);
+          tc_bulk_g2s(dst, Abase + (size_t)a * SK_A_STAGE, SK_A_STAGE, full(st));
 #pragma unroll
           for (int s = 0; s < SK_NSL; ++s)
-            bulk_g2s(dst + SK_A_STAGE + s * SK_B_SLICE, Bbase + (size_t)a * SK_A_STAGE + (size_t)s * SK_A_SLICE,
-                     SK_B_SLICE, full(st));
+            tc_bulk_g2s(dst + SK_A_STAGE + s * SK_B_SLICE, Bbase + (size_t)a * SK_A_STAGE + (size_t)s * SK_A_SLICE,
+                        SK_B_SLICE, full(st));
           ++issued;
           if (++st == SK_S) { st = 0; ++use; }
         }
       }
-      if (!ok) {
-        if (!*vfail && atomicCAS(err, 0, TW_ERR_TIMEOUT) == 0) err[1] = 31;
-        fail = 1;
-      }
+      if (!ok) note(err, vfail, 31);
       // copies already issued must land before the CTA's shared memory goes
-      if (*vfail)
-        for (int a = (issued > SK_S ? issued - SK_S : 0); a < issued; ++a)
-          mbar_drain(full(a % SK_S), (unsigned)((a / SK_S) & 1));
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer
-      const uint32_t idesc = idesc_bf16(SK_TM, SK_TN);
-      bool ok = true;
-      int st = 0, use = 0, g = 0;                     // stage, its use count, chunk count
-      for (int i = 0; i < my_tiles && ok; ++i) {
-        int2 t;
-        if (!tile_at(tl, (int)blockIdx.x + i * (int)gridDim.x, nc, t)) continue;
-        for (int c = 0; c < nchunk && ok; ++c, ++g) {
-          const int bf = g & 1;
-          // the epilogue has read this buffer's previous chunk
-          if (g >= 2 && !mbar_wait(tempty(bf), (unsigned)((g / 2 - 1) & 1), vfail)) { ok = false; break; }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t dbase = tmem + (uint32_t)(bf * SK_NACC * SK_TN);
-          const int a1 = min(natoms, (c + 1) * SK_CHUNK);
-          for (int a = c * SK_CHUNK; a < a1; ++a) {
-            if (!mbar_wait(full(st), (unsigned)(use & 1), vfail)) { ok = false; break; }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t aS = sbase + (uint32_t)st * SK_STAGE, bS = aS + SK_A_STAGE;
-#pragma unroll
-            for (int ks = 0; ks < SK_KA / 16; ++ks) {
-#pragma unroll
-              for (int p = 0; p < 28; ++p) {
-                int si, sj, L;
-                syrk_pair(p, si, sj, L);
-                const int ac = L < 5 ? L : 5;
-                // the first MMA of a chunk into each accumulator overwrites it
-                const bool lead = p == 0 || p == 1 || p == 3 || p == 6 || p == 10 || p == 15;
-                const uint32_t acc = (a > c * SK_CHUNK || ks > 0 || !lead) ? 1u : 0u;
-                mma_bf16(dbase + (uint32_t)(ac * SK_TN), sdesc64(aS + si * SK_A_SLICE + ks * 32),
-                         sdesc64(bS + sj * SK_B_SLICE + ks * 32), idesc, acc);
-              }
-            }
-            mma_commit(empty(st));                   // the stage is free once these finish
-            if (++st == SK_S) { st = 0; ++use; }
-          }
-          if (ok) mma_commit(tfull(bf));             // this chunk's sums are final
-        }
-      }
-      if (!ok && !*vfail && atomicCAS(err, 0, TW_ERR_TIMEOUT) == 0) err[1] = 32;
-      if (!ok) fail = 1;
-      // every issued MMA complete before TMEM is released
-      mma_commit(drain);
-      mbar_drain(drain, 0);
+      for (int a = (issued > SK_S ? issued - SK_S : 0); a < issued; ++a)
+        tc_mbar_wait(full(a % SK_S), (unsigned)((a / SK_S) & 1), nullptr);
     }
   } else {
-    // ---------------- epilogue: exact level sums into int64, added to K at the end
-    const int lg = warp & 3;
-    const int r = 32 * lg + lane;
-    int g = 0;
+    // ---------------- MMA issuer (the warp's lanes run together, one is elected to issue)
+    const uint32_t idesc = tc_idesc_bf16(SK_TM, SK_TN);
     bool ok = true;
+    int st = 0, use = 0, sa = 0, usea = 0, g = 0;       // stages, their use counts, chunk count
+    uint32_t dc[SK_NACC];
+#pragma unroll
+    for (int L = 0; L < SK_NACC; ++L) dc[L] = tmem + (uint32_t)(L * SK_TN);
     for (int i = 0; i < my_tiles && ok; ++i) {
       int2 t;
       if (!tile_at(tl, (int)blockIdx.x + i * (int)gridDim.x, nc, t)) continue;
-      long long T[SK_TN];
-      float F[SK_TN];
+      for (int c = 0; c < nchunk && ok; ++c, ++g) {
+        // the epilogue has read the previous chunk
+        if (g > 0 && !wait(tempty, g - 1)) { ok = false; break; }
+        tc_fence_after();
+        const int ns = 2 * (min(natoms, (c + 1) * SK_CHUNK) - c * SK_CHUNK);
+        if (!wait(full(st), use) || !wait(fullA(sa), usea)) { ok = false; break; }
+        // the next 16 k are waited for between the halves of this step's MMAs
+        for (int s = 0; s < ns; ++s) {
+          const int ks = s & 1;
+          tc_fence_after();
+          const uint32_t aT = tmemA + (uint32_t)(sa * SK_A_COLS);
+          const uint64_t bd0 = tc_sdesc64(sbase + (uint32_t)(st * SK_STAGE + SK_A_STAGE) + 32u * ks);
+          uint64_t bd[SK_NSL];
 #pragma unroll
-      for (int j = 0; j < SK_TN; ++j) { T[j] = 0; F[j] = 0.f; }
-      for (int c = 0; c < nchunk; ++c, ++g) {
-        const int bf = g & 1;
-        if (!mbar_wait(tfull(bf), (unsigned)((g / 2) & 1), vfail) || *vfail) {
-          if (!*vfail && atomicCAS(err, 0, TW_ERR_TIMEOUT) == 0) err[1] = 33;
-          fail = 1;
-          ok = false;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t trow = tmem + ((uint32_t)(32 * lg) << 16) + (uint32_t)(bf * SK_NACC * SK_TN);
-#pragma unroll
-        for (int c0 = 0; c0 < SK_TN; c0 += 8) {
-          uint32_t d[SK_NACC][8];
-#pragma unroll
-          for (int ac = 0; ac < SK_NACC; ++ac)
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                         : "=r"(d[ac][0]), "=r"(d[ac][1]), "=r"(d[ac][2]), "=r"(d[ac][3]), "=r"(d[ac][4]),
-                           "=r"(d[ac][5]), "=r"(d[ac][6]), "=r"(d[ac][7])
-                         : "r"(trow + (uint32_t)(ac * SK_TN + c0)));
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            long long x = __float2int_rn(__uint_as_float(d[0][j]));
-#pragma unroll
-            for (int L = 1; L < 5; ++L)
-              x = x * 256 + __float2int_rn(__uint_as_float(d[L][j]) * pow2f(8 * L));
-            T[c0 + j] += x;
-            F[c0 + j] += __uint_as_float(d[5][j]);
+          for (int j = 0; j < SK_NSL; ++j) bd[j] = bd0 + (uint64_t)(j * (SK_B_SLICE >> 4));
+          const bool last = s == ns - 1;
+          if (tc_elect()) tc_issue_half<0>(s == 0, dc, aT, bd, idesc);
+          __syncwarp();
+          const uint32_t eA = emptyA(sa), eS = empty(st);
+          if (++sa == SK_SA) { sa = 0; ++usea; }
+          if (ks == 1 && ++st == SK_S) { st = 0; ++use; }
+          if (!last && ((ks == 1 && !wait(full(st), use)) || !wait(fullA(sa), usea))) ok = false;
+          if (tc_elect()) {
+            tc_issue_half<1>(s == 0, dc, aT, bd, idesc);
+            tc_commit(eA);
+            if (ks == 1) tc_commit(eS);
+            if (last) tc_commit(tfull);
           }
-        }
-        // the buffer is read: a later chunk's MMAs may overwrite it
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        mbar_arrive(tempty(bf));
-      }
-      if (!ok) break;
-      // a 32-column tile lies inside one 64-block: one mask for the row
-      const long row = (long)t.x * SK_TM + r, col0 = (long)t.y * SK_TN;
-      if (row < n_pad && col0 < n_pad && (col0 >> 6) <= (row >> 6)) {
-        const int ei = eg[row];
-        double2 *Kp = reinterpret_cast<double2 *>(K + row * ldk + col0);
-        double old[SK_TN];
-        if (mode != 0) {
-#pragma unroll
-          for (int q = 0; q < SK_TN / 2; ++q) {
-            const double2 o = Kp[q];
-            old[2 * q] = o.x;
-            old[2 * q + 1] = o.y;
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < SK_TN / 2; ++q) {
-          double v[2];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int j = 2 * q + h;
-            const double p = ldexp((double)T[j] * 0x1p-32 + (double)F[j], ei + eg[col0 + j] - 14);
-            v[h] = mode == 0 ? p : (mode == 1 ? old[j] + p : old[j] - p);
-          }
-          Kp[q] = make_double2(v[0], v[1]);
+          __syncwarp();
+          if (!ok) break;
         }
       }
     }
+    if (!ok && lane == 0) note(err, vfail, 32);
+    // every issued MMA complete before TMEM is released
+    if (tc_elect()) tc_commit(drain);
+    tc_mbar_wait(drain, 0, nullptr);
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  tc_fence_before();
   __syncthreads();
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols)
-                 : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_slot), "r"(512u) : "memory");
 }
 
 }  // namespace
 
 // ------------------------------------------------------------------ host side
-// the lower 64-block triangle as (128-row tile, 32-column tile): groups of 8
+// the lower 64-block triangle as (128-row tile, 64-column tile): groups of 8
 // row tiles, column tile outer, row tile inner
 void syrk_tile_list(int n_pad, std::vector<int2> &tl) {
   const int nt = (n_pad + SK_TM - 1) / SK_TM, nc = (n_pad + SK_TN - 1) / SK_TN;
   tl.clear();
   for (int g0 = 0; g0 < nt; g0 += 8) {
     const int g1 = std::min(nt, g0 + 8);
-    const int jmax = std::min(nc - 1, 4 * (g1 - 1) + 3);
+    const int jmax = std::min(nc - 1, 2 * (g1 - 1) + 1);
     for (int J = 0; J <= jmax; ++J)
       for (int I = g0; I < g1; ++I)
-        if (J <= 4 * I + 3) tl.push_back(make_int2(I, J));
+        if (J <= 2 * I + 1) tl.push_back(make_int2(I, J));
   }
 }
 
@@ -568,7 +516,7 @@ cudaError_t launch_form_P_tc(const dd *G, long ldg, int n, int kdim, double *K, 
     const int na = std::min(per_panel, atoms_total - a0);
     k_syrk_slice<<<dim3((unsigned)na, (unsigned)nt), 256, 0, s>>>(G, ldg, n, kdim, a0 * SK_KA, eg, ws, na);
     count_launches(1);
-    k_syrk_sl<<<grid, SK_NTHR, sm, s>>>(ws, eg, tl, ntl, na, K, ldk, n_pad, a0 == 0 ? 0 : 1, 512u, err);
+    k_syrk_sl<<<grid, SK_NTHR, sm, s>>>(ws, eg, tl, ntl, na, K, ldk, n_pad, a0 == 0 ? 0 : 1, err);
     count_launches(1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -597,9 +545,9 @@ cudaError_t launch_syrk_update_d(const double *A, long lda, int kdim, double *C,
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const int ntl = 2 * nt * (nt + 1);                 // closed-form row-major order
+  const int ntl = nt * (nt + 1);                 // closed-form row-major order
   const unsigned grid = (unsigned)std::max(1, std::min(ntl, nsm));
-  k_syrk_sl<<<grid, SK_NTHR, sm, s>>>(ws, eg, nullptr, ntl, natoms, C, ldc, m, 2, 512u, err);
+  k_syrk_sl<<<grid, SK_NTHR, sm, s>>>(ws, eg, nullptr, ntl, natoms, C, ldc, m, 2, err);
   count_launches(1);
   return cudaGetLastError();
 }
