@@ -54,8 +54,11 @@
 // returns.
 #include <stdint.h>
 
+#include <utility>
+
 #include "../../include/tw.h"
 #include "kernels.h"
+#include "tc.cuh"
 
 namespace tw {
 
@@ -266,10 +269,21 @@ k_bsl_build(const cdd *__restrict__ Y, long y_bstride, int Nr, int B, int P, int
 // ------------------------------------------------------------------ the product
 // pair p = 0..9 of slices (i, j), level L = i + j: p = 0 is level 0 (into
 // D0), p = 1, 2 level 1 (into D1), p = 3..9 levels 2 and 3 (into D2)
-__device__ __forceinline__ int pair_level(int p) { return p == 0 ? 0 : (p < 3 ? 1 : (p < 6 ? 2 : 3)); }
-__device__ __forceinline__ int pair_i(int p) {
-  const int L = pair_level(p);
-  return p - L * (L + 1) / 2;
+__host__ __device__ constexpr int pair_level(int p) { return p == 0 ? 0 : (p < 3 ? 1 : (p < 6 ? 2 : 3)); }
+__host__ __device__ constexpr int pair_i(int p) { return p - pair_level(p) * (pair_level(p) + 1) / 2; }
+
+template <int PR>
+__device__ __forceinline__ void issue_pair(uint32_t d, uint32_t n, uint64_t a, uint64_t b, uint64_t b_step,
+                                           uint32_t idesc, bool acc) {
+  constexpr int L = pair_level(PR), si = pair_i(PR), sj = L - si, ac = L < 2 ? L : 2;
+  // the first MMA of a tile into each accumulator (pairs 0, 1, 3) overwrites it
+  mma_bf16(d + ac * n, a + (uint64_t)(si * (A_SLICE >> 4)), b + sj * b_step, idesc,
+           acc || !(PR == 0 || PR == 1 || PR == 3) ? 1u : 0u);
+}
+template <int... PR>
+__device__ __forceinline__ void issue_pairs(std::integer_sequence<int, PR...>, uint32_t d, uint32_t n, uint64_t a,
+                                            uint64_t b, uint64_t b_step, uint32_t idesc, bool acc) {
+  (issue_pair<PR>(d, n, a, b, b_step, idesc, acc), ...);
 }
 
 // raw-operator ring: RAW_D stages of 16 rows x 128 grid points (8 bytes per
@@ -316,7 +330,7 @@ k_gemm_adj_sl(const void *__restrict__ A, const int8_t *__restrict__ ea, const u
   __shared__ __align__(8) uint64_t bars[3 * MAXST + 5];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int N = 2 * P;
   const int nmt = (Nm + TM - 1) / TM;
   const int T = nmt * Nf * ntiles;
@@ -466,48 +480,53 @@ k_gemm_adj_sl(const void *__restrict__ A, const int8_t *__restrict__ ea, const u
         mbar_drain(fullB(a % S), (unsigned)((a / S) & 1));
     }
   } else if (warp == NPROD / 32) {
-    if (lane == 0) {
-      // ---------------- MMA issuer
-      const uint32_t idesc = idesc_bf16(TM, N);
-      bool ok = true;
-      int st = 0, use = 0;
-      for (int i = 0; i < my_tiles && ok; ++i) {
-        const int bf = i % nbuf;
-        // the epilogue has read this buffer's previous tile
-        if (i >= nbuf && !mbar_wait(tempty(bf), (unsigned)((i / nbuf - 1) & 1), vfail)) { ok = false; break; }
+    // ---------------- MMA issuer: the warp's lanes run together and one is
+    // elected to issue (from a branch of lane 0 an MMA takes 45 cycles whatever its
+    // width); the next stage is waited for between the halves of this one's MMAs
+    const uint32_t idesc = idesc_bf16(TM, N);
+    auto wait = [&](uint32_t bar, int parity) {
+      return __all_sync(0xffffffffu, mbar_wait(bar, (unsigned)(parity & 1), vfail)) != 0;
+    };
+    bool ok = true;
+    int st = 0, use = 0;
+    for (int i = 0; i < my_tiles && ok; ++i) {
+      const int bf = i % nbuf;
+      // the epilogue has read this buffer's previous tile
+      if (i >= nbuf && !wait(tempty(bf), i / nbuf - 1)) { ok = false; break; }
+      if (!wait(fullA(st), use) || !wait(fullB(st), use)) { ok = false; break; }
+      const uint32_t dbase = tmem + (uint32_t)(bf * 3 * N);
+      for (int a = 0; a < natoms; ++a) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t dbase = tmem + (uint32_t)(bf * 3 * N);
-        for (int a = 0; a < natoms; ++a) {
-          const unsigned par = (unsigned)(use & 1);
-          ok = mbar_wait(fullA(st), par, vfail) && mbar_wait(fullB(st), par, vfail);
-          if (!ok) break;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t aS = sA0 + st * A_STAGE, bS = sB0 + st * b_stage;
+        const uint64_t ad0 = sdesc64(sA0 + st * A_STAGE), bd0 = sdesc64(sB0 + st * b_stage);
+        const uint64_t b_step = b_slice >> 4;
+        const uint32_t est = empty(st);
+        const bool last = a == natoms - 1;
 #pragma unroll
-          for (int ks = 0; ks < KA / 16; ++ks) {
-#pragma unroll
-            for (int p = 0; p < 10; ++p) {
-              const int si = pair_i(p), sj = pair_level(p) - pair_i(p);
-              const uint64_t ad = sdesc64(aS + si * A_SLICE + ks * 32);
-              const uint64_t bd = sdesc64(bS + sj * b_slice + ks * 32);
-              const int L = pair_level(p);
-              const uint32_t dcol = (uint32_t)((L < 2 ? L : 2) * N);
-              // the first MMA of a tile into each accumulator (p = 0, 1, 3) overwrites it
-              const uint32_t acc = (a > 0 || ks > 0 || (p != 0 && p != 1 && p != 3)) ? 1u : 0u;
-              mma_bf16(dbase + dcol, ad, bd, idesc, acc);
-            }
+        for (int ks = 0; ks < KA / 16; ++ks) {
+          if (tc_elect())
+            issue_pairs(std::make_integer_sequence<int, 10>{}, dbase, (uint32_t)N, ad0 + 2u * ks, bd0 + 2u * ks,
+                        b_step, idesc, a > 0 || ks > 0);
+          __syncwarp();
+          if (ks == 0) {
+            if (++st == S) { st = 0; ++use; }
+            if (!last && (!wait(fullA(st), use) || !wait(fullB(st), use))) ok = false;
           }
-          mma_commit(empty(st));             // stage reusable once these MMAs finish
-          if (++st == S) { st = 0; ++use; }
         }
-        if (ok) mma_commit(tfull(bf));       // this tile's D final
+        if (tc_elect()) {
+          mma_commit(est);                   // stage reusable once these MMAs finish
+          if (last) mma_commit(tfull(bf));   // this tile's D final
+        }
+        __syncwarp();
+        if (!ok) break;
       }
-      if (!ok && !*vfail && atomicCAS(err, 0, TW_ERR_TIMEOUT) == 0) err[1] = 23;
-      if (!ok) fail = 1;
-      // every issued MMA complete before TMEM is released
-      mma_commit(drain);
-      mbar_drain(drain, 0);
     }
+    if (!ok && lane == 0) {
+      if (!*vfail && atomicCAS(err, 0, TW_ERR_TIMEOUT) == 0) err[1] = 23;
+      fail = 1;
+    }
+    // every issued MMA complete before TMEM is released
+    if (tc_elect()) mma_commit(drain);
+    mbar_drain(drain, 0);
   } else {
     // ---------------- epilogue: (D0 + D1) + D2 from TMEM, scaled, complex64 out
     const int lg = warp & 3;                          // TMEM lanes 32 lg .. 32 lg + 31
