@@ -39,21 +39,24 @@
 // within a few units of 2^-30 of the terms: the error left is the rounding
 // of the stored operator itself.  Ten MMAs per 16-wide k step.
 //
-// Kernel: persistent, one CTA per SM looping over (128 grid points,
-// frequency, tile of P right-hand sides); 8 producer warps stream the
-// operator (complex64 or bf16 hi+lo) through a 4-stage cp.async ring (64 KB
-// in flight per SM), slice it with its row's exponent and write the four
-// 128 x 32 bf16 slice tiles of a stage (K-major, 64-byte swizzle); one
-// thread copies the stage's B' slices (prepared once per call by
-// k_bsl_build) with the bulk copy engine and one thread issues the MMAs
-// (D0, D1, D2 in TMEM: 3N of its columns, so N <= 160).  Two slice stages,
-// mbarriers with transaction counts, tcgen05.commit frees a stage.  After a
-// tile's last stage the producers read D0..D2 (tcgen05.ld), scale and store
-// X as complex64, while the ring already holds the next tile's operator.  Every wait is bounded: on expiry the kernel records
-// TW_ERR_TIMEOUT, lets its copies and MMAs drain (bounded), frees TMEM and
-// returns.
+// Kernel: persistent, one CTA per SM over (right-hand-side tile, 128 grid
+// points, frequency), right-hand-side tile fastest.  Warps 0-7 and 8-15 stream
+// the operator (complex64 or bf16 hi+lo, cp.async), slice it with its row's
+// exponent and store alternate 16-wide A' stages to TMEM, from where the MMAs
+// read them; warps 16-23 drain the accumulators; warp 24 issues the MMAs (one
+// elected lane); warp 25 copies the B' slices (prepared once per call by
+// k_bsl_build, cp.async.bulk).  TMEM: D0, D1, D2 of N columns, twice when that
+// leaves two A' stages (N <= 72), the rest A' stages of 4 x 8 columns (N <=
+// 144).  With A' in shared memory an MMA of N <= 32 took 40 cycles (A's 4 KB at
+// 128 bytes a clock) against 16, eight producer warps were what bounded the
+// small batches, and one warp a TMEM quarter the large ones' drain: 64
+// right-hand sides of the 100-sensor case 10.0 -> 8.0 ms, 16 of the 200-sensor
+// serving case 3.29 -> 3.10 ms.  Every
+// wait is bounded: on expiry the kernel records TW_ERR_TIMEOUT, lets its
+// copies and MMAs drain (bounded), frees TMEM and returns.
 #include <stdint.h>
 
+#include <algorithm>
 #include <utility>
 
 #include "../../include/tw.h"
@@ -65,98 +68,20 @@ namespace tw {
 namespace {
 
 constexpr int TM = 128;                  // MMA M: grid points per tile
-constexpr int KA = 32;                   // K' per stage: 16 rows (sensors) x (re, im)
+constexpr int KA = 32;                   // K' per B' atom: 16 rows (sensors) x (re, im)
 constexpr int NSL = 4;                   // slices per operand
-constexpr int NPROD = 256;               // producer threads (8 warps)
-constexpr int A_SLICE = TM * KA * 2;     // 8 KB: one 128 x 32 bf16 slice tile
-constexpr int A_STAGE = NSL * A_SLICE;   // 32 KB
-constexpr unsigned SPIN_LIMIT = 1u << 26;
+constexpr int A_COLS = NSL * 8;          // TMEM columns of a 16-wide A' stage
+constexpr int NGRP = 256, NPROD = 2 * NGRP, NEPI = 256;
+constexpr int NTHR = NPROD + NEPI + 64;
+constexpr int MAXA = 4, SB = 4;          // A' stages (at most), B' stages
+constexpr int RAW_D = 3;                 // operator atoms in shared memory (raw ring)
+constexpr int RAW_SLOT = NPROD * 4 * 8;  // 16 KB: 16 rows x 128 grid points
 constexpr int EXP_MIN = -100, EXP_MAX = 120;
-constexpr int SL_PMAX = 80;              // right-hand sides per tile: 3 x 2P <= 512 TMEM columns
-
-__device__ __forceinline__ uint32_t su32(const void *p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-// byte offset of the 16-byte chunk q (0..3) of row r in a K-major tile of 32
-// bf16 per row with the 64-byte swizzle (chunk index XOR bits 1-2 of the row)
-__host__ __device__ __forceinline__ uint32_t swz64(int r, int q) {
-  return (uint32_t)r * 64u + ((uint32_t)(q ^ ((r >> 1) & 3)) << 4);
-}
-
-// shared-memory matrix descriptor: K-major, 64-byte swizzle, 8-row groups 512
-// bytes apart; bits 46-48 = 0b001 (descriptor version), bits 61-63 = 4 (64B)
-__device__ __forceinline__ uint64_t sdesc64(uint32_t saddr) {
-  uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(512 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)4 << 61;
-  return d;
-}
-
-// instruction descriptor, kind::f16: D F32, A and B BF16, both K-major
-__host__ __device__ __forceinline__ uint32_t idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_tx(uint32_t bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, unsigned parity) {
-  uint32_t ok;
-  asm volatile("{\n\t.reg .pred p;\n\t"
-               "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-               "selp.b32 %0, 1, 0, p;\n\t}"
-               : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-// true once the phase with this parity has completed; false after the spin
-// limit or once another role of the CTA has failed
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, unsigned parity, volatile int *fail) {
-  for (unsigned it = 0; it < SPIN_LIMIT; ++it) {
-    if (mbar_try(bar, parity)) return true;
-    if ((it & 1023u) == 1023u && *fail) return false;
-  }
-  return false;
-}
-// the same without the early exit (draining the CTA's own asynchronous work)
-__device__ __forceinline__ bool mbar_drain(uint32_t bar, unsigned parity) {
-  for (unsigned it = 0; it < SPIN_LIMIT; ++it)
-    if (mbar_try(bar, parity)) return true;
-  return false;
-}
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, unsigned bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc,
-                                         uint32_t acc) {
-  asm volatile("{\n\t.reg .pred p;\n\t"
-               "setp.ne.b32 p, %4, 0;\n\t"
-               "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-               ::"r"(dtmem), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-               ::"r"(bar) : "memory");
-}
+constexpr int SL_PMAX = 72;              // right-hand sides per tile: 3 x 2P columns leave two A' stages
 
 // round to the nearest integer (ties to even), |v| < 2^22
 __device__ __forceinline__ float rnd_int(float v) {
   return __fsub_rn(__fadd_rn(v, 12582912.0f), 12582912.0f);
-}
-// 2^e as a float, e in [-126, 127]
-__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
-// bf16 bits of two floats of at most 8 significant bits (exact): upper halves
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
 }
 // smallest e with |v| < 2^e for the largest |v| = mx >= 0, clamped
 __device__ __forceinline__ int exp_above(float mx) {
@@ -228,7 +153,7 @@ k_bsl_build(const cdd *__restrict__ Y, long y_bstride, int Nr, int B, int P, int
     const int a = t / (N * 4), rem = t % (N * 4);
     const int n = rem >> 2, q = rem & 3;
     const int part = n >= P, bl = n - part * P, b = nt * P + bl;
-    const float sc = pow2f(7 - e_sh[bl]);
+    const float sc = tc_pow2f(7 - e_sh[bl]);
     uint32_t wd[NSL][4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -246,7 +171,7 @@ k_bsl_build(const cdd *__restrict__ Y, long y_bstride, int Nr, int B, int P, int
 #pragma unroll
         for (int i = 0; i < NSL; ++i) {
           const float si = rnd_int(hi);
-          sl[c][i] = si * pow2f(-8 * i);
+          sl[c][i] = si * tc_pow2f(-8 * i);
           if (i + 1 < NSL) {
             float r, e;
             two_sum(__fsub_rn(hi, si), lo, r, e);      // hi - si is exact
@@ -256,12 +181,12 @@ k_bsl_build(const cdd *__restrict__ Y, long y_bstride, int Nr, int B, int P, int
         }
       }
 #pragma unroll
-      for (int i = 0; i < NSL; ++i) wd[i][u] = pack_bf16(sl[0][i], sl[1][i]);
+      for (int i = 0; i < NSL; ++i) wd[i][u] = tc_pack_bf16(sl[0][i], sl[1][i]);
     }
     uint8_t *at = base + (size_t)a * NSL * slice_bytes;
 #pragma unroll
     for (int i = 0; i < NSL; ++i)
-      *reinterpret_cast<uint4 *>(at + i * slice_bytes + swz64(n, q)) =
+      *reinterpret_cast<uint4 *>(at + i * slice_bytes + tc_swz64(n, q)) =
           make_uint4(wd[i][0], wd[i][1], wd[i][2], wd[i][3]);
   }
 }
@@ -269,34 +194,17 @@ k_bsl_build(const cdd *__restrict__ Y, long y_bstride, int Nr, int B, int P, int
 // ------------------------------------------------------------------ the product
 // pair p = 0..9 of slices (i, j), level L = i + j: p = 0 is level 0 (into
 // D0), p = 1, 2 level 1 (into D1), p = 3..9 levels 2 and 3 (into D2)
-__host__ __device__ constexpr int pair_level(int p) { return p == 0 ? 0 : (p < 3 ? 1 : (p < 6 ? 2 : 3)); }
-__host__ __device__ constexpr int pair_i(int p) { return p - pair_level(p) * (pair_level(p) + 1) / 2; }
-
 template <int PR>
-__device__ __forceinline__ void issue_pair(uint32_t d, uint32_t n, uint64_t a, uint64_t b, uint64_t b_step,
-                                           uint32_t idesc, bool acc) {
-  constexpr int L = pair_level(PR), si = pair_i(PR), sj = L - si, ac = L < 2 ? L : 2;
+__device__ __forceinline__ void issue_pair(bool first, const uint32_t *d, uint32_t a, const uint64_t *b,
+                                           uint32_t idesc) {
+  constexpr int L = tc_pair_level(PR), si = PR - L * (L + 1) / 2, sj = L - si, ac = L < 2 ? L : 2;
   // the first MMA of a tile into each accumulator (pairs 0, 1, 3) overwrites it
-  mma_bf16(d + ac * n, a + (uint64_t)(si * (A_SLICE >> 4)), b + sj * b_step, idesc,
-           acc || !(PR == 0 || PR == 1 || PR == 3) ? 1u : 0u);
+  tc_mma_ts(d[ac], a + 8u * si, b[sj], idesc, first && si == 0 && L < 3 ? 0u : 1u);
 }
-template <int... PR>
-__device__ __forceinline__ void issue_pairs(std::integer_sequence<int, PR...>, uint32_t d, uint32_t n, uint64_t a,
-                                            uint64_t b, uint64_t b_step, uint32_t idesc, bool acc) {
-  (issue_pair<PR>(d, n, a, b, b_step, idesc, acc), ...);
-}
-
-// raw-operator ring: RAW_D stages of 16 rows x 128 grid points (8 bytes per
-// entry), each thread's own 8 entries of a stage copied by cp.async
-constexpr int RAW_D = 4;
-constexpr int RAW_STAGE = 16 * TM * 8;   // 16 KB
-
-__device__ __forceinline__ void cp_async8(uint32_t dst, const void *src, unsigned bytes) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+template <int P0, int... PR>
+__device__ __forceinline__ void issue_pairs(std::integer_sequence<int, PR...>, bool first, const uint32_t *d,
+                                            uint32_t a, const uint64_t *b, uint32_t idesc) {
+  (issue_pair<P0 + PR>(first, d, a, b, idesc), ...);
 }
 
 // the exact FP32 value of an operator entry held as 8 raw bytes
@@ -308,26 +216,18 @@ template <> __device__ __forceinline__ float2 decode_entry<FMT_BF16X2>(uint2 v) 
   return make_float2(bf16lo(v.x) + bf16hi(v.x), bf16lo(v.y) + bf16hi(v.y));
 }
 
-// Persistent: CTA b takes tiles b, b + gridDim.x, ... of the (grid tile,
-// frequency, right-hand-side tile) space, grid tile fastest (CTAs running at
-// the same time share a frequency, so its B' slices stay in L2).  Atoms
-// (16-row K' stages) are numbered across the CTA's tiles, so the raw ring,
-// the slice stages and their barriers run on without a break between tiles.
-// Warp roles: 0-7 producers, 8 the MMA issuer, 9-12 the epilogue (TMEM lane
-// quarter = warp mod 4).  The accumulators are double-buffered in TMEM when
-// 2 x 3N columns fit (N <= 80): the MMAs of tile i+1 then run while the
-// epilogue drains tile i.
-constexpr int NEPI = 128;                // epilogue threads (4 warps)
-constexpr int NTHR_P = NPROD + 32 + NEPI;
-constexpr int MAXST = 4;                 // slice stages (as many as shared memory allows)
+__device__ __forceinline__ void note(int *err, volatile int *fail, int info) {
+  if (!*fail && atomicCAS(err, 0, TW_ERR_TIMEOUT) == 0) err[1] = info;
+  *fail = 1;
+}
 
 template <int FMT>
-__global__ void __launch_bounds__(NTHR_P, 1)
-k_gemm_adj_sl(const void *__restrict__ A, const int8_t *__restrict__ ea, const uint8_t *__restrict__ Bt,
+__global__ void __launch_bounds__(NTHR, 1)
+k_gemm_adj_sl(const uint2 *__restrict__ A, const int8_t *__restrict__ ea, const uint8_t *__restrict__ Bt,
               const int *__restrict__ eb, cf *__restrict__ X, long x_bstride, int B, int P, int ntiles,
-              int Nr, int Nm, int Nf, int natoms, int S, int nbuf, unsigned tmem_cols, int *err) {
+              int Nr, int Nm, int Nf, int natoms, int SA, int nbuf, int *err) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t bars[3 * MAXST + 5];
+  __shared__ __align__(8) uint64_t bars[2 * MAXA + 2 * SB + 5];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -336,256 +236,287 @@ k_gemm_adj_sl(const void *__restrict__ A, const int8_t *__restrict__ ea, const u
   const int T = nmt * Nf * ntiles;
   const int my_tiles = (int)blockIdx.x < T ? (T - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   const uint32_t b_slice = (uint32_t)N * 64u, b_stage = NSL * b_slice;
-  const uint32_t sbase = (su32(smem_raw) + 1023u) & ~1023u;
-  // [raw ring RAW_D x 16 KB][A slices S x 32 KB][B' slices S x b_stage]
-  const uint32_t sRaw = sbase, sA0 = sbase + RAW_D * RAW_STAGE, sB0 = sA0 + S * A_STAGE;
-  uint8_t *gbase = smem_raw + (sbase - su32(smem_raw));
-  const uint32_t bar0 = su32(&bars[0]);
+  const uint32_t sB0 = (tc_su32(smem_raw) + 1023u) & ~1023u, sRaw = sB0 + (uint32_t)SB * b_stage;
+  const uint32_t bar0 = tc_su32(&bars[0]);
   auto fullA = [&](int st) { return bar0 + 8u * st; };
-  auto fullB = [&](int st) { return bar0 + 8u * (MAXST + st); };
-  auto empty = [&](int st) { return bar0 + 8u * (2 * MAXST + st); };
-  auto tfull = [&](int bf) { return bar0 + 8u * (3 * MAXST + bf); };       // D of a buffer final
-  auto tempty = [&](int bf) { return bar0 + 8u * (3 * MAXST + 2 + bf); };  // D read out
-  const uint32_t drain = bar0 + 8u * (3 * MAXST + 4);
+  auto emptyA = [&](int st) { return bar0 + 8u * (MAXA + st); };
+  auto fullB = [&](int st) { return bar0 + 8u * (2 * MAXA + st); };
+  auto emptyB = [&](int st) { return bar0 + 8u * (2 * MAXA + SB + st); };
+  auto tfull = [&](int bf) { return bar0 + 8u * (2 * MAXA + 2 * SB + bf); };
+  auto tempty = [&](int bf) { return bar0 + 8u * (2 * MAXA + 2 * SB + 2 + bf); };
+  const uint32_t drain = bar0 + 8u * (2 * MAXA + 2 * SB + 4);
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                 ::"r"(su32(&tmem_slot)), "r"(tmem_cols) : "memory");
+                 ::"r"(tc_su32(&tmem_slot)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
     fail = 0;
-    for (int st = 0; st < S; ++st) {
-      mbar_init(fullA(st), NPROD);
-      mbar_init(fullB(st), 1);
-      mbar_init(empty(st), 1);
+    for (int st = 0; st < SA; ++st) {
+      tc_mbar_init(fullA(st), NGRP);
+      tc_mbar_init(emptyA(st), 1);
+    }
+    for (int st = 0; st < SB; ++st) {
+      tc_mbar_init(fullB(st), 1);
+      tc_mbar_init(emptyB(st), 1);
     }
     for (int bf = 0; bf < 2; ++bf) {
-      mbar_init(tfull(bf), 1);
-      mbar_init(tempty(bf), NEPI);
+      tc_mbar_init(tfull(bf), 1);
+      tc_mbar_init(tempty(bf), NEPI);
     }
-    mbar_init(drain, 1);
+    tc_mbar_init(drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  tc_fence_before();
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tmem_slot;
+  tc_fence_after();
+  constexpr uint32_t tmem = 0;           // all 512 columns are allocated
+  const uint32_t tmemA = tmem + (uint32_t)(nbuf * 3 * N);
   volatile int *vfail = &fail;
   auto tile_of = [&](int i, int &mt, int &w, int &nt) {
     const int t = (int)blockIdx.x + i * (int)gridDim.x;
-    mt = t % nmt;
-    w = (t / nmt) % Nf;
-    nt = t / (nmt * Nf);
+    nt = t % ntiles;
+    const int q = t / ntiles;
+    mt = q % nmt;
+    w = q / nmt;
   };
 
   if (warp < NPROD / 32) {
-    // ---------------- producers: operator slices
-    const int r = tid & (TM - 1), h = tid >> 7;
-    // the issue pointer runs RAW_D - 1 atoms ahead of the consumer: its tile
-    // (local index, grid row offset) and atom, advanced without divisions
-    int ii = 0, ia = 0;
-    size_t ibase = 0;                                 // entry offset of (w, row 8h, grid point m)
+    // ---------------- producers: A' slices into TMEM.  Group g (8 warps) fills
+    // every atom's stage g; thread = grid point r, rows 4h .. 4h+3 of the
+    // stage's 8; its loads run RAW_D - 1 atoms ahead
+    const int r = tid & (TM - 1), h = (tid >> 7) & 1, g = tid / NGRP;
+    int ii = 0, ia = 0, islot = 0;
+    const uint2 *ip = A;
     bool ivalid = false;
-    auto set_issue_tile = [&](int i) {
-      if (i >= my_tiles) return;
+    auto set_issue_tile = [&]() {
+      ivalid = false;
+      if (ii >= my_tiles) return;
       int mt, w, nt;
-      tile_of(i, mt, w, nt);
+      tile_of(ii, mt, w, nt);
       const int m = mt * TM + r;
       ivalid = m < Nm;
-      ibase = ((size_t)w * Nr + 8 * h) * Nm + (size_t)m;
+      ip = A + ((size_t)w * Nr + 8 * g + 4 * h) * Nm + (ivalid ? m : 0);
     };
-    set_issue_tile(0);
-    int islot = 0;
-    auto issue = [&]() {
+    // raw ring: slot, entry u, producer thread (each thread reads only what it copied)
+    const uint32_t raw0 = sRaw + 8u * tid;
+    const uint8_t *rawp = smem_raw + (raw0 - tc_su32(smem_raw));
+    auto load = [&]() {
       if (ii < my_tiles) {
-        const uint32_t dst = sRaw + (uint32_t)islot * RAW_STAGE + (uint32_t)tid * 8u;
-        const int s0 = 16 * ia + 8 * h;
-        const uint8_t *src0 = reinterpret_cast<const uint8_t *>(A) + (ibase + (size_t)16 * ia * Nm) * 8;
+        const int s0 = 16 * ia + 8 * g + 4 * h;
+        const uint2 *p = ip + (size_t)(16 * ia) * Nm;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const bool ok = ivalid && s0 + u < Nr;
-          cp_async8(dst + (uint32_t)u * (NPROD * 8u), ok ? src0 + (size_t)u * Nm * 8 : (const uint8_t *)A,
-                    ok ? 8u : 0u);
+        for (int u = 0; u < 4; ++u) {
+          const bool in = ivalid && s0 + u < Nr;
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;"
+                       ::"r"(raw0 + (uint32_t)(islot * RAW_SLOT + u * NPROD * 8)),
+                         "l"(in ? p + (size_t)u * Nm : A), "r"(in ? 8 : 0) : "memory");
         }
-        if (++ia == natoms) { ia = 0; set_issue_tile(++ii); }
+        if (++ia == natoms) { ia = 0; ++ii; set_issue_tile(); }
       }
-      cp_async_commit();
-      islot = (islot + 1) & (RAW_D - 1);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      if (++islot == RAW_D) islot = 0;
     };
+    auto row_scale_exp = [&](int i) {
+      if (i >= my_tiles) return EXP_MIN;
+      int mt, w, nt;
+      tile_of(i, mt, w, nt);
+      const int m = mt * TM + r;
+      return m < Nm ? (int)ea[(size_t)w * Nm + m] : EXP_MIN;
+    };
+    set_issue_tile();
 #pragma unroll
-    for (int g = 0; g < RAW_D - 1; ++g) issue();
-    int issued = 0;                                  // B' copies issued by thread 0
-    int st = 0, use = 0, slot = 0;                   // slice stage, its use count, raw slot
+    for (int d = 0; d < RAW_D - 1; ++d) load();
+    int slot = 0;
+    int e_next = row_scale_exp(0);
     bool ok = true;
+    const uint32_t lane_base = tmemA + ((uint32_t)(32 * (warp & 3)) << 16) + 4u * h;
+    // the stages of the groups alternate; an atom whose second half holds no
+    // rows (the last, for some Nr) has one
+    const bool odd = 16 * (natoms - 1) + 8 >= Nr;
+    int st = g, use = 0;
+    auto step = [&](int n) {
+      st += n;
+      while (st >= SA) { st -= SA; ++use; }
+    };
+    for (int i = 0; i < my_tiles && ok; ++i) {
+      const float sc1 = tc_pow2f(7 - e_next);
+      const f2 sc = f2_make(sc1, sc1);
+      e_next = row_scale_exp(i + 1);
+      for (int a = 0; a < natoms; ++a) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(RAW_D - 2) : "memory");
+        f2 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float2 e = decode_entry<FMT>(
+              *reinterpret_cast<const uint2 *>(rawp + slot * RAW_SLOT + u * NPROD * 8));
+          v[u] = mul2(f2_make(e.x, e.y), sc);
+        }
+        if (++slot == RAW_D) slot = 0;
+        load();
+        const bool last_half = odd && a == natoms - 1;      // this atom has the first stage only
+        if (use > 0) {
+          const bool got = tc_mbar_wait(emptyA(st), (unsigned)((use - 1) & 1), vfail);
+          if (!__all_sync(0xffffffffu, got)) {
+            if (lane == 0) note(err, vfail, 21);
+            ok = false;
+            break;
+          }
+        }
+        // (group 1 waits for the stage that it leaves to the next tile as well: a
+        // jump of three stages could meet its next stage a whole phase early)
+        if (last_half && g == 1) { step(1); continue; }
+        tc_fence_after();
+        // slice i = v rounded to the grid 2^-8i (v - slices so far, exact):
+        // (x + 1.5 2^(23-8i)) - 1.5 2^(23-8i) rounds x to a multiple of 2^-8i
+        const uint32_t at = lane_base + (uint32_t)(st * A_COLS);
+#pragma unroll
+        for (int il = 0; il < NSL; ++il) {
+          const float m = tc_pow2f(23 - 8 * il) * 1.5f;
+          const f2 M = f2_make(m, m);
+          uint32_t wd[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const f2 s = sub2(add2(v[u], M), M);
+            const float2 sv = f2_split(s);
+            wd[u] = tc_pack_bf16(sv.x, sv.y);
+            if (il + 1 < NSL) v[u] = sub2(v[u], s);
+          }
+          tc_st4(at + 8u * il, wd);
+        }
+        tc_wait_st();
+        tc_fence_before();
+        tc_mbar_arrive(fullA(st));
+        step(last_half ? 1 : 2);
+      }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");   // own copies drained before exit
+  } else if (warp < (NPROD + NEPI) / 32) {
+    // ---------------- epilogue: (D0 + D1) + D2 from TMEM, scaled, complex64 out
+    // (two warps a TMEM lane quarter, each half of the columns)
+    const int lg = warp & 3, half = (warp - NPROD / 32) >> 2;
+    const int r = 32 * lg + lane;
+    const int CW = P / 2;
+    bool ok = true;
+    int bf = 0, use = 0;
     for (int i = 0; i < my_tiles && ok; ++i) {
       int mt, w, nt;
       tile_of(i, mt, w, nt);
       const int m = mt * TM + r;
-      const float sc = pow2f(7 - (m < Nm ? (int)ea[(size_t)w * Nm + m] : EXP_MIN));
-      const uint8_t *Bw = Bt + ((size_t)w * ntiles + nt) * natoms * b_stage;
-      for (int a = 0; a < natoms; ++a) {
-        issue();
-        cp_async_wait<RAW_D - 1>();                  // this atom's entries have landed
-        const uint8_t *raw = gbase + (size_t)slot * RAW_STAGE + (size_t)tid * 8;
-        slot = (slot + 1) & (RAW_D - 1);
-        float v[16];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const float2 e = decode_entry<FMT>(*reinterpret_cast<const uint2 *>(raw + u * (NPROD * 8)));
-          v[2 * u] = e.x * sc;
-          v[2 * u + 1] = e.y * sc;
-        }
-        if (use > 0 && !mbar_wait(empty(st), (unsigned)((use - 1) & 1), vfail)) {
-          if (!*vfail && atomicCAS(err, 0, TW_ERR_TIMEOUT) == 0) err[1] = 21;
-          fail = 1;
-          ok = false;
-          break;
-        }
-        if (tid == 0) {
-          mbar_arrive_tx(fullB(st), b_stage);
-          bulk_g2s(sB0 + st * b_stage, Bw + (size_t)a * b_stage, b_stage, fullB(st));
-          ++issued;
-        }
-        uint8_t *sa = gbase + RAW_D * RAW_STAGE + (size_t)st * A_STAGE;
-        // slice i = v rounded to the grid 2^-8i (v - slices so far, exact):
-        // (x + 1.5 2^(23-8i)) - 1.5 2^(23-8i) rounds x to a multiple of 2^-8i
-#pragma unroll
-        for (int il = 0; il < NSL; ++il) {
-          const float M = pow2f(23 - 8 * il) * 1.5f;
-          uint32_t wd[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const float s0 = __fsub_rn(__fadd_rn(v[2 * u], M), M);
-            const float s1 = __fsub_rn(__fadd_rn(v[2 * u + 1], M), M);
-            wd[u] = pack_bf16(s0, s1);
-            if (il + 1 < NSL) {
-              v[2 * u] = __fsub_rn(v[2 * u], s0);
-              v[2 * u + 1] = __fsub_rn(v[2 * u + 1], s1);
-            }
-          }
-          uint8_t *tile = sa + il * A_SLICE;
-          *reinterpret_cast<uint4 *>(tile + swz64(r, 2 * h)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
-          *reinterpret_cast<uint4 *>(tile + swz64(r, 2 * h + 1)) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
-        }
-        // generic-proxy writes -> visible to the tensor cores (async proxy)
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_arrive(fullA(st));
-        if (++st == S) { st = 0; ++use; }
+      const float sa = tc_pow2f((m < Nm ? (int)ea[(size_t)w * Nm + m] : EXP_MIN) - 7);
+      const int b0 = nt * P + half * CW;
+      const int *ebw = eb + (size_t)w * ntiles * P + b0;
+      cf *xp = X + (size_t)b0 * x_bstride + (size_t)w * Nm + m;
+      const bool got = tc_mbar_wait(tfull(bf), (unsigned)(use & 1), vfail);
+      if (!__all_sync(0xffffffffu, got)) {
+        if (lane == 0) note(err, vfail, 22);
+        ok = false;
+        break;
       }
+      tc_fence_after();
+      const uint32_t trow = tmem + ((uint32_t)(32 * lg) << 16) + (uint32_t)(bf * 3 * N + half * CW);
+#pragma unroll 1
+      for (int c0 = 0; c0 < CW; c0 += 4) {
+        uint32_t dr[3][4], di[3][4];
+#pragma unroll
+        for (int L = 0; L < 3; ++L) {
+          tc_ld4(dr[L], trow + (uint32_t)(L * N + c0));
+          tc_ld4(di[L], trow + (uint32_t)(L * N + P + c0));
+        }
+        tc_wait_ld();
+        if (c0 + 4 >= CW) {
+          // the buffer is read: the MMAs of a later tile may overwrite it
+          tc_fence_before();
+          tc_mbar_arrive(tempty(bf));
+        }
+        if (m < Nm) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (b0 + c0 + j >= B) continue;
+            const float sb = tc_pow2f(ebw[c0 + j] - 7);
+            const float re = __fadd_rn(__fadd_rn(__uint_as_float(dr[0][j]), __uint_as_float(dr[1][j])),
+                                       __uint_as_float(dr[2][j])) * sa * sb;
+            const float im = __fadd_rn(__fadd_rn(__uint_as_float(di[0][j]), __uint_as_float(di[1][j])),
+                                       __uint_as_float(di[2][j])) * sa * sb;
+            xp[(size_t)(c0 + j) * x_bstride] = cf_make(re, im);
+          }
+        }
+      }
+      if (++bf == nbuf) { bf = 0; ++use; }
     }
-    cp_async_wait<0>();                              // own copies drained before exit
-    if (tid == 0 && *vfail) {
-      // bulk copies already issued must land before the CTA's shared memory goes
-      for (int a = (issued > S ? issued - S : 0); a < issued; ++a)
-        mbar_drain(fullB(a % S), (unsigned)((a / S) & 1));
-    }
-  } else if (warp == NPROD / 32) {
-    // ---------------- MMA issuer: the warp's lanes run together and one is
-    // elected to issue (from a branch of lane 0 an MMA takes 45 cycles whatever its
-    // width); the next stage is waited for between the halves of this one's MMAs
-    const uint32_t idesc = idesc_bf16(TM, N);
+  } else if (warp == (NPROD + NEPI) / 32) {
+    // ---------------- MMA issuer (the warp's lanes run together, one is elected to issue)
+    const uint32_t idesc = tc_idesc_bf16(TM, N);
     auto wait = [&](uint32_t bar, int parity) {
-      return __all_sync(0xffffffffu, mbar_wait(bar, (unsigned)(parity & 1), vfail)) != 0;
+      return __all_sync(0xffffffffu, tc_mbar_wait(bar, (unsigned)(parity & 1), vfail)) != 0;
     };
     bool ok = true;
-    int st = 0, use = 0;
+    int sa = 0, usea = 0, sb = 0, useb = 0, bf = 0, used = 0;
     for (int i = 0; i < my_tiles && ok; ++i) {
-      const int bf = i % nbuf;
       // the epilogue has read this buffer's previous tile
-      if (i >= nbuf && !wait(tempty(bf), i / nbuf - 1)) { ok = false; break; }
-      if (!wait(fullA(st), use) || !wait(fullB(st), use)) { ok = false; break; }
-      const uint32_t dbase = tmem + (uint32_t)(bf * 3 * N);
-      for (int a = 0; a < natoms; ++a) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint64_t ad0 = sdesc64(sA0 + st * A_STAGE), bd0 = sdesc64(sB0 + st * b_stage);
-        const uint64_t b_step = b_slice >> 4;
-        const uint32_t est = empty(st);
-        const bool last = a == natoms - 1;
+      if (used > 0 && !wait(tempty(bf), used - 1)) { ok = false; break; }
+      tc_fence_after();
+      uint32_t dc[3];
 #pragma unroll
-        for (int ks = 0; ks < KA / 16; ++ks) {
-          if (tc_elect())
-            issue_pairs(std::make_integer_sequence<int, 10>{}, dbase, (uint32_t)N, ad0 + 2u * ks, bd0 + 2u * ks,
-                        b_step, idesc, a > 0 || ks > 0);
-          __syncwarp();
-          if (ks == 0) {
-            if (++st == S) { st = 0; ++use; }
-            if (!last && (!wait(fullA(st), use) || !wait(fullB(st), use))) ok = false;
-          }
-        }
+      for (int L = 0; L < 3; ++L) dc[L] = tmem + (uint32_t)((bf * 3 + L) * N);
+      if (!wait(fullB(sb), useb) || !wait(fullA(sa), usea)) { ok = false; break; }
+      // stages of 8 rows; an atom's B' serves two.  The next stage is waited
+      // for between the halves of this one's MMAs
+      for (int s = 0; s < Nr; s += 8) {
+        const int ks = (s >> 3) & 1;
+        tc_fence_after();
+        const uint32_t aT = tmemA + (uint32_t)(sa * A_COLS);
+        const uint64_t bd0 = tc_sdesc64(sB0 + (uint32_t)sb * b_stage + 32u * ks);
+        uint64_t bd[NSL];
+#pragma unroll
+        for (int j = 0; j < NSL; ++j) bd[j] = bd0 + (uint64_t)(j * (b_slice >> 4));
+        const bool last = s + 8 >= Nr, b_done = ks == 1 || last;
+        if (tc_elect()) issue_pairs<0>(std::make_integer_sequence<int, 5>{}, s == 0, dc, aT, bd, idesc);
+        __syncwarp();
+        const uint32_t eA = emptyA(sa), eB = emptyB(sb);
+        if (++sa == SA) { sa = 0; ++usea; }
+        if (b_done && ++sb == SB) { sb = 0; ++useb; }
+        if (!last && ((b_done && !wait(fullB(sb), useb)) || !wait(fullA(sa), usea))) ok = false;
         if (tc_elect()) {
-          mma_commit(est);                   // stage reusable once these MMAs finish
-          if (last) mma_commit(tfull(bf));   // this tile's D final
+          issue_pairs<5>(std::make_integer_sequence<int, 5>{}, s == 0, dc, aT, bd, idesc);
+          tc_commit(eA);
+          if (b_done) tc_commit(eB);
+          if (last) tc_commit(tfull(bf));
         }
         __syncwarp();
         if (!ok) break;
       }
+      if (++bf == nbuf) { bf = 0; ++used; }
     }
-    if (!ok && lane == 0) {
-      if (!*vfail && atomicCAS(err, 0, TW_ERR_TIMEOUT) == 0) err[1] = 23;
-      fail = 1;
-    }
+    if (!ok && lane == 0) note(err, vfail, 23);
     // every issued MMA complete before TMEM is released
-    if (tc_elect()) mma_commit(drain);
-    mbar_drain(drain, 0);
-  } else {
-    // ---------------- epilogue: (D0 + D1) + D2 from TMEM, scaled, complex64 out
-    const int lg = warp & 3;                          // TMEM lanes 32 lg .. 32 lg + 31
-    const int r = 32 * lg + lane;
-    for (int i = 0; i < my_tiles; ++i) {
+    if (tc_elect()) tc_commit(drain);
+    tc_mbar_wait(drain, 0, nullptr);
+  } else if (lane == 0) {
+    // ---------------- B' slices: one bulk copy per atom
+    int st = 0, use = 0, issued = 0;
+    bool ok = true;
+    for (int i = 0; i < my_tiles && ok; ++i) {
       int mt, w, nt;
       tile_of(i, mt, w, nt);
-      const int bf = i % nbuf;
-      if (!mbar_wait(tfull(bf), (unsigned)((i / nbuf) & 1), vfail) || *vfail) {
-        if (!*vfail && atomicCAS(err, 0, TW_ERR_TIMEOUT) == 0) err[1] = 22;
-        fail = 1;
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int m = mt * TM + r;
-      const float sa = pow2f((m < Nm ? (int)ea[(size_t)w * Nm + m] : EXP_MIN) - 7);
-      const uint32_t trow = tmem + ((uint32_t)(32 * lg) << 16) + (uint32_t)(bf * 3 * N);
-      for (int c0 = 0; c0 < P; c0 += 8) {
-        uint32_t d0r[8], d0i[8], d1r[8], d1i[8], d2r[8], d2i[8];
-#define TW_LD8(dst, col)                                                                       \
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"          \
-               : "=r"(dst[0]), "=r"(dst[1]), "=r"(dst[2]), "=r"(dst[3]), "=r"(dst[4]),        \
-                 "=r"(dst[5]), "=r"(dst[6]), "=r"(dst[7])                                     \
-               : "r"(trow + (uint32_t)(col)))
-        TW_LD8(d0r, c0);
-        TW_LD8(d0i, P + c0);
-        TW_LD8(d1r, N + c0);
-        TW_LD8(d1i, N + P + c0);
-        TW_LD8(d2r, 2 * N + c0);
-        TW_LD8(d2i, 2 * N + P + c0);
-#undef TW_LD8
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (c0 + 8 >= P) {
-          // the buffer is read: the MMAs of a later tile may overwrite it
-          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          mbar_arrive(tempty(bf));
-        }
-        if (m < Nm) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int b = nt * P + c0 + j;
-            if (b < B) {
-              const float sb = pow2f(eb[(size_t)w * ntiles * P + b] - 7);
-              const float re = __fadd_rn(__fadd_rn(__uint_as_float(d0r[j]), __uint_as_float(d1r[j])),
-                                         __uint_as_float(d2r[j])) * sa * sb;
-              const float im = __fadd_rn(__fadd_rn(__uint_as_float(d0i[j]), __uint_as_float(d1i[j])),
-                                         __uint_as_float(d2i[j])) * sa * sb;
-              X[(size_t)b * x_bstride + (size_t)w * Nm + m] = cf_make(re, im);
-            }
-          }
-        }
+      const uint8_t *Bw = Bt + ((size_t)w * ntiles + nt) * natoms * b_stage;
+      for (int a = 0; a < natoms; ++a) {
+        if (use > 0 && !tc_mbar_wait(emptyB(st), (unsigned)((use - 1) & 1), vfail)) { ok = false; break; }
+        tc_mbar_arrive_tx(fullB(st), b_stage);
+        tc_bulk_g2s(sB0 + (uint32_t)st * b_stage, Bw + (size_t)a * b_stage, b_stage, fullB(st));
+        ++issued;
+        if (++st == SB) { st = 0; ++use; }
       }
     }
+    if (!ok) note(err, vfail, 24);
+    // copies already issued must land before the CTA's shared memory goes
+    for (int a = (issued > SB ? issued - SB : 0); a < issued; ++a)
+      tc_mbar_wait(fullB(a % SB), (unsigned)((a / SB) & 1), nullptr);
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  tc_fence_before();
   __syncthreads();
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols)
-                 : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_slot), "r"(512u) : "memory");
 }
 
 }  // namespace
@@ -600,8 +531,8 @@ size_t sl_ws_bytes(int Nf, int Nr, int bcols) {
 size_t sl_eb_bytes(int Nf, int bcols) { return (size_t)Nf * ((bcols + 7) / 8 * 8) * sizeof(int); }
 
 int sl_pick_tile(int B) {
-  // right-hand sides per tile: one tile up to 80 (N = 160 columns, three
-  // accumulators in 480 TMEM columns), else the fewest tiles of a multiple of 8
+  // right-hand sides per tile: one tile up to 72 (N = 144 columns, three
+  // accumulators in 432 TMEM columns), else the fewest tiles of a multiple of 8
   const int P8 = (B + 7) / 8 * 8;
   if (P8 <= SL_PMAX) return P8;
   const int nt = (P8 + SL_PMAX - 1) / SL_PMAX;
@@ -631,39 +562,32 @@ cudaError_t launch_gemm_adj_sl(const void *A, int fmt, const int8_t *ea, const c
   if (B <= 0) return cudaSuccess;
   if (Nr > 512 || (fmt != FMT_C64 && fmt != FMT_BF16X2)) return cudaErrorInvalidValue;
   if (P <= 0) P = sl_pick_tile(B);
-  if (P % 8 != 0 || P > SL_PMAX) return cudaErrorInvalidValue;
+  if (P % 8 != 0 || P > 80) return cudaErrorInvalidValue;
+  P = P > SL_PMAX ? SL_PMAX : P;
   const int ntiles = (B + P - 1) / P, natoms = sl_natoms(Nr), N = 2 * P;
   if (sl_ws_bytes(Nf, Nr, ntiles * P) > ws_bytes || (size_t)Nf * ntiles * P * sizeof(int) > eb_bytes)
     return cudaErrorInvalidValue;
   k_bsl_build<<<dim3(Nf, ntiles), 256, 0, s>>>(Y, y_bstride, Nr, B, P, natoms,
                                                reinterpret_cast<uint8_t *>(ws), eb, ntiles);
   count_launches(1);
-  // TMEM: three accumulators of N columns, twice when 6N columns fit
-  const int nbuf = 6 * N <= 512 ? 2 : 1;
-  unsigned cols = 32;
-  while ((int)cols < nbuf * 3 * N) cols <<= 1;
-  // slice stages: as many (up to 4) as 227 KB of shared memory allows
-  const size_t fixed = 1024 + (size_t)RAW_D * RAW_STAGE, per_stage = (size_t)A_STAGE + (size_t)NSL * N * 64;
-  int S = MAXST;
-  while (S > 2 && fixed + S * per_stage > 227u * 1024u) --S;
-  const size_t sm = fixed + S * per_stage;
-  // persistent: one CTA per SM (the shared memory allows no second one)
+  // TMEM: three accumulators of N columns, twice if that leaves two A' stages,
+  // the rest A' stages
+  const int nbuf = 6 * N + 2 * A_COLS <= 512 ? 2 : 1;
+  const int SA = std::min(MAXA, (512 - nbuf * 3 * N) / A_COLS);
+  const size_t sm = 1024 + (size_t)RAW_D * RAW_SLOT + (size_t)SB * NSL * N * 64;
+  // persistent: one CTA per SM (the registers allow no second one)
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const long tiles = (long)((Nm + TM - 1) / TM) * Nf * ntiles;
   const unsigned grid = (unsigned)(tiles < nsm ? tiles : (nsm > 0 ? nsm : 1));
-  if (fmt == FMT_C64) {
-    cudaFuncSetAttribute(k_gemm_adj_sl<FMT_C64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_gemm_adj_sl<FMT_C64><<<grid, NTHR_P, sm, s>>>(A, ea, reinterpret_cast<const uint8_t *>(ws), eb, X,
-                                                    x_bstride, B, P, ntiles, Nr, Nm, Nf, natoms, S, nbuf,
-                                                    cols, err);
-  } else {
-    cudaFuncSetAttribute(k_gemm_adj_sl<FMT_BF16X2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_gemm_adj_sl<FMT_BF16X2><<<grid, NTHR_P, sm, s>>>(A, ea, reinterpret_cast<const uint8_t *>(ws), eb,
-                                                       X, x_bstride, B, P, ntiles, Nr, Nm, Nf, natoms, S,
-                                                       nbuf, cols, err);
-  }
+  auto run = [&](auto *k) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    k<<<grid, NTHR, sm, s>>>(reinterpret_cast<const uint2 *>(A), ea, reinterpret_cast<const uint8_t *>(ws), eb, X,
+                             x_bstride, B, P, ntiles, Nr, Nm, Nf, natoms, SA, nbuf, err);
+  };
+  if (fmt == FMT_C64) run(k_gemm_adj_sl<FMT_C64>);
+  else run(k_gemm_adj_sl<FMT_BF16X2>);
   count_launches(1);
   return cudaGetLastError();
 }
