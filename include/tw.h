@@ -428,12 +428,13 @@ tw_status tw_infer_batch(tw_ctx *ctx, tw_prec prec, int nrhs, const int *nt_wind
  * later context of the same shape takes it without measuring.  The
  * environment variable TW_AUTOTUNE=0 keeps the built-in rules instead.
  *   adj_tile  : right-hand sides per tensor-core tile of the reduced-
- *               precision adjoint (multiple of 8, <= 80; more tiles re-read
+ *               precision adjoint (multiple of 8, <= 80, 80 as 72; more tiles re-read
  *               the operator, fewer leave the MMA narrow)
  *   adj_rw    : right-hand sides per warp of the FP64-class adjoint on the
  *               FP32 pipes (1, 2, 4), the forward product there too; 0 = both
  *               on the tensor cores (on the FP32 pipes by batch size if their
- *               workspaces did not fit)
+ *               workspaces did not fit): exact fixed-point slices, 56 bits below
+ *               the largest entry of an operator row and of a data column
  *   fwd_lanes : lanes per right-hand side of the forward products (1, 2)
  * A column's result never depends on its batch mates for any choice; it
  * can differ in the last bits between choices (fwd_lanes changes the order
