@@ -19,8 +19,9 @@
 // take no part in the dependency chain.  In a row, every dependency but
 // the last is summed as soon as it is ready (factor blocks streamed into
 // shared memory with asynchronous copies, double-buffered); the diagonal
-// inverse is applied before waiting for the last one, which costs a single
-// 64x64 product with the precomputed chain block.  Every wait is bounded
+// inverse is applied before waiting for the last one (with pre-multiplied
+// blocks: before the first), which costs a single 64x64 product with its own
+// or the precomputed chain block.  Every wait is bounded
 // (2 s), after which the kernel records TW_ERR_TIMEOUT, raises the abort
 // flag that all CTAs poll, and returns.
 //
@@ -45,7 +46,7 @@ constexpr int CS = 8;      // right-hand sides per column slice
 // with four threads sharing each row's 64 products (16 dependent ones instead
 // of 64; the sums are joined in another order).  The blocks are read (from
 // L2) once per slice.  Measured (us a sweep, CS / CSN / CSP): 118 block rows, 11
-// right-hand sides 740 / 480 / 350; 188 and 16 1,370 / 1,000 / 760.
+// right-hand sides 740 / 420 / 350; 188 and 16 1,370 / 980 / 760.
 constexpr int CSN = 4, CSP = 2;
 constexpr int LDA = 66;    // padded row stride (elements) of shared 64x64 tiles
 constexpr int LDZ = 66;    // padded column stride of shared 64 x CS tiles
@@ -236,7 +237,27 @@ k_trsm(const T *__restrict__ Lp, const T *__restrict__ Linv, const T *__restrict
         if (has1 && k0 == 0) acc[1] = S::from(S::ld_cg(o1 + gi));
       }
     }
-    const int nbulk = u > dlo ? u - 1 : dlo;
+    // SCALED: Linv d does not wait for anything, so it comes first, and the last
+    // dependency's block (its own chain block) is one more of the bulk, staged
+    // under the product before it.  Both were between the last but one z and
+    // the last product: 4.1 -> 3.6 us a row with slices of four (118 block rows, 11
+    // right-hand sides).
+    typename S::acc cacc[2] = {S::zero(), S::zero()};
+    T res[2] = {S::zv(), S::zv()};
+    if constexpr (SCALED) {
+      stage_block(As, Linv + (size_t)I * NB_ * NB_);
+      cp_commit();
+      Vs[c0 * LDZ + r] = (gi < nrows[0]) ? bv[0] : S::zv();
+      if (NCT == 2) Vs[(c0 + 1) * LDZ + r] = (gi < nrows[1]) ? bv[1] : S::zv();
+      cp_wait<0>();
+      __syncthreads();
+      typename S::acc wacc[2] = {S::zero(), S::zero()};
+      tile_mac<T, FWD, KS, NCT>(wacc, As, Vs, r, c0, k0);
+      res[0] = S::get(wacc[0]);
+      res[1] = S::get(wacc[1]);
+      __syncthreads();                   // As is free again
+    }
+    const int nbulk = SCALED ? u : (u > dlo ? u - 1 : dlo);
     auto dep_block = [&](int d) -> const T * {
       const int J = FWD ? d : NBs - 1 - d;
       return Lp + (FWD ? packed_index(I, J) : packed_index(J, I)) * NB_ * NB_;
@@ -258,7 +279,7 @@ k_trsm(const T *__restrict__ Lp, const T *__restrict__ Linv, const T *__restrict
               break;
             }
             const int behind = u - p;
-            __nanosleep(behind > 2 ? min(4096, 256 * (behind - 2)) : 64);
+            __nanosleep(behind > 2 ? min(4096, 256 * (behind - 2)) : 32);
           }
         }
         sP = p;
@@ -288,65 +309,66 @@ k_trsm(const T *__restrict__ Lp, const T *__restrict__ Linv, const T *__restrict
           cp_wait<0>();
         }
         __syncthreads();
-        tile_mac<T, FWD, KS, NCT>(acc, As + (d & 1) * NB_ * LDA, Zs + (d & 1) * NC * LDZ, r, c0, k0);
+        const T *Ad = As + (d & 1) * NB_ * LDA, *Zd = Zs + (d & 1) * NC * LDZ;
+        if (SCALED && d == u - 1) tile_mac<T, FWD, KS, NCT>(cacc, Ad, Zd, r, c0, k0);
+        else tile_mac<T, FWD, KS, NCT>(acc, Ad, Zd, r, c0, k0);
         __syncthreads();
         zpre = znext;
       }
     }
-    // ---- v = b - bulk;  w = Linv v (FWD) or Linv^T v (BWD)
-    //      (SCALED: v = b, and the bulk is subtracted from w)
-    stage_block(As, Linv + (size_t)I * NB_ * NB_);
-    cp_commit();
-    const bool chain = u > dlo;
-    if (chain) {
-      stage_block(As + NB_ * LDA, SCALED ? dep_block(u - 1) : Lchain + (size_t)I * NB_ * NB_);
-      cp_commit();
-    }
-    if constexpr (SCALED) {
-      Vs[c0 * LDZ + r] = (gi < nrows[0]) ? bv[0] : S::zv();
-      if (NCT == 2) Vs[(c0 + 1) * LDZ + r] = (gi < nrows[1]) ? bv[1] : S::zv();
-    } else {
-      Vs[c0 * LDZ + r] = (gi < nrows[0]) ? S::sub(bv[0], S::get(acc[0])) : S::zv();
-      if (NCT == 2) Vs[(c0 + 1) * LDZ + r] = (gi < nrows[1]) ? S::sub(bv[1], S::get(acc[1])) : S::zv();
-    }
-    if (chain) cp_wait<1>(); else cp_wait<0>();
-    __syncthreads();
-    typename S::acc wacc[2] = {S::zero(), S::zero()};
-    tile_mac<T, FWD, KS, NCT>(wacc, As, Vs, r, c0, k0);
-    T res[2] = {S::get(wacc[0]), S::get(wacc[1])};
     if constexpr (SCALED) {
       res[0] = S::sub(res[0], S::get(acc[0]));
       res[1] = S::sub(res[1], S::get(acc[1]));
-    }
-    // ---- the last dependency: one product with the chain block
-    if (chain) {
-      if (tid == 0) {
-        const unsigned long long t0 = now_ns();
-        while (ld_acq(progress) < u) {
-          if (*(volatile int *)abort_flag) { sbail = 1; break; }
-          if (now_ns() - t0 > WAIT_NS) {
-            note_error(err, TW_ERR_TIMEOUT, FWD ? 7 : 8);
-            atomicExch(abort_flag, 1);
-            sbail = 1;
-            break;
+      if (u > dlo) {
+        res[0] = S::sub(res[0], S::get(cacc[0]));
+        res[1] = S::sub(res[1], S::get(cacc[1]));
+      }
+    } else {
+      // ---- v = b - bulk;  w = Linv v (FWD) or Linv^T v (BWD)
+      stage_block(As, Linv + (size_t)I * NB_ * NB_);
+      cp_commit();
+      const bool chain = u > dlo;
+      if (chain) {
+        stage_block(As + NB_ * LDA, Lchain + (size_t)I * NB_ * NB_);
+        cp_commit();
+      }
+      Vs[c0 * LDZ + r] = (gi < nrows[0]) ? S::sub(bv[0], S::get(acc[0])) : S::zv();
+      if (NCT == 2) Vs[(c0 + 1) * LDZ + r] = (gi < nrows[1]) ? S::sub(bv[1], S::get(acc[1])) : S::zv();
+      if (chain) cp_wait<1>(); else cp_wait<0>();
+      __syncthreads();
+      typename S::acc wacc[2] = {S::zero(), S::zero()};
+      tile_mac<T, FWD, KS, NCT>(wacc, As, Vs, r, c0, k0);
+      res[0] = S::get(wacc[0]);
+      res[1] = S::get(wacc[1]);
+      // ---- the last dependency: one product with the chain block
+      if (chain) {
+        if (tid == 0) {
+          const unsigned long long t0 = now_ns();
+          while (ld_acq(progress) < u) {
+            if (*(volatile int *)abort_flag) { sbail = 1; break; }
+            if (now_ns() - t0 > WAIT_NS) {
+              note_error(err, TW_ERR_TIMEOUT, FWD ? 7 : 8);
+              atomicExch(abort_flag, 1);
+              sbail = 1;
+              break;
+            }
+            __nanosleep(32);
           }
-          __nanosleep(32);
         }
+        __syncthreads();
+        if (sbail) { cp_wait<0>(); return; }
+        const int J = FWD ? I - 1 : I + 1;
+        for (int i = tid; i < NC * NB_; i += 256) {
+          const int c = i >> 6, k = i & 63;
+          Zs[c * LDZ + k] = (b0 + c < B) ? S::ld_cg(out + (long)(b0 + c) * out_bstride + (long)J * NB_ + k)
+                                         : S::zv();
+        }
+        cp_wait<0>();
+        __syncthreads();
+        tile_mac<T, FWD, KS, NCT>(cacc, As + NB_ * LDA, Zs, r, c0, k0);
+        res[0] = S::sub(res[0], S::get(cacc[0]));
+        res[1] = S::sub(res[1], S::get(cacc[1]));
       }
-      __syncthreads();
-      if (sbail) { cp_wait<0>(); return; }
-      const int J = FWD ? I - 1 : I + 1;
-      for (int i = tid; i < NC * NB_; i += 256) {
-        const int c = i >> 6, k = i & 63;
-        Zs[c * LDZ + k] = (b0 + c < B) ? S::ld_cg(out + (long)(b0 + c) * out_bstride + (long)J * NB_ + k)
-                                       : S::zv();
-      }
-      cp_wait<0>();
-      __syncthreads();
-      typename S::acc cacc[2] = {S::zero(), S::zero()};
-      tile_mac<T, FWD, KS, NCT>(cacc, As + NB_ * LDA, Zs, r, c0, k0);
-      res[0] = S::sub(res[0], S::get(cacc[0]));
-      res[1] = S::sub(res[1], S::get(cacc[1]));
     }
     if constexpr (NC == 2) {             // the four partial sums of the row
 #pragma unroll
@@ -421,7 +443,7 @@ cudaError_t launch_trsm_dd_scaled(const dd *Lx, const dd *Linv, const void *rhs,
   if (split)
     return trsm_all<dd, true, CSP>(Lx, Linv, nullptr, rhs, rhs_kind, rhs_bstride, out, out_bstride, win, Nd, Nt,
                                    B, NB, prog, fwd, err, abort_flag, s);
-  // Slices of four while the chain bounds the sweep: it takes NB (about 4.4 us a
+  // Slices of four while the chain bounds the sweep: it takes NB (about 3.6 us a
   // row, 6.4 with slices of eight) against the products, NB / 2 blocks a row and
   // about 12 ns a block and eight right-hand sides on 152 SMs.
   if ((long)((B + CS - 1) / CS) * NB <= 800)
