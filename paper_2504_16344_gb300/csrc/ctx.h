@@ -55,13 +55,15 @@ struct tw_ctx {
   // G^ = F^ C per frequency (the paper's G* = Gamma_pr F* of Phase 2), per kept
   // format, when TW_KEEP_G: the adjoint applies of tw_infer then need no prior filter
   void *opG[3] = {nullptr, nullptr, nullptr};
-  // row exponents of the stored operators for the batched adjoint on the tensor
-  // cores: ea[which][fmt][w][m], eaG[fmt] for G^ (gemm_sl.cu; fmt 0, F only:
-  // gemm_sl64.cu, null if they did not fit)
+  // row exponents of the FP32 storages for the batched adjoint on the tensor
+  // cores: ea[which][fmt][w][m] (fmt 1, 2), eaG[fmt] for G^ (gemm_sl.cu)
   int8_t *ea[2][3] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};
   int8_t *eaG[3] = {nullptr, nullptr, nullptr};
-  // exponents of each row of the FP64-class operators over the grid, ef[which][w][r]
-  // (gemm_fwd_sl64.cu; null if they did not fit)
+  // the same of the FP64-class operators, held while a batch is reserved (null:
+  // not reserved, or they did not fit): ea64[w][m] of the one the batched adjoint
+  // reads (G^ if kept, else F^; gemm_sl64.cu), ef[which][w][r] of each row over
+  // the grid (gemm_fwd_sl64.cu)
+  int8_t *ea64 = nullptr;
   int8_t *ef[2] = {nullptr, nullptr};
   std::vector<char> loaded[2];     // per row: loaded?
   std::vector<unsigned long long> col_hash;   // per row of F: fingerprint of its block column

@@ -63,9 +63,9 @@ __device__ __forceinline__ void note(int *err, volatile int *fail, int info) {
 }
 
 // e[w][r] (or e[w][b]): exponent of one row of Nm complex entries; row y of
-// frequency x = blockIdx.x starts at A + x * ws + y * rs
+// frequency x = blockIdx.x starts at A + x * ws + y * rs, its exponent is e[x es + y]
 __global__ void __launch_bounds__(256)
-k_rowmax_exp(const float4 *__restrict__ A, long ws, long rs, int Nm, int8_t *__restrict__ e) {
+k_rowmax_exp(const float4 *__restrict__ A, long ws, long rs, int Nm, int8_t *__restrict__ e, int es) {
   __shared__ float red[8];
   const float4 *p = A + (long)blockIdx.x * ws + (long)blockIdx.y * rs;
   float mx = 0.f;
@@ -80,7 +80,7 @@ k_rowmax_exp(const float4 *__restrict__ A, long ws, long rs, int Nm, int8_t *__r
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int i = 1; i < 8; ++i) mx = fmaxf(mx, red[i]);
-    e[(size_t)blockIdx.x * gridDim.y + blockIdx.y] = (int8_t)tc_exp_above(mx);
+    e[(size_t)blockIdx.x * es + blockIdx.y] = (int8_t)tc_exp_above(mx);
   }
 }
 
@@ -509,8 +509,11 @@ long stage_cost(int mtiles, int ntiles, int N) { return (long)mtiles * ntiles * 
 // ------------------------------------------------------------------ host side
 int gemm_fwd_sl64_nrange(int Nm) { return (Nm + RANGE - 1) / RANGE; }
 
-cudaError_t launch_fwd_exp64(const void *F, int8_t *ef, int Nf, int Nr, int Nm, cudaStream_t s) {
-  k_rowmax_exp<<<dim3(Nf, Nr), 256, 0, s>>>(reinterpret_cast<const float4 *>(F), (long)Nr * Nm, Nm, Nm, ef);
+cudaError_t launch_fwd_exp64(const void *F, int8_t *ef, int Nf, int Nr, int Nm, int row0, int nrows,
+                             cudaStream_t s) {
+  if (nrows <= 0) return cudaSuccess;
+  k_rowmax_exp<<<dim3(Nf, nrows), 256, 0, s>>>(reinterpret_cast<const float4 *>(F) + (size_t)row0 * Nm, (long)Nr * Nm,
+                                               Nm, Nm, ef + row0, Nr);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -522,7 +525,7 @@ cudaError_t launch_gemm_fwd_sl64(const void *F, const int8_t *ef, const cdd *X, 
                                  cdd *part, int Nf, int Nr, int Nm, int B, int bmax, int *err, cudaStream_t s) {
   if (B <= 0) return cudaSuccess;
   const float4 *Xp = reinterpret_cast<const float4 *>(X), *Fp = reinterpret_cast<const float4 *>(F);
-  k_rowmax_exp<<<dim3(Nf, B), 256, 0, s>>>(Xp, Nm, x_bstride, Nm, ex);
+  k_rowmax_exp<<<dim3(Nf, B), 256, 0, s>>>(Xp, Nm, x_bstride, Nm, ex, B);
   count_launches(1);
   const int nr = gemm_fwd_sl64_nrange(Nm);
   int dev = 0, nsm = 0;

@@ -150,10 +150,11 @@ cudaError_t launch_gemm_adj_sl64(const void *A, const int8_t *ea, const cdd *Y, 
 // ---- FP64-class forward product on the tensor cores (gemm_fwd_sl64.cu) -----
 // partial sums of Yo[b][w][r] = sum_k F[w][r][k] X[b][w][k] per range of grid
 // points (gemm_fwd_sl64_nrange <= gemm_fwd_nchunk of them), to be added by
-// launch_gemm_fwd_reduce_dd; ef: [Nf][Nr] row exponents (launch_fwd_exp64), ex:
+// launch_gemm_fwd_reduce_dd; ef: [Nf][Nr] row exponents (launch_fwd_exp64: of rows row0 .. row0 + nrows-1), ex:
 // Nf * B bytes of workspace, bmax: the reserved batch
 int gemm_fwd_sl64_nrange(int Nm);
-cudaError_t launch_fwd_exp64(const void *F, int8_t *ef, int Nf, int Nr, int Nm, cudaStream_t s);
+cudaError_t launch_fwd_exp64(const void *F, int8_t *ef, int Nf, int Nr, int Nm, int row0, int nrows,
+                             cudaStream_t s);
 cudaError_t launch_gemm_fwd_sl64(const void *F, const int8_t *ef, const cdd *X, long x_bstride, int8_t *ex,
                                  cdd *part, int Nf, int Nr, int Nm, int B, int bmax, int *err, cudaStream_t s);
 cudaError_t launch_gemm_fwd_reduce_dd(const cdd *part, cdd *Yo, long y_bstride, int nchunk, int Nf, int Nr, int B,

@@ -317,13 +317,6 @@ tw_status tw_create(tw_ctx **out, int Nd, int Nq, int Nx, int Ny, int Nt, double
           if (!c->ea[which][fmt]) st = twh::fail(c, TW_ERR_OOM, "row exponent tables");
         }
   }
-  // the FP64-class operator's are optional: without them its batched adjoint
-  // and forward product run on the FP32 pipes
-  if (st == TW_OK && c->op[TW_MAP_F][0]) {
-    c->ea[TW_MAP_F][0] = (int8_t *)twh::dalloc(c, Nf * Nm);
-    for (int which = 0; which < 2; ++which)
-      c->ef[which] = (int8_t *)twh::dalloc(c, Nf * (size_t)rows_of(c, which));
-  }
   if (st != TW_OK) {
     // keep the message for the caller: report via stderr since ctx is freed
     fprintf(stderr, "tw_create: %s\n", c->err.c_str());
@@ -393,16 +386,18 @@ tw_status tw_set_block_column(tw_ctx *c, tw_map which, int row0, int nrows, cons
     TW_CUDA(c, cudaStreamSynchronize(s));
     twh::dfree(c, dh);
   }
-  // every row present: the row exponents of the storages (one pass each)
+  // every row present: the row exponents of the FP32 storages (one pass each)
   bool all = true;
   for (char l : c->loaded[which]) all = all && l;
   for (int fmt = 1; fmt < 3 && all; ++fmt)
     if (c->ea[which][fmt])
       TW_CUDA(c, launch_row_exp(c->op[which][fmt], fmt, c->ea[which][fmt], c->Nf, R, c->Nm, s));
-  if (all && c->ea[which][0])
-    TW_CUDA(c, launch_row_exp64(c->op[which][0], c->ea[which][0], c->Nf, R, c->Nm, s));
-  if (all && c->ef[which])
-    TW_CUDA(c, launch_fwd_exp64(c->op[which][0], c->ef[which], c->Nf, R, c->Nm, s));
+  // a reservation's tables follow the operator: the forward product's are per
+  // row, so these rows' are valid whether or not the others are loaded
+  if (c->ef[which])
+    TW_CUDA(c, launch_fwd_exp64(c->op[which][0], c->ef[which], c->Nf, R, c->Nm, row0, nrows, s));
+  if (which == TW_MAP_F && c->ea64 && !c->opG[0])
+    TW_CUDA(c, launch_row_exp64(c->op[which][0], c->ea64, c->Nf, R, c->Nm, s));
   // with the prior known, keep G = Phi C^{1/2} of these rows for tw_factor_K,
   // computed in FP64 from the caller's FP64 column
   if (which == TW_MAP_F && c->prior_set) {

@@ -153,9 +153,8 @@ tw_status infer_core(tw_ctx *c, tw_lane &L, tw_prec prec, int B, const int *win,
     { twh::Phase p(c, TW_PH_GEMV_ADJ, s);
       // tensor cores unless a SIMT tile was chosen (tw_batch_tiles) or their
       // exponents or workspace did not fit
-      const int8_t *ea = useG ? c->eaG[0] : c->ea[TW_MAP_F][0];
-      if (L.adj_rw == 0 && ea && L.sl64_ws)
-        TW_CUDA(c, launch_gemm_adj_sl64(A, ea, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm,
+      if (L.adj_rw == 0 && c->ea64 && L.sl64_ws)
+        TW_CUDA(c, launch_gemm_adj_sl64(A, c->ea64, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm,
                                         Nf, Nd, Nm, B, L.sl64_ws, L.sl64_ws_n, L.sl64_eb, L.sl64_eb_n,
                                         c->d_err, s));
       else
@@ -263,7 +262,7 @@ size_t lane_bytes(const tw_ctx *c, int bmax) {
     b += 2 * B * np * sizeof(dd) + sl_ws_bytes(c->Nf, c->Rmax, cols) + sl_eb_bytes(c->Nf, cols);
   }
   if (c->trsm_eb) b += trsm_tc_ws_bytes(bmax);
-  if (c->ea[TW_MAP_F][0]) b += sl64_ws_bytes(c->Nf, c->Nd, bmax) + sl64_eb_bytes(c->Nf, bmax) + (size_t)c->Nf * bmax;
+  if (c->ea64) b += sl64_ws_bytes(c->Nf, c->Nd, bmax) + sl64_eb_bytes(c->Nf, bmax) + (size_t)c->Nf * bmax;
   return b;
 }
 
@@ -310,7 +309,7 @@ tw_status alloc_lane(tw_ctx *c, tw_lane &L, int bmax) {
     L.trsm_ws_n = trsm_tc_ws_bytes(bmax);
     L.trsm_ws = twh::dalloc(c, L.trsm_ws_n);
   }
-  if (ok && c->ea[TW_MAP_F][0]) {     // optional: null leaves the SIMT product
+  if (ok && c->ea64) {                // optional: null leaves the SIMT product
     L.sl64_ws_n = sl64_ws_bytes(c->Nf, c->Nd, bmax);
     L.sl64_eb_n = sl64_eb_bytes(c->Nf, bmax);
     L.sl64_eb = (int *)twh::dalloc(c, L.sl64_eb_n);
@@ -338,8 +337,10 @@ void free_batch(tw_ctx *c) {
   twh::dfree(c, c->inv_dd);
   twh::dfree(c, c->trsm_ef);
   twh::dfree(c, c->trsm_eb);
+  twh::dfree(c, c->ea64);
+  for (int8_t *&e : c->ef) { twh::dfree(c, e); e = nullptr; }
   c->inv_dd = nullptr;
-  c->trsm_ef = c->trsm_eb = nullptr;
+  c->trsm_ef = c->trsm_eb = c->ea64 = nullptr;
 }
 
 }  // namespace
@@ -348,6 +349,8 @@ tw_status twh::refresh_dd_factor(tw_ctx *c, cudaStream_t s) {
   if (!c->have64) return TW_OK;
   if (c->inv_dd) TW_CUDA(c, launch_double_to_dd(c->inv64, c->inv_dd, (size_t)c->NB * NB_ * NB_, s));
   if (c->trsm_eb) TW_CUDA(c, launch_trsm_tc_exp(c->Lfs, c->Lbs, c->trsm_ef, c->trsm_eb, c->NB, s));
+  if (c->ea64)
+    TW_CUDA(c, launch_row_exp64(c->opG[0] ? c->opG[0] : c->op[TW_MAP_F][0], c->ea64, c->Nf, c->Nd, c->Nm, s));
   TW_CUDA(c, cudaStreamSynchronize(s));
   return TW_OK;
 }
@@ -373,6 +376,13 @@ tw_status tw_reserve_batch(tw_ctx *c, int bmax) {
     c->trsm_ef = (int8_t *)twh::dalloc(c, trsm_tc_exp_bytes(c->NB));
     if (c->trsm_ef) c->trsm_eb = (int8_t *)twh::dalloc(c, trsm_tc_exp_bytes(c->NB));
   }
+  // optional as well: exponents of the operators that the sliced products read;
+  // without them those products run on the FP32 pipes
+  if (c->op[TW_MAP_F][TW_PREC_FP64]) {
+    c->ea64 = (int8_t *)twh::dalloc(c, (size_t)c->Nf * c->Nm);
+    for (int which = 0; which < 2; ++which)
+      c->ef[which] = (int8_t *)twh::dalloc(c, (size_t)c->Nf * (which == TW_MAP_F ? c->Nd : c->Nq));
+  }
   tw_status st = twb::alloc_lane(c, c->lane, bmax);
   if (st != TW_OK) {
     free_batch(c);
@@ -380,6 +390,12 @@ tw_status tw_reserve_batch(tw_ctx *c, int bmax) {
   }
   st = twh::refresh_dd_factor(c, 0);
   if (st != TW_OK) return st;
+  // (rows of F_q that are not loaded yet get theirs in tw_set_block_column)
+  for (int which = 0; which < 2; ++which)
+    if (c->ef[which]) {
+      const int R = which == TW_MAP_F ? c->Nd : c->Nq;
+      TW_CUDA(c, launch_fwd_exp64(c->op[which][TW_PREC_FP64], c->ef[which], c->Nf, R, c->Nm, 0, R, 0));
+    }
   return twb::autotune_lane(c, c->lane);
 }
 

@@ -122,8 +122,6 @@ tw_status form_gstar(tw_ctx *c, cudaStream_t s) {
                              cudaMemcpyDeviceToDevice, s));
   TW_CUDA(c, launch_prior_cfields_d((cdd *)c->opG[0], (long)c->Nf * c->Nd, c->Nx, c->Ny, (cd *)c->ws,
                                     (c->Nt + 1) / 2, c->lam1d, c->plX, c->plY, c->twXd, c->twYd, s));
-  if (!c->eaG[0]) c->eaG[0] = (int8_t *)twh::dalloc(c, (size_t)c->Nf * c->Nm);   // optional, as ea
-  if (c->eaG[0]) TW_CUDA(c, launch_row_exp64(c->opG[0], c->eaG[0], c->Nf, c->Nd, c->Nm, s));
   for (int fmt = 1; fmt < 2; ++fmt)
     if (c->opG[fmt]) {
       TW_CUDA(c, launch_convert_op((const cdd *)c->opG[0], (long)per_w, c->opG[fmt], fmt, (long)per_w,
