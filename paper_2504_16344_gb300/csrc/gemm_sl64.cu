@@ -18,9 +18,11 @@
 // 2^-8L and at most (L+1) K' 2^14 2^-8L (one slice may reach 129: + 0.4%),
 // below 2^24 units for K' <= 204.  Levels 5 and 6 share a sixth accumulator,
 // 2^-40 below the terms, where truncation does no harm.  More than 102 rows
-// are summed in chunks of 96 (K' = 192), added to X^ in double-float.  The
-// double-float product this replaces rounds its running sum at 2^-48 after
-// every one of the 2 Nr terms.
+// are summed in chunks of 96 (K' = 192), added to X^ in double-float.  An entry
+// 2^-p of its row's largest keeps 56 - p bits, so a sum whose large entries meet
+// small ones would come out with fewer digits than in double-float, which rounds its
+// running sum at 2^-48 after every one of the 2 Nr terms: those sums are found from
+// their magnitudes and formed in double-float (k_adj_check, k_adj_guard).
 //
 // What bounds it.  The SIMT double-float product (gemm.cu) spends about 60
 // FP32 operations per operator entry and right-hand side and is bound by the
@@ -93,11 +95,13 @@ __global__ void k_row_exp64(const float4 *__restrict__ A, int8_t *__restrict__ e
 }
 
 // B' slices: tiles [w][nt][atom][slice][2P rows][32 bf16] (64-byte swizzle),
-// column exponents eb[w][nt P + b]
+// column exponents eb[w][nt P + b], magnitudes mag[w][nt P + b][nrp] (bf16)
 __global__ void __launch_bounds__(256)
 k_bsl64_build(const cdd *__restrict__ Y, long y_bstride, int Nr, int B, int P, int natoms,
-              uint8_t *__restrict__ tiles, int *__restrict__ eb, int ntiles) {
+              uint8_t *__restrict__ tiles, int *__restrict__ eb, uint16_t *__restrict__ mag, int nrp, int *__restrict__ todo,
+              int ntiles) {
   __shared__ int e_sh[PMAX];
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) todo[0] = 0;
   const int w = blockIdx.x, nt = blockIdx.y, N = 2 * P;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int bl = warp; bl < P; bl += 8) {
@@ -116,6 +120,16 @@ k_bsl64_build(const cdd *__restrict__ Y, long y_bstride, int Nr, int B, int P, i
     }
   }
   __syncthreads();
+  // |Re| + |Im| below 2, for the guard
+  for (int t = threadIdx.x; t < P * nrp; t += blockDim.x) {
+    const int bl = t / nrp, s = t % nrp, b = nt * P + bl;
+    float v = 0.f;
+    if (b < B && s < Nr) {
+      const cdd y = ld_cdd(Y + (size_t)b * y_bstride + (size_t)w * Nr + s);
+      v = (fabsf(y.re.hi) + fabsf(y.im.hi)) * tc_pow2f(-e_sh[bl]);
+    }
+    mag[((size_t)w * ntiles * P + b) * nrp + s] = (uint16_t)(__float_as_uint(v) >> 16);
+  }
   const size_t slice_bytes = (size_t)N * 64;
   uint8_t *base = tiles + ((size_t)w * ntiles + nt) * natoms * NSL * slice_bytes;
   for (int t = threadIdx.x; t < natoms * N * 4; t += blockDim.x) {
@@ -467,7 +481,154 @@ k_gemm_adj_sl64(const float4 *__restrict__ A, const int8_t *__restrict__ ea, con
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_slot), "r"(512u) : "memory");
 }
 
+// ------------------------------------------------------ the guard (tc.cuh)
+// low[w][tile][s]: the least |F^[s][m]| of a tile's 128 grid points, in units of
+// the point's exponent (bf16, rounded down; rows past Nr zero).  Points that no
+// sensor sees (no entry of 2^-100) are left out: their sums are zero
+__global__ void __launch_bounds__(TM)
+k_adj_low(const float4 *__restrict__ A, const int8_t *__restrict__ ea, uint16_t *__restrict__ low, int nrp, int Nr,
+          int Nm) {
+  __shared__ unsigned sh[2][TM / 32];
+  const int w = blockIdx.y, m = blockIdx.x * TM + threadIdx.x;
+  const int e = m < Nm ? (int)ea[(size_t)w * Nm + m] : -100;
+  const float4 *p = A + (size_t)w * Nr * Nm + min(m, Nm - 1);
+  uint16_t *out = low + ((size_t)w * gridDim.x + blockIdx.x) * nrp;
+  for (int s = 0; s < nrp; ++s) {
+    unsigned v = 0x7f800000u;
+    if (s >= Nr) v = 0;
+    else if (e > -100) {
+      const float4 a = __ldcs(p + (size_t)s * Nm);
+      v = __float_as_uint((fabsf(a.x) + fabsf(a.z)) * tc_pow2f(-e));
+    }
+    v = __reduce_min_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) sh[s & 1][threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      v = min(min(sh[s & 1][0], sh[s & 1][1]), min(sh[s & 1][2], sh[s & 1][3]));
+      out[s] = (uint16_t)(min(v, 0x3f800000u) >> 16);      // (a tile without such points: any value)
+    }
+  }
+}
+
+// The tiles of 128 grid points and up to 64 columns (a piece of 64 of the ncols)
+// with a sum whose bound over the whole tile, sum_s low |Y|, does not settle it:
+// todo[1 ..], todo[0] of them (zeroed by k_bsl64_build).  A warp takes 16 tiles
+__global__ void __launch_bounds__(128)
+k_adj_check(const uint16_t *__restrict__ low, const uint16_t *__restrict__ mag, int nrp, int Nr, int ntl, int B,
+            int ncols, int *__restrict__ todo) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+  const int w = blockIdx.y, col0 = blockIdx.z * 64, t0 = (blockIdx.x * 4 + warp) * 16;
+  if (t0 >= ntl) return;
+  const int nf = min(8, (ncols - col0) / 8);
+  const uint16_t *lo = low + (size_t)w * ntl * nrp + 4 * c;
+  const uint16_t *mw = mag + ((size_t)w * ncols + col0 + g) * nrp + 4 * c;
+  const size_t ra = (size_t)min(t0 + g, ntl - 1) * nrp, rb = (size_t)min(t0 + g + 8, ntl - 1) * nrp;
+  float S[8][4] = {}, M[8][4] = {};
+  for (int s = 0; s < nrp; s += 16) {
+    const uint2 p = __ldg(reinterpret_cast<const uint2 *>(lo + ra + s)), q = __ldg(reinterpret_cast<const uint2 *>(lo + rb + s));
+    const uint32_t a[4] = {p.x, q.x, p.y, q.y}, one[4] = {0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u};
+#pragma unroll
+    for (int f = 0; f < 8; ++f)
+      if (f < nf) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(mw + (size_t)(8 * f) * nrp + s));
+        const uint32_t b[2] = {v.x, v.y};
+        tc_mma_mag(S[f], a, b);
+        tc_mma_mag(M[f], one, b);                          // zero: an empty column
+      }
+  }
+  const float thr = sqrtf(2.f * (float)Nr);
+  bool open[2] = {false, false};
+#pragma unroll
+  for (int f = 0; f < 8; ++f)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (col0 + 8 * f + 2 * c + (i & 1) < B && M[f][i] != 0.f && !(512.f * S[f][i] >= thr)) open[i >> 1] = true;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const unsigned any = __ballot_sync(0xffffffffu, open[h]);
+    if (c == 0 && ((any >> lane) & 15u) && t0 + g + 8 * h < ntl)
+      todo[1 + atomicAdd(todo, 1)] = (w * ntl + t0 + g + 8 * h) * (int)gridDim.z + (int)blockIdx.z;
+  }
+}
+
+// S[m][b] = sum_s |F^[s][m]| |Y[s][b]| of those tiles, from the operator; sums that
+// fail are formed in double-float and stored over the sliced ones.  A warp takes 16
+// points.  Bound by the operator's second reading where every tile is on the list:
+// 5.4 ms at 5.7 TB/s for 32 GB (64 right-hand sides of 100 sensors on 50,000
+// points), beside the product's 25; with G^ there, smooth in space, few are, and
+// both guard kernels take 0.7 ms.  Complex magnitudes: Re and Im of a sum share their
+// bound, as in the complex double-float product.
+__global__ void __launch_bounds__(256, 2)
+k_adj_guard(const float4 *__restrict__ A, const int8_t *__restrict__ ea, const uint16_t *__restrict__ mag, int nrp,
+            const cdd *__restrict__ Y, long y_bstride, cdd *__restrict__ X, long x_bstride, int Nr, int Nm, int B,
+            int ncols, int ntl, int ngrp, const int *__restrict__ todo) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+  const float thr = sqrtf(2.f * (float)Nr);                // T = 1: both sides are scaled
+  const int ntodo = todo[0];
+  for (int it = blockIdx.x; it < ntodo; it += gridDim.x) {
+    const int item = todo[1 + it], col0 = item % ngrp * 64, w = item / ngrp / ntl;
+    const int m0 = item / ngrp % ntl * TM + 16 * warp;
+    if (m0 >= Nm) continue;
+    const int nf = min(8, (ncols - col0) / 8);               // fragments of 8 columns
+    const int ma = min(m0 + g, Nm - 1), mb = min(m0 + g + 8, Nm - 1);
+    const float sa = tc_pow2f(-(int)ea[(size_t)w * Nm + ma]), sb = tc_pow2f(-(int)ea[(size_t)w * Nm + mb]);
+    const float4 *Aw = A + (size_t)w * Nr * Nm;
+    const uint16_t *Mw = mag + ((size_t)w * ncols + col0 + g) * nrp + 4 * c;
+    float4 v[2][4];
+    auto load = [&](int s0) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int s = min(s0 + 4 * c + j, Nr - 1);           // past the rows: the data's magnitude is zero
+        v[0][j] = __ldcs(Aw + (size_t)s * Nm + ma);
+        v[1][j] = __ldcs(Aw + (size_t)s * Nm + mb);
+      }
+    };
+    float d[8][4] = {};
+    load(0);
+    for (int s0 = 0; s0 < Nr; s0 += 16) {
+      float r[2][4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        r[0][j] = (fabsf(v[0][j].x) + fabsf(v[0][j].z)) * sa;
+        r[1][j] = (fabsf(v[1][j].x) + fabsf(v[1][j].z)) * sb;
+      }
+      if (s0 + 16 < Nr) load(s0 + 16);
+      const uint32_t a[4] = {tc_pack_bf16(r[0][0], r[0][1]), tc_pack_bf16(r[1][0], r[1][1]),
+                             tc_pack_bf16(r[0][2], r[0][3]), tc_pack_bf16(r[1][2], r[1][3])};
+#pragma unroll
+      for (int f = 0; f < 8; ++f)
+        if (f < nf) {
+          const uint2 q = __ldg(reinterpret_cast<const uint2 *>(Mw + (size_t)(8 * f) * nrp + s0));
+          const uint32_t b[2] = {q.x, q.y};
+          tc_mma_mag(d[f], a, b);
+        }
+    }
+    unsigned bad = 0;
+#pragma unroll
+    for (int f = 0; f < 8; ++f)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (m0 + g + 8 * (i >> 1) < Nm && col0 + 8 * f + 2 * c + (i & 1) < B && tc_guard_fails(d[f][i], thr))
+          bad |= 1u << (4 * f + i);
+    for (unsigned any = __reduce_or_sync(0xffffffffu, bad); any; any &= any - 1) {
+      const int e = __ffs(any) - 1, f = e >> 2, i = e & 3;
+      for (unsigned who = __ballot_sync(0xffffffffu, (bad >> e) & 1); who; who &= who - 1) {
+        const int l = __ffs(who) - 1;
+        const int m = m0 + (l >> 2) + 8 * (i >> 1), b = col0 + 8 * f + 2 * (l & 3) + (i & 1);
+        const cdd *Yb = Y + (size_t)b * y_bstride + (size_t)w * Nr;
+        cdd x = cdd_zero();
+        for (int s = lane; s < Nr; s += 32)
+          x = cdd_add(x, cdd_mul(cdd_conj(ld_cdd(reinterpret_cast<const cdd *>(Aw + (size_t)s * Nm + m))), ld_cdd(Yb + s)));
+        x.re = tc_warp_sum(x.re);
+        x.im = tc_warp_sum(x.im);
+        if (lane == 0) st_cdd(X + (size_t)b * x_bstride + (size_t)w * Nm + m, x);
+      }
+    }
+  }
+}
+
 int sl64_natoms(int Nr) { return (Nr + KA / 2 - 1) / (KA / 2); }
+int sl64_nrp(int Nr) { return (Nr + 15) / 16 * 16; }
 // right-hand sides per tile: the fewest tiles of at most PMAX, a multiple of 8
 int sl64_tile(int B) {
   const int nt = (B + PMAX - 1) / PMAX;
@@ -480,16 +641,28 @@ int sl64_tile(int B) {
 // workspace for any batch of at most bcols right-hand sides: tiles hold fewer
 // than 8 unused columns each, and there are at most ceil(bcols / PMAX) of them
 static int sl64_cols(int bcols) { return bcols + 8 * ((bcols + PMAX - 1) / PMAX); }
-size_t sl64_ws_bytes(int Nf, int Nr, int bcols) {
-  return (size_t)Nf * sl64_natoms(Nr) * NSL * 2 * (size_t)sl64_cols(bcols) * 64;
+size_t sl64_ws_bytes(int Nf, int Nr, int Nm, int bcols) {
+  // slices, then the magnitudes, then the guard's list of tiles
+  return (size_t)Nf * sl64_cols(bcols) * ((size_t)sl64_natoms(Nr) * NSL * 2 * 64 + (size_t)sl64_nrp(Nr) * 2) +
+         sizeof(int) * (1 + (size_t)Nf * ((Nm + TM - 1) / TM) * ((sl64_cols(bcols) + 63) / 64));
 }
 size_t sl64_eb_bytes(int Nf, int bcols) { return (size_t)Nf * sl64_cols(bcols) * sizeof(int); }
 
+// the operator's tables: row exponents, then (16-byte aligned) the guard's magnitudes
+static const uint16_t *sl64_low(const int8_t *ea, int Nf, int Nm) {
+  return reinterpret_cast<const uint16_t *>(ea + ((size_t)Nf * Nm + 15) / 16 * 16);
+}
+size_t row_exp64_bytes(int Nf, int Nr, int Nm) {
+  return ((size_t)Nf * Nm + 15) / 16 * 16 + (size_t)Nf * ((Nm + TM - 1) / TM) * sl64_nrp(Nr) * sizeof(uint16_t);
+}
 cudaError_t launch_row_exp64(const void *A, int8_t *ea, int Nf, int Nr, int Nm, cudaStream_t s) {
   const long total = (long)Nf * Nm;
   const long blocks = std::min<long>((total + 255) / 256, 152 * 32);
   k_row_exp64<<<(unsigned)blocks, 256, 0, s>>>(reinterpret_cast<const float4 *>(A), ea, Nf, Nr, Nm);
-  count_launches(1);
+  k_adj_low<<<dim3((Nm + TM - 1) / TM, Nf), TM, 0, s>>>(reinterpret_cast<const float4 *>(A), ea,
+                                                        const_cast<uint16_t *>(sl64_low(ea, Nf, Nm)), sl64_nrp(Nr),
+                                                        Nr, Nm);
+  count_launches(2);
   return cudaGetLastError();
 }
 
@@ -499,11 +672,17 @@ cudaError_t launch_gemm_adj_sl64(const void *A, const int8_t *ea, const cdd *Y, 
                                  int *eb, size_t eb_bytes, int *err, cudaStream_t s) {
   if (B <= 0) return cudaSuccess;
   const int P = sl64_tile(B), N = 2 * P, ntiles = (B + P - 1) / P, natoms = sl64_natoms(Nr);
-  const size_t b_stage = (size_t)NSL * N * 64;
-  if ((size_t)Nf * ntiles * natoms * b_stage > ws_bytes || (size_t)Nf * ntiles * P * sizeof(int) > eb_bytes)
+  const size_t b_stage = (size_t)NSL * N * 64, sl_bytes = (size_t)Nf * ntiles * natoms * b_stage;
+  const int nrp = sl64_nrp(Nr), ncols = ntiles * P;
+  const int ntl = (Nm + TM - 1) / TM, ngrp = (ncols + 63) / 64;
+  const size_t mag_bytes = (size_t)Nf * ncols * nrp * 2;
+  if (sl_bytes + mag_bytes + sizeof(int) * (1 + (size_t)Nf * ntl * ngrp) > ws_bytes || (size_t)Nf * ntiles * P * sizeof(int) > eb_bytes)
     return cudaErrorInvalidValue;
+  uint16_t *mag = reinterpret_cast<uint16_t *>(reinterpret_cast<uint8_t *>(ws) + sl_bytes);
+  int *todo = reinterpret_cast<int *>(reinterpret_cast<uint8_t *>(ws) + sl_bytes + mag_bytes);
   k_bsl64_build<<<dim3(Nf, ntiles), 256, 0, s>>>(Y, y_bstride, Nr, B, P, natoms,
-                                                 reinterpret_cast<uint8_t *>(ws), eb, ntiles);
+                                                 reinterpret_cast<uint8_t *>(ws), eb, mag, nrp, todo,
+                                                 ntiles);
   count_launches(1);
   const int chunk = Nr <= EXACT_ROWS ? natoms : CHUNK_ATOMS;
   int dev = 0, nsm = 0;
@@ -524,7 +703,10 @@ cudaError_t launch_gemm_adj_sl64(const void *A, const int8_t *ea, const cdd *Y, 
     case 24: run(std::integral_constant<int, 24>{}); break;
     default: run(std::integral_constant<int, 32>{}); break;
   }
-  count_launches(1);
+  k_adj_check<<<dim3((ntl + 63) / 64, Nf, ngrp), 128, 0, s>>>(sl64_low(ea, Nf, Nm), mag, nrp, Nr, ntl, B, ncols, todo);
+  k_adj_guard<<<(unsigned)std::max<long>(1, std::min<long>((long)Nf * ntl * ngrp, 2L * nsm)), 256, 0, s>>>(
+      reinterpret_cast<const float4 *>(A), ea, mag, nrp, Y, y_bstride, X, x_bstride, Nr, Nm, B, ncols, ntl, ngrp, todo);
+  count_launches(3);
   return cudaGetLastError();
 }
 

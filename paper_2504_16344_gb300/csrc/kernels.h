@@ -137,11 +137,12 @@ cudaError_t launch_gemm_adj_sl(const void *A, int fmt, const int8_t *ea, const c
 
 // ---- FP64-class adjoint product on the tensor cores (gemm_sl64.cu) --------
 // X[b][w][k] = sum_s conj(A[w][s][k]) Y[b][w][s] with float-pair operands cut
-// into seven exact bf16 slices; ea: the operator's row exponents
-// (launch_row_exp64); ws / eb: data-side slices and exponents, at least
+// into seven exact bf16 slices; ea: the operator's row exponents and what its
+// guard needs (launch_row_exp64, row_exp64_bytes); ws / eb: data-side slices and exponents, at least
 // sl64_ws_bytes / sl64_eb_bytes for bcols >= B columns
-size_t sl64_ws_bytes(int Nf, int Nr, int bcols);
+size_t sl64_ws_bytes(int Nf, int Nr, int Nm, int bcols);
 size_t sl64_eb_bytes(int Nf, int bcols);
+size_t row_exp64_bytes(int Nf, int Nr, int Nm);
 cudaError_t launch_row_exp64(const void *A, int8_t *ea, int Nf, int Nr, int Nm, cudaStream_t s);
 cudaError_t launch_gemm_adj_sl64(const void *A, const int8_t *ea, const cdd *Y, long y_bstride, cdd *X,
                                  long x_bstride, int Nf, int Nr, int Nm, int B, void *ws, size_t ws_bytes,

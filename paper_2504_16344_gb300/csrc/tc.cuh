@@ -236,4 +236,41 @@ __device__ __forceinline__ void tc_join_levels(const f2 *d, f2 &hi, f2 &lo) {
   lo = sub2(e, sub2(hi, s));
 }
 
+// ------------------------------------------- guards of the sliced products
+// A sum of n products of sliced operands is off by about sqrt(n) 2^-56 T (rms),
+// T the product of the two exponents' powers: the dropped levels and residues
+// are uniform over 2^-56 of the largest entries, however small the entries that
+// meet.  Double-float rounds such a sum at about 2^-47 of S, the sum of the
+// products' magnitudes.  A guard computes S (bf16 magnitudes rounded down, FP32
+// sums: a lower bound to a few percent) and has every sum with
+//   sqrt(n) 2^-56 T > 2^-47 S
+// formed again in double-float, so that no sum loses digits to the slices.  S = 0: every
+// product is zero, in slices as well.  A NaN or infinite S is taken again too.
+__device__ __forceinline__ bool tc_guard_fails(float S, float sqrt_n_T) {
+  return S != 0.f && !(512.f * S >= sqrt_n_T && S < __int_as_float(0x7f800000));
+}
+// C (16 x 8) += A (16 x 16) B (16 x 8), one warp, fragments in registers.  With
+// g = lane / 4, c = lane % 4 the 16 k are dealt out alike on both sides (a sum
+// does not mind): a[0], a[2] are row g, k 4c .. 4c+3, a[1], a[3] row g + 8; b[0],
+// b[1] column g, k 4c .. 4c+3; d[0], d[1] are (g, 2c), (g, 2c+1), d[2], d[3] row g + 8.
+// (Magnitudes take a hundredth of the slices' arithmetic: mma.sync from
+// registers, with nothing staged, keeps up with HBM.)
+__device__ __forceinline__ void tc_mma_mag(float *d, const uint32_t *a, const uint32_t *b) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+               "{%0,%1,%2,%3};"
+               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+// sum over the warp's lanes, the same bits in every lane (dd_add commutes)
+__device__ __forceinline__ dd tc_warp_sum(dd a) {
+#pragma unroll
+  for (int m = 16; m >= 1; m >>= 1) {
+    dd o;
+    o.hi = __shfl_xor_sync(0xffffffffu, a.hi, m);
+    o.lo = __shfl_xor_sync(0xffffffffu, a.lo, m);
+    a = dd_add(a, o);
+  }
+  return a;
+}
+
 }  // namespace tw

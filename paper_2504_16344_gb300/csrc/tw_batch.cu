@@ -262,7 +262,7 @@ size_t lane_bytes(const tw_ctx *c, int bmax) {
     b += 2 * B * np * sizeof(dd) + sl_ws_bytes(c->Nf, c->Rmax, cols) + sl_eb_bytes(c->Nf, cols);
   }
   if (c->trsm_eb) b += trsm_tc_ws_bytes(bmax);
-  if (c->ea64) b += sl64_ws_bytes(c->Nf, c->Nd, bmax) + sl64_eb_bytes(c->Nf, bmax) + (size_t)c->Nf * bmax;
+  if (c->ea64) b += sl64_ws_bytes(c->Nf, c->Nd, c->Nm, bmax) + sl64_eb_bytes(c->Nf, bmax) + (size_t)c->Nf * bmax;
   return b;
 }
 
@@ -310,7 +310,7 @@ tw_status alloc_lane(tw_ctx *c, tw_lane &L, int bmax) {
     L.trsm_ws = twh::dalloc(c, L.trsm_ws_n);
   }
   if (ok && c->ea64) {                // optional: null leaves the SIMT product
-    L.sl64_ws_n = sl64_ws_bytes(c->Nf, c->Nd, bmax);
+    L.sl64_ws_n = sl64_ws_bytes(c->Nf, c->Nd, c->Nm, bmax);
     L.sl64_eb_n = sl64_eb_bytes(c->Nf, bmax);
     L.sl64_eb = (int *)twh::dalloc(c, L.sl64_eb_n);
     if (L.sl64_eb) L.sl64_ws = twh::dalloc(c, L.sl64_ws_n);
@@ -379,7 +379,7 @@ tw_status tw_reserve_batch(tw_ctx *c, int bmax) {
   // optional as well: exponents of the operators that the sliced products read;
   // without them those products run on the FP32 pipes
   if (c->op[TW_MAP_F][TW_PREC_FP64]) {
-    c->ea64 = (int8_t *)twh::dalloc(c, (size_t)c->Nf * c->Nm);
+    c->ea64 = (int8_t *)twh::dalloc(c, row_exp64_bytes(c->Nf, c->Nd, c->Nm));
     for (int which = 0; which < 2; ++which)
       c->ef[which] = (int8_t *)twh::dalloc(c, (size_t)c->Nf * (which == TW_MAP_F ? c->Nd : c->Nq));
   }
