@@ -30,7 +30,8 @@ struct tw_lane {
   void *sl64_ws = nullptr;
   int *sl64_eb = nullptr;
   size_t sl64_ws_n = 0, sl64_eb_n = 0;
-  int8_t *sl64_ex = nullptr;         // [Nf][bmax] exponents of x^ (gemm_fwd_sl64.cu)
+  void *sl64_fx = nullptr;           // the forward product's (gemm_fwd_sl64.cu)
+  size_t sl64_fx_n = 0;
   // z slices of the solves' panel updates (trsm_tc.cu); null: the sweeps run
   // as one SIMT launch
   void *trsm_ws = nullptr;

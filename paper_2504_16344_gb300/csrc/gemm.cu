@@ -375,11 +375,7 @@ cudaError_t launch_gemm_fwd_dd(const void *A, const cdd *X, long x_bstride, cdd 
   if (B <= 0) return cudaSuccess;
   cudaError_t e = gemm_fwd_pick<cdd, 32, FMT_DD>(A, X, x_bstride, part, Nf, Nr, Nm, B, lpb, s);
   if (e != cudaSuccess) return e;
-  return launch_gemm_fwd_reduce_dd(part, Yo, y_bstride, gemm_fwd_nchunk(Nm), Nf, Nr, B, s);
-}
-
-cudaError_t launch_gemm_fwd_reduce_dd(const cdd *part, cdd *Yo, long y_bstride, int nchunk, int Nf, int Nr, int B,
-                                      cudaStream_t s) {
+  const int nchunk = gemm_fwd_nchunk(Nm);
   const long total = (long)B * Nf * Nr;
   k_gemm_fwd_reduce_dd<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(part, Yo, y_bstride, nchunk,
                                                                       Nf, Nr, B);

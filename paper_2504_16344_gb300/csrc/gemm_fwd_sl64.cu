@@ -13,12 +13,16 @@
 // forecast points leave the 128 rows of FM mostly empty.
 //
 // Accuracy.  Every row of F^ and of X^ has one power-of-two exponent per
-// frequency, over the whole grid (F^: once per load; X^: k_xexp, one pass per
-// call); slices, levels and exact accumulation as in gemm_sl64.cu.  The level
-// sums are exact over chunks of 96 grid points (K' = 192); the chunks of a
-// range of 4128 grid points are added in double-float in shared memory, the
-// ranges in a fixed order by k_gemm_fwd_reduce_dd.  The SIMT product rounds
-// its running sum after every one of the 2 Nm terms.
+// frequency and range of 4128 grid points (k_row_scan; F^: once per load; X^: one
+// pass per call); slices, levels and exact accumulation as in gemm_sl64.cu.  The
+// level sums are exact over chunks of 96 grid points (K' = 192); the chunks of a
+// range are added in double-float in shared memory, the
+// ranges in a fixed order by k_fwd_join.  The SIMT product rounds its running sum
+// after every one of the 2 Nm terms.  A field that is large where a row of F^ is small
+// leaves fewer digits to their sum than double-float does; such sums are found from
+// their magnitudes, bounded from below per 32 grid points for every frequency
+// (k_fwd_check) and formed in full for those that this leaves open (k_fwd_mag), and
+// taken again in double-float (k_fwd_join).
 //
 // What bounds it.  The SIMT form (gemm.cu) spends about 60 FP32 operations on
 // an entry and right-hand side.  Here 28 MMAs of 128 x N x 16 serve 8 grid
@@ -62,25 +66,213 @@ __device__ __forceinline__ void note(int *err, volatile int *fail, int info) {
   *fail = 1;
 }
 
-// e[w][r] (or e[w][b]): exponent of one row of Nm complex entries; row y of
-// frequency x = blockIdx.x starts at A + x * ws + y * rs, its exponent is e[x es + y]
+// One pass over rows of Nm complex entries, row y of frequency x = blockIdx.x from
+// A + x * ws + y * rs, range z = blockIdx.z of it: its exponent e[(x nrange + z) es +
+// y], and for the guard one bf16 value (rounded down) per block of 32 entries, blk[(x
+// es + y) nbp + i]: the least |Re| + |Im| of the block (LOW: the operator) or their
+// sum (the data)
+template <bool LOW>
 __global__ void __launch_bounds__(256)
-k_rowmax_exp(const float4 *__restrict__ A, long ws, long rs, int Nm, int8_t *__restrict__ e, int es) {
+k_row_scan(const float4 *__restrict__ A, long ws, long rs, int Nm, int8_t *__restrict__ e, int es,
+           uint16_t *__restrict__ blk, int nbp) {
   __shared__ float red[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rg = blockIdx.z;
+  const int kb = rg * RANGE, kend = min(Nm, kb + RANGE);
   const float4 *p = A + (long)blockIdx.x * ws + (long)blockIdx.y * rs;
+  uint16_t *out = blk + ((size_t)blockIdx.x * es + blockIdx.y) * nbp;
   float mx = 0.f;
-#pragma unroll 4
-  for (int k = threadIdx.x; k < Nm; k += 256) {
-    const float4 v = __ldg(p + k);
-    mx = fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.z)));
+  for (int k0 = kb + 128 * warp; k0 < kend; k0 += 1024) {
+    float s[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int k = k0 + 32 * j + lane;
+      s[j] = LOW ? __int_as_float(0x7f800000) : 0.f;
+      if (k < kend) {
+        const float4 v = __ldg(p + k);
+        mx = fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.z)));
+        s[j] = fabsf(v.x) + fabsf(v.z);
+      }
+    }
+    // four values a lane over 32 lanes: block j ends in the lanes whose bits 4 and 3 are j's bits 0 and 1
+    auto join = [](float a, float b) { return LOW ? fminf(a, b) : a + b; };
+    auto halve = [&](float lo, float hi, int m) {
+      const float keep = lane & m ? hi : lo;
+      return join(keep, __shfl_xor_sync(0xffffffffu, lane & m ? lo : hi, m));
+    };
+    float r = halve(halve(s[0], s[1], 16), halve(s[2], s[3], 16), 8);
+#pragma unroll
+    for (int m = 4; m >= 1; m >>= 1) r = join(r, __shfl_xor_sync(0xffffffffu, r, m));
+    const int i = k0 / 32 + (lane >> 4) + 2 * ((lane >> 3) & 1);
+    if ((lane & 7) == 0 && 32 * i < kend) out[i] = (uint16_t)(__float_as_uint(r) >> 16);
   }
+  if (kend == Nm)
+    for (int i = (Nm + 31) / 32 + threadIdx.x; i < nbp; i += 256) out[i] = 0;
 #pragma unroll
   for (int m = 16; m >= 1; m >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, m));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+  if (lane == 0) red[warp] = mx;
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int i = 1; i < 8; ++i) mx = fmaxf(mx, red[i]);
-    e[(size_t)blockIdx.x * es + blockIdx.y] = (int8_t)tc_exp_above(mx);
+    e[((size_t)blockIdx.x * gridDim.z + rg) * es + blockIdx.y] = (int8_t)tc_exp_above(mx);
+  }
+}
+
+// ------------------------------------------------------ the guard (tc.cuh)
+// sqrt(n) T of a row and a column: root of the sum of n T^2 over the ranges, n = 2
+// entries a point; er, eb: their exponents in range 0, strides sr, sb
+__device__ __forceinline__ float guard_scale(int Nm, int nrange, const int8_t *er, int sr, const int8_t *eb, int sb) {
+  int top = -1000;
+  for (int g = 0; g < nrange; ++g) top = max(top, (int)er[(size_t)g * sr] + (int)eb[(size_t)g * sb]);
+  float t = 0.f;
+  for (int g = 0; g < nrange; ++g)
+    t += scalbnf(2.f * (float)min(RANGE, Nm - g * RANGE), 2 * ((int)er[(size_t)g * sr] + (int)eb[(size_t)g * sb] - top));
+  return scalbnf(sqrtf(t), top);
+}
+
+// open[w] = 1 if the blocks' bound sum_i low F^ x (sum of |X^|) leaves some sum of
+// this frequency unsettled.  A CTA takes 16 rows and 64 columns, its warps the
+// blocks in turn
+__global__ void __launch_bounds__(256)
+k_fwd_check(const int8_t *__restrict__ ef, const uint16_t *__restrict__ low, const int8_t *__restrict__ ex,
+            const uint16_t *__restrict__ xsum, int nbp, int nrange, int Nr, int Nm, int B, int *__restrict__ open) {
+  __shared__ float sS[8][16][65], sM[8][64];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+  const int w = blockIdx.y, col0 = blockIdx.z * 64, r0 = blockIdx.x * 16, nf = min(8, (B - col0 + 7) / 8);
+  const uint16_t *la = low + ((size_t)w * Nr + min(r0 + g, Nr - 1)) * nbp + 4 * c;
+  const uint16_t *lb = low + ((size_t)w * Nr + min(r0 + g + 8, Nr - 1)) * nbp + 4 * c;
+  float S[8][4] = {}, M[8][4] = {};
+  for (int s = 16 * warp; s < nbp; s += 128) {
+    const uint2 p = __ldg(reinterpret_cast<const uint2 *>(la + s)), q = __ldg(reinterpret_cast<const uint2 *>(lb + s));
+    const uint32_t a[4] = {p.x, q.x, p.y, q.y}, one[4] = {0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u};
+#pragma unroll
+    for (int f = 0; f < 8; ++f)
+      if (f < nf) {
+        const int b = min(col0 + 8 * f + g, B - 1);
+        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(xsum + ((size_t)w * B + b) * nbp + 4 * c + s));
+        const uint32_t bb[2] = {v.x, v.y};
+        tc_mma_mag(S[f], a, bb);
+        tc_mma_mag(M[f], one, bb);                         // zero: an empty column
+      }
+  }
+#pragma unroll
+  for (int f = 0; f < 8; ++f)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      sS[warp][g + 8 * (i >> 1)][8 * f + 2 * c + (i & 1)] = S[f][i];
+      if (g == 0 && i < 2) sM[warp][8 * f + 2 * c + i] = M[f][i];
+    }
+  __syncthreads();
+  for (int t = threadIdx.x; t < 1024; t += 256) {
+    const int rl = t >> 6, bl = t & 63, r = r0 + rl, b = col0 + bl;
+    if (r >= Nr || b >= B) continue;
+    float v = 0.f, m = 0.f;
+    for (int k = 0; k < 8; ++k) { v += sS[k][rl][bl]; m += sM[k][bl]; }
+    if (m != 0.f && (v == 0.f || tc_guard_fails(v, guard_scale(Nm, nrange, ef + (size_t)w * nrange * Nr + r, Nr,
+                                                               ex + (size_t)w * nrange * B + b, B))))
+      open[w] = 1;
+  }
+}
+
+// Sp[w][range][r][b] = sum_k |F^[r][k]| |X^[b][k]| over a range of grid points, of
+// the open frequencies: 32 rows and 32 columns a CTA, whose warps take 16 points
+// in turn, straight from both operands.  Bound by their second reading.
+__global__ void __launch_bounds__(256, 2)
+k_fwd_mag(const float4 *__restrict__ F, const float4 *__restrict__ X, long xs, const int *__restrict__ open, int nrt,
+          int nbt, int nrange, int Nr, int Nm, int B, float *__restrict__ Sp) {
+  const int w = blockIdx.y;
+  if (!open[w]) return;
+  __shared__ float sh[8][32][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+  const int r0 = blockIdx.x % nrt * 32, b0 = blockIdx.x / nrt % nbt * 32, rg = blockIdx.x / (nrt * nbt);
+  const int kend = min(Nm, (rg + 1) * RANGE);
+  float d[2][4][4] = {};
+  for (int k = rg * RANGE + 16 * warp + c; k - c < kend; k += 128) {
+    // four entries' magnitudes, zero past the range (a lane's k are c, c + 4, .. on
+    // both sides: a load instruction takes 64 bytes in a row)
+    auto quad = [&](const float4 *row, uint32_t *o) {
+      float m[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float4 v = __ldg(row + min(k + 4 * j, kend - 1));
+        m[j] = k + 4 * j < kend ? fabsf(v.x) + fabsf(v.z) : 0.f;
+      }
+      o[0] = tc_pack_bf16(m[0], m[1]);
+      o[1] = tc_pack_bf16(m[2], m[3]);
+    };
+    uint32_t bq[4][2];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) quad(X + (long)min(b0 + 8 * f + g, B - 1) * xs + (long)w * Nm, bq[f]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      uint32_t lo[2], hi[2];
+      quad(F + ((long)w * Nr + min(r0 + 16 * h + g, Nr - 1)) * Nm, lo);
+      quad(F + ((long)w * Nr + min(r0 + 16 * h + g + 8, Nr - 1)) * Nm, hi);
+      const uint32_t a[4] = {lo[0], hi[0], lo[1], hi[1]};
+#pragma unroll
+      for (int f = 0; f < 4; ++f) tc_mma_mag(d[h][f], a, bq[f]);
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) sh[warp][16 * h + g + 8 * (i >> 1)][8 * f + 2 * c + (i & 1)] = d[h][f][i];
+  __syncthreads();
+  for (int t = threadIdx.x; t < 1024; t += 256) {
+    const int r = t >> 5, b = t & 31;
+    if (r0 + r >= Nr || b0 + b >= B) continue;
+    float S = 0.f;
+    for (int v = 0; v < 8; ++v) S += sh[v][r][b];
+    Sp[(((size_t)w * nrange + rg) * Nr + r0 + r) * B + b0 + b] = S;
+  }
+}
+
+// Yo[b][w][r]: the ranges' partial sums in order; the sums of open frequencies that
+// fail the guard go on the list todo[1 ..], todo[0] of them
+__global__ void __launch_bounds__(256)
+k_fwd_join(const cdd *__restrict__ part, const int8_t *__restrict__ ef, const int8_t *__restrict__ ex,
+           const int *__restrict__ open, const float *__restrict__ Sp, cdd *__restrict__ Yo, long y_bstride,
+           int nrange, int Nf, int Nr, int Nm, int B, int *__restrict__ todo) {
+  const long i = (long)blockIdx.x * 256 + threadIdx.x;
+  if (i >= (long)B * Nf * Nr) return;
+  const int r = (int)(i % Nr), w = (int)(i / Nr % Nf), b = (int)(i / Nr / Nf);
+  const cdd *p = part + (size_t)(i / Nr) * nrange * Nr + r;
+  cdd acc = cdd_zero();
+  for (int c = 0; c < nrange; ++c) acc = cdd_add(acc, ld_cdd(p + (size_t)c * Nr));
+  st_cdd(Yo + (size_t)b * y_bstride + (size_t)w * Nr + r, acc);
+  if (!open[w]) return;
+  float S = 0.f;
+  for (int c = 0; c < nrange; ++c) S += Sp[(((size_t)w * nrange + c) * Nr + r) * B + b];
+  if (tc_guard_fails(S, guard_scale(Nm, nrange, ef + (size_t)w * nrange * Nr + r, Nr,
+                                    ex + (size_t)w * nrange * B + b, B)))
+    todo[1 + atomicAdd(todo, 1)] = (int)i;
+}
+
+// the listed sums in double-float, one CTA each
+__global__ void __launch_bounds__(256)
+k_fwd_redo(const cdd *__restrict__ F, const cdd *__restrict__ X, long xs, const int *__restrict__ todo,
+           cdd *__restrict__ Yo, long y_bstride, int Nf, int Nr, int Nm) {
+  __shared__ cdd sh[8];
+  const int lane = threadIdx.x & 31, ntodo = todo[0];
+  for (int it = blockIdx.x; it < ntodo; it += gridDim.x) {
+    const int i = todo[1 + it], r = i % Nr, w = i / Nr % Nf, b = i / Nr / Nf;
+    const cdd *f = F + ((size_t)w * Nr + r) * Nm, *x = X + (long)b * xs + (size_t)w * Nm;
+    cdd a[4] = {cdd_zero(), cdd_zero(), cdd_zero(), cdd_zero()};      // four chains in flight
+    for (int k = threadIdx.x; k < Nm; k += 1024)
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k + 256 * u < Nm) a[u] = cdd_add(a[u], cdd_mul(ld_cdd(f + k + 256 * u), ld_cdd(x + k + 256 * u)));
+    cdd y = cdd_add(cdd_add(a[0], a[1]), cdd_add(a[2], a[3]));
+    y.re = tc_warp_sum(y.re);
+    y.im = tc_warp_sum(y.im);
+    __syncthreads();                     // the item before is read
+    if (lane == 0) sh[threadIdx.x >> 5] = y;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int v = 1; v < 8; ++v) y = cdd_add(y, sh[v]);
+      st_cdd(Yo + (size_t)b * y_bstride + (size_t)w * Nr + r, y);
+    }
   }
 }
 
@@ -172,13 +364,15 @@ k_gemm_fwd_sl64(const float4 *__restrict__ F, const int8_t *__restrict__ ef, con
   auto n_row = [&](const Item &it, int q) {
     return XM ? f_row(it.w, it.nt * N + q) : x_row(it.w, it.nt * (N / 2) + q);
   };
+  auto x_exp = [&](const Item &it, int b) { return (int)ex[((size_t)it.w * nrange + it.rg) * B + b]; };
+  auto f_exp = [&](const Item &it, int r) { return (int)ef[((size_t)it.w * nrange + it.rg) * Nr + r]; };
   auto m_exp = [&](const Item &it, int q) {
     const int i = XM ? it.mt * 64 + q : it.mt * 128 + q;
-    return XM ? (i < B ? (int)ex[(size_t)it.w * B + i] : 0) : (i < Nr ? (int)ef[(size_t)it.w * Nr + i] : 0);
+    return XM ? (i < B ? x_exp(it, i) : 0) : (i < Nr ? f_exp(it, i) : 0);
   };
   auto n_exp = [&](const Item &it, int q) {
     const int i = XM ? it.nt * N + q : it.nt * (N / 2) + q;
-    return XM ? (i < Nr ? (int)ef[(size_t)it.w * Nr + i] : 0) : (i < B ? (int)ex[(size_t)it.w * B + i] : 0);
+    return XM ? (i < Nr ? f_exp(it, i) : 0) : (i < B ? x_exp(it, i) : 0);
   };
   auto copy16 = [&](uint32_t dst, const float4 *row, int k, int kend) {
     const bool in = row != nullptr && k < kend;
@@ -509,25 +703,57 @@ long stage_cost(int mtiles, int ntiles, int N) { return (long)mtiles * ntiles * 
 // ------------------------------------------------------------------ host side
 int gemm_fwd_sl64_nrange(int Nm) { return (Nm + RANGE - 1) / RANGE; }
 
+static int fwd_nbp(int Nm) { return ((Nm + 31) / 32 + 15) / 16 * 16; }
+static size_t up16(size_t n) { return (n + 15) / 16 * 16; }
+// a map's tables: row exponents, then (16-byte aligned) the guard's block minima
+size_t fwd_exp64_bytes(int Nf, int Nr, int Nm) {
+  return up16((size_t)Nf * gemm_fwd_sl64_nrange(Nm) * Nr) + (size_t)Nf * Nr * fwd_nbp(Nm) * sizeof(uint16_t);
+}
+static const uint16_t *fwd_low(const int8_t *ef, int Nf, int Nr, int Nm) {
+  return reinterpret_cast<const uint16_t *>(ef + up16((size_t)Nf * gemm_fwd_sl64_nrange(Nm) * Nr));
+}
 cudaError_t launch_fwd_exp64(const void *F, int8_t *ef, int Nf, int Nr, int Nm, int row0, int nrows,
                              cudaStream_t s) {
   if (nrows <= 0) return cudaSuccess;
-  k_rowmax_exp<<<dim3(Nf, nrows), 256, 0, s>>>(reinterpret_cast<const float4 *>(F) + (size_t)row0 * Nm, (long)Nr * Nm,
-                                               Nm, Nm, ef + row0, Nr);
+  const int nbp = fwd_nbp(Nm);
+  k_row_scan<true><<<dim3(Nf, nrows, gemm_fwd_sl64_nrange(Nm)), 256, 0, s>>>(reinterpret_cast<const float4 *>(F) + (size_t)row0 * Nm,
+                                                   (long)Nr * Nm, Nm, Nm, ef + row0, Nr,
+                                                   const_cast<uint16_t *>(fwd_low(ef, Nf, Nr, Nm)) + (size_t)row0 * nbp, nbp);
   count_launches(1);
   return cudaGetLastError();
 }
 
-// part[b][w][range][r] of the forward product for b < B; ef: launch_fwd_exp64,
-// ex: Nf * B bytes of workspace.  bmax (the reserved batch) fixes which operand
-// takes the MMA rows, so that a column's rounding does not depend on its batch
-cudaError_t launch_gemm_fwd_sl64(const void *F, const int8_t *ef, const cdd *X, long x_bstride, int8_t *ex,
-                                 cdd *part, int Nf, int Nr, int Nm, int B, int bmax, int *err, cudaStream_t s) {
+// per call: open frequencies and the number of sums on the list, exponents and block
+// sums of X^, magnitude sums, the list
+size_t gemm_fwd_sl64_ws_bytes(int Nf, int Nr, int Nm, int B) {
+  const size_t nr = gemm_fwd_sl64_nrange(Nm);
+  return up16((size_t)Nf * sizeof(int)) + up16(Nf * nr * B) + (size_t)Nf * B * fwd_nbp(Nm) * sizeof(uint16_t) +
+         Nf * nr * Nr * B * sizeof(float) + (1 + (size_t)Nf * Nr * B) * sizeof(int);
+}
+
+// Yo[b][w][r] for b < B; ef: launch_fwd_exp64; ws: gemm_fwd_sl64_ws_bytes(B).
+// bmax (the reserved batch) fixes which operand takes the MMA rows, so that a
+// column's rounding does not depend on its batch
+cudaError_t launch_gemm_fwd_sl64(const void *F, const int8_t *ef, const cdd *X, long x_bstride, void *ws,
+                                 size_t ws_bytes, cdd *part, cdd *Yo, long y_bstride, int Nf, int Nr, int Nm, int B,
+                                 int bmax, int *err, cudaStream_t s) {
   if (B <= 0) return cudaSuccess;
+  if (gemm_fwd_sl64_ws_bytes(Nf, Nr, Nm, B) > ws_bytes) return cudaErrorInvalidValue;
   const float4 *Xp = reinterpret_cast<const float4 *>(X), *Fp = reinterpret_cast<const float4 *>(F);
-  k_rowmax_exp<<<dim3(Nf, B), 256, 0, s>>>(Xp, Nm, x_bstride, Nm, ex, B);
-  count_launches(1);
-  const int nr = gemm_fwd_sl64_nrange(Nm);
+  const int nbp = fwd_nbp(Nm), nr = gemm_fwd_sl64_nrange(Nm);
+  uint8_t *wp = reinterpret_cast<uint8_t *>(ws);
+  int *open = reinterpret_cast<int *>(wp);
+  int8_t *ex = reinterpret_cast<int8_t *>(wp += up16((size_t)Nf * sizeof(int)));
+  uint16_t *xsum = reinterpret_cast<uint16_t *>(wp += up16((size_t)Nf * nr * B));
+  float *Sp = reinterpret_cast<float *>(wp += (size_t)Nf * B * nbp * sizeof(uint16_t));
+  int *todo = reinterpret_cast<int *>(wp + (size_t)Nf * nr * Nr * B * sizeof(float));
+  cudaError_t e = cudaMemsetAsync(open, 0, (size_t)Nf * sizeof(int), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(todo, 0, sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  k_row_scan<false><<<dim3(Nf, B, nr), 256, 0, s>>>(Xp, Nm, x_bstride, Nm, ex, B, xsum, nbp);
+  k_fwd_check<<<dim3((Nr + 15) / 16, Nf, (B + 63) / 64), 256, 0, s>>>(ef, fwd_low(ef, Nf, Nr, Nm), ex, xsum, nbp, nr, Nr,
+                                                                     Nm, B, open);
+  count_launches(2);
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -562,7 +788,13 @@ cudaError_t launch_gemm_fwd_sl64(const void *F, const int8_t *ef, const cdd *X, 
   };
   if (xm) pick(std::true_type{});
   else pick(std::false_type{});
-  count_launches(1);
+  const int nrt = (Nr + 31) / 32, nbt = (B + 31) / 32;
+  k_fwd_mag<<<dim3(nrt * nbt * nr, Nf), 256, 0, s>>>(Fp, Xp, x_bstride, open, nrt, nbt, nr, Nr, Nm, B, Sp);
+  k_fwd_join<<<(unsigned)(((long)B * Nf * Nr + 255) / 256), 256, 0, s>>>(part, ef, ex, open, Sp, Yo, y_bstride, nr, Nf,
+                                                                        Nr, Nm, B, todo);
+  k_fwd_redo<<<(unsigned)std::max(1, 4 * nsm), 256, 0, s>>>(reinterpret_cast<const cdd *>(F), X, x_bstride, todo, Yo,
+                                                           y_bstride, Nf, Nr, Nm);
+  count_launches(4);
   return cudaGetLastError();
 }
 

@@ -149,17 +149,18 @@ cudaError_t launch_gemm_adj_sl64(const void *A, const int8_t *ea, const cdd *Y, 
                                  int *eb, size_t eb_bytes, int *err, cudaStream_t s);
 
 // ---- FP64-class forward product on the tensor cores (gemm_fwd_sl64.cu) -----
-// partial sums of Yo[b][w][r] = sum_k F[w][r][k] X[b][w][k] per range of grid
-// points (gemm_fwd_sl64_nrange <= gemm_fwd_nchunk of them), to be added by
-// launch_gemm_fwd_reduce_dd; ef: [Nf][Nr] row exponents (launch_fwd_exp64: of rows row0 .. row0 + nrows-1), ex:
-// Nf * B bytes of workspace, bmax: the reserved batch
+// Yo[b][w][r] = sum_k F[w][r][k] X[b][w][k]; ef: the map's row exponents and what
+// its guard needs (launch_fwd_exp64 of rows row0 .. row0 + nrows-1, fwd_exp64_bytes);
+// part: partial sums per range of grid points (gemm_fwd_sl64_nrange <=
+// gemm_fwd_nchunk of them); ws: gemm_fwd_sl64_ws_bytes of B; bmax: the reserved batch
 int gemm_fwd_sl64_nrange(int Nm);
+size_t fwd_exp64_bytes(int Nf, int Nr, int Nm);
+size_t gemm_fwd_sl64_ws_bytes(int Nf, int Nr, int Nm, int B);
 cudaError_t launch_fwd_exp64(const void *F, int8_t *ef, int Nf, int Nr, int Nm, int row0, int nrows,
                              cudaStream_t s);
-cudaError_t launch_gemm_fwd_sl64(const void *F, const int8_t *ef, const cdd *X, long x_bstride, int8_t *ex,
-                                 cdd *part, int Nf, int Nr, int Nm, int B, int bmax, int *err, cudaStream_t s);
-cudaError_t launch_gemm_fwd_reduce_dd(const cdd *part, cdd *Yo, long y_bstride, int nchunk, int Nf, int Nr, int B,
-                                      cudaStream_t s);
+cudaError_t launch_gemm_fwd_sl64(const void *F, const int8_t *ef, const cdd *X, long x_bstride, void *ws,
+                                 size_t ws_bytes, cdd *part, cdd *Yo, long y_bstride, int Nf, int Nr, int Nm, int B,
+                                 int bmax, int *err, cudaStream_t s);
 
 // ---- operator storage conversion: dst[w][row0+r][k] from src (cdd) -----
 cudaError_t launch_convert_op(const cdd *src, long src_ld_w, void *dst, int fmt, long dst_ld_w,

@@ -81,14 +81,11 @@ static cudaError_t forward_dd(tw_ctx *c, tw_lane &L, int which, int B, cudaStrea
   const int Nf = c->Nf, Nr = which == TW_MAP_F ? c->Nd : c->Nq, Nm = c->Nm;
   const void *A = c->op[which][TW_PREC_FP64];
   const cdd *x = (const cdd *)L.bxh;
-  if (L.adj_rw != 0 || !c->ef[which] || !L.sl64_ex)
+  if (L.adj_rw != 0 || !c->ef[which] || !L.sl64_fx)
     return launch_gemm_fwd_dd(A, x, (long)Nf * Nm, (cdd *)L.bpart, (cdd *)L.byh, (long)Nf * Nr, Nf, Nr, Nm, B, s,
                               fwd_lpb(L));
-  cudaError_t e = launch_gemm_fwd_sl64(A, c->ef[which], x, (long)Nf * Nm, L.sl64_ex, (cdd *)L.bpart, Nf, Nr, Nm, B,
-                                       L.bmax, c->d_err, s);
-  if (e != cudaSuccess) return e;
-  return launch_gemm_fwd_reduce_dd((const cdd *)L.bpart, (cdd *)L.byh, (long)Nf * Nr, gemm_fwd_sl64_nrange(Nm), Nf,
-                                   Nr, B, s);
+  return launch_gemm_fwd_sl64(A, c->ef[which], x, (long)Nf * Nm, L.sl64_fx, L.sl64_fx_n, (cdd *)L.bpart, (cdd *)L.byh,
+                              (long)Nf * Nr, Nf, Nr, Nm, B, L.bmax, c->d_err, s);
 }
 
 // q = F_q m for B right-hand sides; rows t >= win[b] of m are taken as zero
@@ -262,14 +259,15 @@ size_t lane_bytes(const tw_ctx *c, int bmax) {
     b += 2 * B * np * sizeof(dd) + sl_ws_bytes(c->Nf, c->Rmax, cols) + sl_eb_bytes(c->Nf, cols);
   }
   if (c->trsm_eb) b += trsm_tc_ws_bytes(bmax);
-  if (c->ea64) b += sl64_ws_bytes(c->Nf, c->Nd, c->Nm, bmax) + sl64_eb_bytes(c->Nf, bmax) + (size_t)c->Nf * bmax;
+  if (c->ea64) b += sl64_ws_bytes(c->Nf, c->Nd, c->Nm, bmax) + sl64_eb_bytes(c->Nf, bmax) +
+                   gemm_fwd_sl64_ws_bytes(c->Nf, c->Rmax, c->Nm, bmax);
   return b;
 }
 
 void free_lane(tw_ctx *c, tw_lane &L) {
   void **bufs[] = {(void **)&L.win_dev, (void **)&L.trsm_prog, (void **)&L.bz, (void **)&L.by,
                    (void **)&L.bzd, (void **)&L.byd, (void **)&L.brd, &L.byh, &L.bxh, &L.bpart,
-                   &L.bsl_ws, (void **)&L.bsl_eb, &L.sl64_ws, (void **)&L.sl64_eb, &L.trsm_ws, (void **)&L.sl64_ex};
+                   &L.bsl_ws, (void **)&L.bsl_eb, &L.sl64_ws, (void **)&L.sl64_eb, &L.trsm_ws, &L.sl64_fx};
   for (void **b : bufs) { twh::dfree(c, *b); *b = nullptr; }
   L.bmax = 0;
   L.bytes = 0;
@@ -314,7 +312,8 @@ tw_status alloc_lane(tw_ctx *c, tw_lane &L, int bmax) {
     L.sl64_eb_n = sl64_eb_bytes(c->Nf, bmax);
     L.sl64_eb = (int *)twh::dalloc(c, L.sl64_eb_n);
     if (L.sl64_eb) L.sl64_ws = twh::dalloc(c, L.sl64_ws_n);
-    if (L.sl64_ws) L.sl64_ex = (int8_t *)twh::dalloc(c, (size_t)c->Nf * bmax);
+    L.sl64_fx_n = gemm_fwd_sl64_ws_bytes(c->Nf, c->Rmax, c->Nm, bmax);
+    if (L.sl64_ws) L.sl64_fx = twh::dalloc(c, L.sl64_fx_n);
   }
   if (!ok) {
     free_lane(c, L);
@@ -381,7 +380,7 @@ tw_status tw_reserve_batch(tw_ctx *c, int bmax) {
   if (c->op[TW_MAP_F][TW_PREC_FP64]) {
     c->ea64 = (int8_t *)twh::dalloc(c, row_exp64_bytes(c->Nf, c->Nd, c->Nm));
     for (int which = 0; which < 2; ++which)
-      c->ef[which] = (int8_t *)twh::dalloc(c, (size_t)c->Nf * (which == TW_MAP_F ? c->Nd : c->Nq));
+      c->ef[which] = (int8_t *)twh::dalloc(c, fwd_exp64_bytes(c->Nf, which == TW_MAP_F ? c->Nd : c->Nq, c->Nm));
   }
   tw_status st = twb::alloc_lane(c, c->lane, bmax);
   if (st != TW_OK) {

@@ -82,3 +82,39 @@ def test_adjoint_over_several_tiles_per_cta(Nd, B):
     for b in range(B):
         e = (m[0][b] - m[4][b]).norm() / m[4][b].norm()
         assert e < 2.0 ** -47 * (2 * Nd) ** 1.5, (b, float(e))
+
+
+# a forecast of fields that are large where the map is small.  Rows: X^ on the MMA
+# rows (16 and 32 columns), F^ on them (100 rows); grid points: two ranges, the
+# second of 32; columns: part of a tile and more than one
+@pytest.mark.parametrize("spread", [0, 24, 40])
+@pytest.mark.parametrize("Nq,B", [(2, 2), (20, 70), (100, 33)])
+def test_forward_of_wide_range(Nq, B, spread):
+    import torch
+    Nd, Nx, Ny, Nt = 2, 65, 64, 5
+    F, Fq, m = _randn(1, Nt, Nd, Nx * Ny), _randn(2, Nt, Nq, Nx * Ny), _randn(3, B, Nt, Nx * Ny)
+    Fq[:, 1:, 100:] *= 2.0 ** -spread                  # row 0 stays as it is
+    m[:, :, :100] *= 2.0 ** -spread
+    m[B - 1] = 0.0
+    tw, ctx = _context(Nd, Nx, Ny, Nt, B, F, Fq, 1e6 * Nx * Ny)
+    q = {}
+    for rw in (0, 4):
+        ctx.set_batch_tiles(8, rw, 1)
+        q[rw] = ctx.forecast_batch(tw.PREC_FP64, m)
+    ctx.set_batch_tiles(8, 0, 1)
+    one = ctx.forecast_batch(tw.PREC_FP64, m[:1].contiguous())
+    bad = m.clone()
+    bad[1, 0, 7] = float("nan")
+    mates = ctx.forecast_batch(tw.PREC_FP64, bad)
+    ctx.check()
+    ctx.close()
+    # n terms of random sign: running sums grow as sqrt(k), n independent roundings of
+    # 2^-48 of them come to sqrt(n / 2) 2^-48 of the result; four times that for each side
+    tol = 8 * 2.0 ** -48 * (2 * Nx * Ny) ** 0.5
+    for b in range(B - 1):
+        e = ((q[0][b] - q[4][b]).norm(dim=0) / q[4][b].norm(dim=0)).max()        # every forecast point by itself
+        assert e < tol, (b, float(e))
+    assert not q[0][B - 1].any()
+    assert torch.equal(one[0], q[0][0])
+    keep = [b for b in range(B) if b != 1]
+    assert torch.equal(mates[keep], q[0][keep]) and torch.isnan(mates[1]).all()
