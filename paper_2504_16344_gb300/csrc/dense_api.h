@@ -96,10 +96,10 @@ cudaError_t launch_trsm_dd_panel(const dd *Lx, const dd *Linv, const void *rhs, 
                                  cudaStream_t s);
 // the whole sweep in panels, the products between panels on the tensor cores
 // (trsm_tc.cu); ea: row exponents of Lx (launch_trsm_tc_exp, trsm_tc_exp_bytes
-// each); ws: trsm_tc_ws_bytes(B)
+// each); ws: trsm_tc_ws_bytes
 bool trsm_tc_applies(int NB, int bmax);
 size_t trsm_tc_exp_bytes(int NB);
-size_t trsm_tc_ws_bytes(int B);
+size_t trsm_tc_ws_bytes(int NB, int B);
 cudaError_t launch_trsm_tc_exp(const dd *Lf, const dd *Lb, int8_t *ef, int8_t *eb, int NB, cudaStream_t s);
 cudaError_t launch_trsm_dd_tc(const dd *Lx, const int8_t *ea, const dd *Linv, const void *rhs, int rhs_kind,
                               long rhs_bstride, dd *out, long out_bstride, const int *win, int Nd, int Nt, int B,

@@ -20,7 +20,10 @@
 // Accuracy.  As in gemm_sl64.cu: a row of the factor and a column of z have a
 // power-of-two exponent per chunk of 192 (three blocks), the level sums of a
 // chunk are exact, and chunks are added in double-float; k_trsm rounds its
-// running sum after every product.
+// running sum after every product.  Loud entries of z that meet small ones of the
+// factor leave fewer digits to a sum than double-float does: such sums are found from
+// their magnitudes (k_trsm_mag) and formed again in double-float before their row is
+// solved (k_trsm_redo).
 //
 // Panels are separate launches: the products need no flags, and the order of
 // every column's sum is fixed by the block rows alone, so a right-hand side
@@ -39,6 +42,7 @@ namespace {
 constexpr int PW = 12;                   // block rows per panel (a multiple of 6)
 constexpr int CB = 3;                    // blocks per exact chunk (192 k)
 constexpr int NCH = PW / CB;             // chunks per panel
+constexpr int PK = PW * NB_;             // k per panel
 constexpr int TM = 128;                  // MMA M: factor rows per tile
 constexpr int CH_ATOMS = CB * NB_ / 32;  // 32-wide atoms per chunk
 constexpr int ATOMS = NCH * CH_ATOMS;    // atoms per panel
@@ -87,19 +91,23 @@ k_upd_exp(const dd *__restrict__ Lx, int8_t *__restrict__ e, int NB) {
 }
 
 // ------------------------------------------------ slices of a panel's z
-// tiles [nt][chunk][atom][slice][N][32 bf16] (64-byte swizzle) and column
-// exponents ez[nt][chunk][N]; blocks at or past NB are zero.  grid (NCH, ntiles)
+// tiles [nt][chunk][atom][slice][N][32 bf16] (64-byte swizzle), column exponents
+// ez[nt][chunk][N] and magnitudes mag[nt][N][PK] (bf16, for the guard); blocks at or
+// past NB are zero.  grid (NCH, ntiles, tasks / 256): a CTA cuts 256 pieces of eight
+// entries, after the exponents of the columns they lie in
 __global__ void __launch_bounds__(256)
 k_zslice(const dd *__restrict__ z, long zs, int J0, int NB, int B, int N, uint8_t *__restrict__ tiles,
-         int *__restrict__ ez) {
+         int *__restrict__ ez, uint16_t *__restrict__ mag) {
   __shared__ int e_sh[NMAX];
   const int c = blockIdx.x, nt = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long k0 = (long)(J0 + c * CB) * NB_, kend = min((long)NB * NB_, k0 + CB * NB_);
-  for (int n = warp; n < N; n += 8) {
+  const int t = blockIdx.z * 256 + threadIdx.x, per_col = 4 * CH_ATOMS;
+  for (int n = blockIdx.z * 256 / per_col + warp; n <= (int)(blockIdx.z * 256 + 255) / per_col && n < N; n += 8) {
     const int b = nt * N + n;
     float mx = 0.f;
     if (b < B)
+#pragma unroll
       for (long k = k0 + lane; k < kend; k += 32) mx = fmaxf(mx, fabsf(z[(long)b * zs + k].hi));
 #pragma unroll
     for (int m = 16; m >= 1; m >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, m));
@@ -111,19 +119,23 @@ k_zslice(const dd *__restrict__ z, long zs, int J0, int NB, int B, int N, uint8_
   __syncthreads();
   const size_t slice_bytes = (size_t)N * 64;
   uint8_t *base = tiles + (size_t)(nt * NCH + c) * CH_ATOMS * NSL * slice_bytes;
-  for (int t = threadIdx.x; t < CH_ATOMS * N * 4; t += blockDim.x) {
+  if (t < CH_ATOMS * N * 4) {
     // consecutive threads take consecutive 8-entry pieces of a column
     const int q = t & 3, a = (t >> 2) % CH_ATOMS, n = t / (4 * CH_ATOMS), b = nt * N + n;
     const long k = k0 + 32 * a + 8 * q;
     const float sc1 = tc_pow2f(7 - e_sh[n]);
     const f2 sc = f2_make(sc1, sc1);
     Slicer7 sl[4];
+    uint32_t mg[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);      // two entries (k is a multiple of 8)
       if (b < B && k < kend) v = *reinterpret_cast<const float4 *>(z + (long)b * zs + k + 2 * u);
       sl[u].init(v.x, v.y, v.z, v.w, sc);
+      mg[u] = tc_pack_bf16(fabsf(v.x), fabsf(v.z));
     }
+    *reinterpret_cast<uint4 *>(mag + (size_t)(nt * N + n) * PK + c * CB * NB_ + 32 * a + 8 * q) =
+        make_uint4(mg[0], mg[1], mg[2], mg[3]);
     uint8_t *at = base + (size_t)a * NSL * slice_bytes + tc_swz64(n, q);
     auto put = [&](auto S) {
       uint32_t wd[4];
@@ -132,6 +144,155 @@ k_zslice(const dd *__restrict__ z, long zs, int J0, int NB, int B, int N, uint8_
       *reinterpret_cast<uint4 *>(at + S.value * slice_bytes) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
     };
     for_slices7(put);
+  }
+}
+
+// ------------------------------------------------ the guard (tc.cuh)
+// A row's sum runs over all panels before it, so it is judged when its own panel
+// is due: se[nt][row][N] holds S and (a bound of) the root of the sum of 192 T^2 so
+// far.  S is
+// taken from 16 of every 64 k, a quarter of the factor: a lower bound still, and one
+// that settles all but a few sums in a thousand (first and last panels apart; panel
+// by panel, a tenth to a half of the early panels' sums stayed open).  A CTA takes
+// 16 rows and N columns, each of its four warps three of the panel's blocks and a
+// quarter of the columns' ends: a panel's latency counts more than its reads.
+template <bool FWD>
+__global__ void __launch_bounds__(128)
+k_trsm_mag(const dd *__restrict__ Lx, const int8_t *__restrict__ ea, const uint16_t *__restrict__ mag,
+           const int *__restrict__ ez, float2 *__restrict__ se, const int *__restrict__ win, int Nd, int Nt, int B,
+           int N, int J0, int row0, int NB) {
+  __shared__ float4 part[4][8][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+  const int nmax = max_rows(win, B, Nd, Nt), nt = blockIdx.y;
+  const int i0 = row0 + blockIdx.x * 16;                   // 16 rows of one block row
+  if ((long)J0 * NB_ >= nmax || i0 >= nmax) return;
+  const int ia = i0 + g, I = ia >> 6, nf = N / 8;
+  const uint16_t *mw = mag + (size_t)(nt * N + g) * PK + 4 * c;
+  float d[8][4] = {};
+#pragma unroll
+  for (int jj = 0; jj < PW / 4; ++jj) {
+    const int J = J0 + warp * (PW / 4) + jj;
+    if (J >= NB) continue;
+    const dd *blk = Lx + (FWD ? packed_index(I, J) : packed_index(J, I)) * NB_ * NB_;
+    const int k0 = 16 * (J & 3), k = k0 + 4 * c;
+    float r[2][4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = (ia & 63) + 8 * h;
+      if (FWD) {
+        const float4 *p = reinterpret_cast<const float4 *>(blk + i * NB_ + k);
+        const float4 u = __ldg(p), v = __ldg(p + 1);
+        r[h][0] = fabsf(u.x), r[h][1] = fabsf(u.z), r[h][2] = fabsf(v.x), r[h][3] = fabsf(v.z);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) r[h][j] = fabsf(__ldg(&blk[(k + j) * NB_ + i].hi));
+      }
+    }
+    const uint32_t a[4] = {tc_pack_bf16(r[0][0], r[0][1]), tc_pack_bf16(r[1][0], r[1][1]),
+                           tc_pack_bf16(r[0][2], r[0][3]), tc_pack_bf16(r[1][2], r[1][3])};
+#pragma unroll
+    for (int f = 0; f < 8; ++f)
+      if (f < nf) {
+        const uint2 q = __ldg(reinterpret_cast<const uint2 *>(mw + (size_t)(8 * f) * PK + (J - J0) * NB_ + k0));
+        const uint32_t b[2] = {q.x, q.y};
+        tc_mma_mag(d[f], a, b);
+      }
+  }
+#pragma unroll
+  for (int f = 0; f < 8; ++f) part[warp][f][lane] = make_float4(d[f][0], d[f][1], d[f][2], d[f][3]);
+  __syncthreads();
+  int er[2][NCH];
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int q = 0; q < NCH; ++q) er[h][q] = __ldg(ea + (size_t)(J0 / CB + q) * NB * NB_ + ia + 8 * h);
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int f = 2 * warp + u, n = 8 * f + 2 * c;
+    if (f >= nf) break;
+    float S[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const float4 q = part[v][f][lane];
+      S[0] += q.x, S[1] += q.y, S[2] += q.z, S[3] += q.w;
+    }
+    int ec[2][NCH];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int q = 0; q < NCH; ++q) ec[i][q] = __ldg(ez + (nt * NCH + q) * N + n + i);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float4 *p = reinterpret_cast<float4 *>(se + ((size_t)nt * NB * NB_ + ia + 8 * h) * N + n);
+      float4 o = *p;
+      o.x += S[2 * h];
+      o.z += S[2 * h + 1];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        int top = -1000;
+#pragma unroll
+        for (int q = 0; q < NCH; ++q) top = max(top, er[h][q] + ec[i][q]);
+        // four chunks of 192: at most 2 sqrt(192) times the largest T; added in quadrature, rounded up
+        const float t = top > 120 ? __int_as_float(0x7f800000) : 2.f * 13.8565f * tc_pow2f(max(top, -126));
+        float &E = i ? o.w : o.y;
+        const float hi = fmaxf(E, t), r = __fdividef(fminf(E, t), hi);
+        E = hi * (1.f + 0.5f * r * r);
+      }
+      *p = o;
+    }
+  }
+}
+
+// before panel I0 .. I1-1 is solved: its rows' sums that fail are formed in double-float
+// over all k before the panel (FWD: below I0, else from I1 up), a CTA each
+template <bool FWD>
+__global__ void __launch_bounds__(256)
+k_trsm_redo(const dd *__restrict__ Lx, const float2 *__restrict__ se, dd *__restrict__ out, long zs,
+            const int *__restrict__ win, int Nd, int Nt, int B, int N, int I0, int I1, int NB) {
+  __shared__ int list[256], count;
+  __shared__ dd sh[8];
+  const int lane = threadIdx.x & 31, nmax = max_rows(win, B, Nd, Nt);
+  const int kb = FWD ? 0 : I1 * NB_, ke = FWD ? I0 * NB_ : min(NB * NB_, (nmax + NB_ - 1) / NB_ * NB_);
+  const int rows = min((I1 - I0) * NB_, nmax - I0 * NB_);
+  const long pairs = ke > kb && rows > 0 ? (long)rows * B : 0;
+  for (long p0 = blockIdx.x; p0 < pairs; p0 += 256L * gridDim.x) {
+    if (threadIdx.x == 0) count = 0;
+    __syncthreads();
+    const long p = p0 + (long)gridDim.x * threadIdx.x;     // a column's rows go to different CTAs
+    if (p < pairs) {
+      const int b = (int)(p / rows), row = I0 * NB_ + (int)(p % rows);
+      const float2 v = se[((size_t)(b / N) * NB * NB_ + row) * N + b % N];
+      // the sum itself bounds S as well: where a few k make most of it, the sample may
+      // miss them, but they hardly cancel
+      const float S = fmaxf(v.x, fabsf(out[(long)b * zs + row].hi));
+      if (row < Nd * min(max(__ldg(win + b), 0), Nt) && tc_guard_fails(S, v.y)) list[atomicAdd(&count, 1)] = threadIdx.x;
+    }
+    __syncthreads();
+    const int n = count;
+    for (int q = 0; q < n; ++q) {
+      const long pq = p0 + (long)gridDim.x * list[q];
+      const int b = (int)(pq / rows), row = I0 * NB_ + (int)(pq % rows), I = row >> 6;
+      const dd *zb = out + (long)b * zs;
+      dd a[4] = {dd_zero(), dd_zero(), dd_zero(), dd_zero()};      // four chains in flight
+      for (int k = kb + threadIdx.x; k < ke; k += 1024)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int kk = k + 256 * u, J = kk >> 6;
+          if (kk >= ke) continue;
+          const dd *blk = Lx + (FWD ? packed_index(I, J) : packed_index(J, I)) * NB_ * NB_;
+          a[u] = dd_add(a[u], dd_mul(FWD ? blk[(row & 63) * NB_ + (kk & 63)] : blk[(kk & 63) * NB_ + (row & 63)], zb[kk]));
+        }
+      const dd y = tc_warp_sum(dd_add(dd_add(a[0], a[1]), dd_add(a[2], a[3])));
+      __syncthreads();                   // the sum before is read
+      if (lane == 0) sh[threadIdx.x >> 5] = y;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        dd x = sh[0];
+        for (int v = 1; v < 8; ++v) x = dd_add(x, sh[v]);
+        out[(long)b * zs + row] = x;
+      }
+    }
+    __syncthreads();                     // the list is read
   }
 }
 
@@ -502,10 +663,13 @@ bool trsm_tc_applies(int NB, int bmax) { return NB > 2 * PW && (long)((bmax + 1)
 
 static int exp_chunks(int NB) { return (NB + PW - 1) / PW * NCH; }   // whole panels
 size_t trsm_tc_exp_bytes(int NB) { return (size_t)exp_chunks(NB) * NB * NB_; }
-// slices, then exponents, of one panel for at most B right-hand sides (tiles
-// hold fewer than 16 unused columns each)
+// for at most B right-hand sides (tiles hold fewer than 16 unused columns each): one
+// panel's slices, magnitudes and exponents, and the guard's sums per row
 static size_t z_cols(int B) { return (size_t)B + 16 * ((B + NMAX - 1) / NMAX); }
-size_t trsm_tc_ws_bytes(int B) { return z_cols(B) * (ATOMS * NSL * 64 + NCH * sizeof(int)); }
+size_t trsm_tc_ws_bytes(int NB, int B) {
+  return z_cols(B) *
+         (ATOMS * NSL * 64 + PK * sizeof(uint16_t) + NCH * sizeof(int) + (size_t)NB * NB_ * sizeof(float2));
+}
 
 cudaError_t launch_trsm_tc_exp(const dd *Lf, const dd *Lb, int8_t *ef, int8_t *eb, int NB, cudaStream_t s) {
   const dim3 grid(NB, exp_chunks(NB));
@@ -515,23 +679,41 @@ cudaError_t launch_trsm_tc_exp(const dd *Lf, const dd *Lb, int8_t *ef, int8_t *e
   return cudaGetLastError();
 }
 
-// one panel's update of the rows past it; ws: trsm_tc_ws_bytes(B)
+struct PanelWs {
+  uint8_t *slices;
+  uint16_t *mag;
+  int *ez;
+  float2 *se;
+  size_t se_bytes;
+};
+static PanelWs panel_ws(void *ws, int NB, int B) {
+  const size_t cols = (size_t)tile_count(B) * tile_cols(B);
+  PanelWs p;
+  p.slices = reinterpret_cast<uint8_t *>(ws);
+  p.mag = reinterpret_cast<uint16_t *>(p.slices + cols * ATOMS * NSL * 64);
+  p.ez = reinterpret_cast<int *>(p.mag + cols * PK);
+  p.se = reinterpret_cast<float2 *>(p.ez + cols * NCH);
+  p.se_bytes = cols * NB * NB_ * sizeof(float2);
+  return p;
+}
+
+// one panel's update of the rows past it
 template <bool FWD>
 static cudaError_t update_panel(const dd *Lx, const int8_t *ea, dd *out, long zs, const int *win, int Nd, int Nt,
-                                int B, int NB, int J0, uint8_t *ws, int nsm, int *err, cudaStream_t s) {
+                                int B, int NB, int J0, const PanelWs &ws, int nsm, int *err, cudaStream_t s) {
   const int J1 = std::min(NB, J0 + PW);
   const int row0 = FWD ? J1 * NB_ : 0;
   const int nrt = FWD ? ((NB - J1) * NB_ + TM - 1) / TM : J0 * NB_ / TM;
   if (nrt <= 0) return cudaSuccess;
   const int N = tile_cols(B), ntiles = tile_count(B);
-  int *ez = reinterpret_cast<int *>(ws + (size_t)ntiles * N * ATOMS * NSL * 64);
-  k_zslice<<<dim3(NCH, ntiles), 256, 0, s>>>(out, zs, J0, NB, B, N, ws, ez);
-  count_launches(1);
+  k_zslice<<<dim3(NCH, ntiles, (4 * CH_ATOMS * N + 255) / 256), 256, 0, s>>>(out, zs, J0, NB, B, N, ws.slices, ws.ez, ws.mag);
+  k_trsm_mag<FWD><<<dim3(((FWD ? NB - J1 : J0) * NB_) / 16, ntiles), 128, 0, s>>>(Lx, ea, ws.mag, ws.ez, ws.se, win, Nd, Nt, B, N, J0, row0, NB);
+  count_launches(2);
   const int grid = std::min(nrt * ntiles, nsm);
   auto run = [&](auto NC) {
     constexpr int NN = NC.value;
     cudaFuncSetAttribute(k_trsm_upd<NN, FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<NN>::smem);
-    k_trsm_upd<NN, FWD><<<grid, NTHR, Cfg<NN>::smem, s>>>(Lx, ea, ws, ez, out, zs, win, Nd, Nt, B, ntiles, J0,
+    k_trsm_upd<NN, FWD><<<grid, NTHR, Cfg<NN>::smem, s>>>(Lx, ea, ws.slices, ws.ez, out, zs, win, Nd, Nt, B, ntiles, J0,
                                                           row0, nrt, NB, err);
   };
   switch (N) {
@@ -540,7 +722,11 @@ static cudaError_t update_panel(const dd *Lx, const int8_t *ea, dd *out, long zs
     case 48: run(std::integral_constant<int, 48>{}); break;
     default: run(std::integral_constant<int, 64>{}); break;
   }
-  count_launches(1);
+  // the next panel's rows have all their products now
+  const int p0 = FWD ? J1 : J0 - PW, p1 = FWD ? std::min(NB, J1 + PW) : J0;
+  k_trsm_redo<FWD><<<(unsigned)std::min<long>((long)(p1 - p0) * NB_ * B, 4L * nsm), 256, 0, s>>>(
+      Lx, ws.se, out, zs, win, Nd, Nt, B, N, p0, p1, NB);
+  count_launches(2);
   return cudaGetLastError();
 }
 
@@ -549,12 +735,14 @@ cudaError_t launch_trsm_dd_tc(const dd *Lx, const int8_t *ea, const dd *Linv, co
                               int NB, int *prog, bool fwd, void *ws, size_t ws_bytes, int *err, int *abort_flag,
                               cudaStream_t s) {
   if (B <= 0 || NB <= 0) return cudaSuccess;
-  if (ws_bytes < trsm_tc_ws_bytes(B) || out_bstride < (long)NB * NB_) return cudaErrorInvalidValue;
+  if (ws_bytes < trsm_tc_ws_bytes(NB, B) || out_bstride < (long)NB * NB_) return cudaErrorInvalidValue;
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   nsm = std::max(nsm, 1);
   cudaError_t e = cudaMemsetAsync(prog, 0, sizeof(int) * trsm_prog_ints(B), s);
+  const PanelWs w = panel_ws(ws, NB, B);
+  if (e == cudaSuccess) e = cudaMemsetAsync(w.se, 0, w.se_bytes, s);
   // the running sums start at zero
   if (e == cudaSuccess)
     e = cudaMemset2DAsync(out, (size_t)out_bstride * sizeof(dd), 0, (size_t)NB * NB_ * sizeof(dd), B, s);
@@ -565,8 +753,8 @@ cudaError_t launch_trsm_dd_tc(const dd *Lx, const int8_t *ea, const dd *Linv, co
     e = launch_trsm_dd_panel(Lx, Linv, rhs, rhs_kind, rhs_bstride, out, out_bstride, win, Nd, Nt, B, NB, J0, J1,
                              &base, prog, fwd, err, abort_flag, s);
     if (e == cudaSuccess)
-      e = fwd ? update_panel<true>(Lx, ea, out, out_bstride, win, Nd, Nt, B, NB, J0, (uint8_t *)ws, nsm, err, s)
-              : update_panel<false>(Lx, ea, out, out_bstride, win, Nd, Nt, B, NB, J0, (uint8_t *)ws, nsm, err, s);
+      e = fwd ? update_panel<true>(Lx, ea, out, out_bstride, win, Nd, Nt, B, NB, J0, w, nsm, err, s)
+              : update_panel<false>(Lx, ea, out, out_bstride, win, Nd, Nt, B, NB, J0, w, nsm, err, s);
   }
   return e;
 }

@@ -258,7 +258,7 @@ size_t lane_bytes(const tw_ctx *c, int bmax) {
     const int cols = (bmax + 7) / 8 * 8 + 80;
     b += 2 * B * np * sizeof(dd) + sl_ws_bytes(c->Nf, c->Rmax, cols) + sl_eb_bytes(c->Nf, cols);
   }
-  if (c->trsm_eb) b += trsm_tc_ws_bytes(bmax);
+  if (c->trsm_eb) b += trsm_tc_ws_bytes(c->NB, bmax);
   if (c->ea64) b += sl64_ws_bytes(c->Nf, c->Nd, c->Nm, bmax) + sl64_eb_bytes(c->Nf, bmax) +
                    gemm_fwd_sl64_ws_bytes(c->Nf, c->Rmax, c->Nm, bmax);
   return b;
@@ -304,7 +304,7 @@ tw_status alloc_lane(tw_ctx *c, tw_lane &L, int bmax) {
     L.bsl_eb = (int *)take(L.bsl_eb_n);
   }
   if (ok && c->trsm_eb) {             // optional: null leaves the sweeps in one launch
-    L.trsm_ws_n = trsm_tc_ws_bytes(bmax);
+    L.trsm_ws_n = trsm_tc_ws_bytes(c->NB, bmax);
     L.trsm_ws = twh::dalloc(c, L.trsm_ws_n);
   }
   if (ok && c->ea64) {                // optional: null leaves the SIMT product

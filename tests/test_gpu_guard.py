@@ -118,3 +118,38 @@ def test_forward_of_wide_range(Nq, B, spread):
     assert torch.equal(one[0], q[0][0])
     keep = [b for b in range(B) if b != 1]
     assert torch.equal(mates[keep], q[0][keep]) and torch.isnan(mates[1]).all()
+
+
+# sweeps in panels (132 block rows) whose loud right-hand sides meet small entries of
+# the factor: half of the sensors measure 2^spread times less, and their data are
+# that much larger, so the two halves' terms come out alike
+@pytest.mark.parametrize("spread", [0, 24, 40])
+@pytest.mark.parametrize("B", [64, 70])
+def test_sweeps_of_wide_range(B, spread):
+    import torch
+    Nd, Nx, Ny, Nt = 200, 6, 5, 42
+    F, Fq = _randn(1, Nt, Nd, Nx * Ny), _randn(2, Nt, 2, Nx * Ny)
+    F[:, ::2] *= 2.0 ** -spread
+    tw, ctx = _context(Nd, Nx, Ny, Nt, 1, F, Fq, 1.0 * Nx * Ny * Nt)
+    d = _randn(3, B, Nt, Nd)
+    d[:, :, ::2] *= 2.0 ** spread
+    win = [1 + (7 * b + Nt - 1) % Nt for b in range(B)]
+    ctx.reserve_batch(0)                               # single-vector solves
+    ref = ctx.infer(tw.PREC_FP64, d, windows=win)
+    ctx.reserve_batch(B)
+    dev = torch.tensor(win, dtype=torch.int32, device="cuda")
+    m, _ = ctx.infer_batch(tw.PREC_FP64, d, dev)
+    one, _ = ctx.infer_batch(tw.PREC_FP64, d[B - 1:], dev[B - 1:])
+    bad = d.clone()
+    bad[1, 0, 0] = float("nan")
+    mates, _ = ctx.infer_batch(tw.PREC_FP64, bad, dev)
+    ctx.check()
+    ctx.close()
+    # two solves in 48-bit arithmetic, K's condition a few hundred: the bound of
+    # test_batched_solves in test_gpu_slices.py
+    for b in range(B):
+        e = (m[b] - ref[b]).norm() / ref[b].norm()
+        assert e < 1e-11, (b, float(e))
+    assert torch.equal(one[0], m[B - 1])
+    keep = [b for b in range(B) if b != 1]
+    assert torch.equal(mates[keep], m[keep])
