@@ -125,7 +125,7 @@ tw_status autotune_lane(tw_ctx *c, tw_lane &L) {
   if (c->op[TW_MAP_F][TW_PREC_FP64]) {
     const void *A = c->opG[0] ? c->opG[0] : c->op[TW_MAP_F][0];
     const int8_t *ea = c->ea64;
-    const bool tc = ea && L.sl64_ws;
+    const bool tc = ea != nullptr;
     const int cand[4] = {0, 4, 2, 1};
     double ms[4];
     for (int k = 0; k < 4; ++k)

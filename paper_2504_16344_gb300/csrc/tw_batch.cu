@@ -10,6 +10,7 @@
 // the calls below neither allocate nor synchronise and can be captured into
 // one CUDA graph that is relaunched with new data and windows.
 #include <algorithm>
+#include <initializer_list>
 
 #include "ctx.h"
 #include "dense_api.h"
@@ -67,7 +68,7 @@ static cudaError_t sweep(tw_ctx *c, tw_lane &L, tw_prec prec, bool fwd, const vo
   const dd *Lx = fwd ? c->Lfs : c->Lbs;
   int *prog = L.trsm_prog + (fwd ? 0 : trsm_prog_ints(L.bmax));
   const bool f64 = prec == TW_PREC_FP64, panels = trsm_tc_applies(c->NB, c->lane.bmax);
-  if (f64 && panels && c->trsm_eb && L.trsm_ws)
+  if (f64 && panels && c->trsm_eb)
     return launch_trsm_dd_tc(Lx, fwd ? c->trsm_ef : c->trsm_eb, c->inv_dd, rhs, rhs_kind, rhs_bstride, out,
                              c->n_pad, win, c->Nd, c->Nt, B, c->NB, prog, fwd, L.trsm_ws, L.trsm_ws_n, c->d_err,
                              c->abort_flag, s);
@@ -81,7 +82,7 @@ static cudaError_t forward_dd(tw_ctx *c, tw_lane &L, int which, int B, cudaStrea
   const int Nf = c->Nf, Nr = which == TW_MAP_F ? c->Nd : c->Nq, Nm = c->Nm;
   const void *A = c->op[which][TW_PREC_FP64];
   const cdd *x = (const cdd *)L.bxh;
-  if (L.adj_rw != 0 || !c->ef[which] || !L.sl64_fx)
+  if (L.adj_rw != 0 || !c->ea64)
     return launch_gemm_fwd_dd(A, x, (long)Nf * Nm, (cdd *)L.bpart, (cdd *)L.byh, (long)Nf * Nr, Nf, Nr, Nm, B, s,
                               fwd_lpb(L));
   return launch_gemm_fwd_sl64(A, c->ef[which], x, (long)Nf * Nm, L.sl64_fx, L.sl64_fx_n, (cdd *)L.bpart, (cdd *)L.byh,
@@ -150,7 +151,7 @@ tw_status infer_core(tw_ctx *c, tw_lane &L, tw_prec prec, int B, const int *win,
     { twh::Phase p(c, TW_PH_GEMV_ADJ, s);
       // tensor cores unless a SIMT tile was chosen (tw_batch_tiles) or their
       // exponents or workspace did not fit
-      if (L.adj_rw == 0 && c->ea64 && L.sl64_ws)
+      if (L.adj_rw == 0 && c->ea64)
         TW_CUDA(c, launch_gemm_adj_sl64(A, c->ea64, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm,
                                         Nf, Nd, Nm, B, L.sl64_ws, L.sl64_ws_n, L.sl64_eb, L.sl64_eb_n,
                                         c->d_err, s));
@@ -273,6 +274,22 @@ void free_lane(tw_ctx *c, tw_lane &L) {
   L.bytes = 0;
 }
 
+// workspaces of the panel sweeps and of the sliced products, for the tables that
+// the context holds; false if they do not fit
+bool panel_ws(tw_ctx *c, tw_lane &L, int bmax) {
+  if (!c->trsm_eb) return true;
+  L.trsm_ws_n = trsm_tc_ws_bytes(c->NB, bmax);
+  return (L.trsm_ws = twh::dalloc(c, L.trsm_ws_n)) != nullptr;
+}
+bool product_ws(tw_ctx *c, tw_lane &L, int bmax) {
+  if (!c->ea64) return true;
+  L.sl64_ws_n = sl64_ws_bytes(c->Nf, c->Nd, c->Nm, bmax);
+  L.sl64_eb_n = sl64_eb_bytes(c->Nf, bmax);
+  L.sl64_fx_n = gemm_fwd_sl64_ws_bytes(c->Nf, c->Rmax, c->Nm, bmax);
+  return (L.sl64_eb = (int *)twh::dalloc(c, L.sl64_eb_n)) && (L.sl64_ws = twh::dalloc(c, L.sl64_ws_n)) &&
+         (L.sl64_fx = twh::dalloc(c, L.sl64_fx_n));
+}
+
 tw_status alloc_lane(tw_ctx *c, tw_lane &L, int bmax) {
   free_lane(c, L);
   const size_t B = bmax, np = c->n_pad, Nt = c->Nt, Nf = c->Nf, Nm = c->Nm, R = c->Rmax;
@@ -303,18 +320,9 @@ tw_status alloc_lane(tw_ctx *c, tw_lane &L, int bmax) {
     L.bsl_ws = take(L.bsl_ws_n);
     L.bsl_eb = (int *)take(L.bsl_eb_n);
   }
-  if (ok && c->trsm_eb) {             // optional: null leaves the sweeps in one launch
-    L.trsm_ws_n = trsm_tc_ws_bytes(c->NB, bmax);
-    L.trsm_ws = twh::dalloc(c, L.trsm_ws_n);
-  }
-  if (ok && c->ea64) {                // optional: null leaves the SIMT product
-    L.sl64_ws_n = sl64_ws_bytes(c->Nf, c->Nd, c->Nm, bmax);
-    L.sl64_eb_n = sl64_eb_bytes(c->Nf, bmax);
-    L.sl64_eb = (int *)twh::dalloc(c, L.sl64_eb_n);
-    if (L.sl64_eb) L.sl64_ws = twh::dalloc(c, L.sl64_ws_n);
-    L.sl64_fx_n = gemm_fwd_sl64_ws_bytes(c->Nf, c->Rmax, c->Nm, bmax);
-    if (L.sl64_ws) L.sl64_fx = twh::dalloc(c, L.sl64_fx_n);
-  }
+  // a further lane of a context that holds the tables runs the sliced products and
+  // panel sweeps too (a result must not depend on its lane), or not at all
+  ok = ok && panel_ws(c, L, bmax) && product_ws(c, L, bmax);
   if (!ok) {
     free_lane(c, L);
     return twh::fail(c, TW_ERR_OOM, "batch workspaces");
@@ -331,15 +339,35 @@ tw_status alloc_lane(tw_ctx *c, tw_lane &L, int bmax) {
 
 namespace {
 
+void drop(tw_ctx *c, std::initializer_list<void **> bufs) {
+  for (void **b : bufs) { twh::dfree(c, *b); *b = nullptr; }
+}
+void free_panel_tables(tw_ctx *c) { drop(c, {(void **)&c->trsm_ef, (void **)&c->trsm_eb, &c->lane.trsm_ws}); }
+void free_product_tables(tw_ctx *c) {
+  drop(c, {(void **)&c->ea64, (void **)&c->ef[0], (void **)&c->ef[1], (void **)&c->lane.sl64_eb, &c->lane.sl64_ws,
+           &c->lane.sl64_fx});
+}
 void free_batch(tw_ctx *c) {
+  free_panel_tables(c);
+  free_product_tables(c);
   twb::free_lane(c, c->lane);
-  twh::dfree(c, c->inv_dd);
-  twh::dfree(c, c->trsm_ef);
-  twh::dfree(c, c->trsm_eb);
-  twh::dfree(c, c->ea64);
-  for (int8_t *&e : c->ef) { twh::dfree(c, e); e = nullptr; }
-  c->inv_dd = nullptr;
-  c->trsm_ef = c->trsm_eb = c->ea64 = nullptr;
+  drop(c, {(void **)&c->inv_dd});
+}
+
+// tables and workspaces of the panel sweeps and of the sliced products, after what
+// every batch needs and each all or nothing: without them the sweeps run as one
+// launch and the products on the FP32 pipes
+void hold_sliced(tw_ctx *c, int bmax) {
+  if (!c->op[TW_MAP_F][TW_PREC_FP64]) return;
+  if (trsm_tc_applies(c->NB, bmax)) {
+    c->trsm_ef = (int8_t *)twh::dalloc(c, trsm_tc_exp_bytes(c->NB));
+    c->trsm_eb = (int8_t *)twh::dalloc(c, trsm_tc_exp_bytes(c->NB));
+    if (!c->trsm_ef || !c->trsm_eb || !twb::panel_ws(c, c->lane, bmax)) free_panel_tables(c);
+  }
+  c->ea64 = (int8_t *)twh::dalloc(c, row_exp64_bytes(c->Nf, c->Nd, c->Nm));
+  for (int which = 0; which < 2; ++which)
+    c->ef[which] = (int8_t *)twh::dalloc(c, fwd_exp64_bytes(c->Nf, which == TW_MAP_F ? c->Nd : c->Nq, c->Nm));
+  if (!c->ea64 || !c->ef[0] || !c->ef[1] || !twb::product_ws(c, c->lane, bmax)) free_product_tables(c);
 }
 
 }  // namespace
@@ -371,22 +399,13 @@ tw_status tw_reserve_batch(tw_ctx *c, int bmax) {
     free_batch(c);
     return twh::fail(c, TW_ERR_OOM, "batch workspaces");
   }
-  if (trsm_tc_applies(c->NB, bmax) && c->op[TW_MAP_F][TW_PREC_FP64]) {       // optional: without both the sweeps stay on the FP32 pipes
-    c->trsm_ef = (int8_t *)twh::dalloc(c, trsm_tc_exp_bytes(c->NB));
-    if (c->trsm_ef) c->trsm_eb = (int8_t *)twh::dalloc(c, trsm_tc_exp_bytes(c->NB));
-  }
-  // optional as well: exponents of the operators that the sliced products read;
-  // without them those products run on the FP32 pipes
-  if (c->op[TW_MAP_F][TW_PREC_FP64]) {
-    c->ea64 = (int8_t *)twh::dalloc(c, row_exp64_bytes(c->Nf, c->Nd, c->Nm));
-    for (int which = 0; which < 2; ++which)
-      c->ef[which] = (int8_t *)twh::dalloc(c, fwd_exp64_bytes(c->Nf, which == TW_MAP_F ? c->Nd : c->Nq, c->Nm));
-  }
   tw_status st = twb::alloc_lane(c, c->lane, bmax);
   if (st != TW_OK) {
     free_batch(c);
     return st;
   }
+  hold_sliced(c, bmax);
+  c->lane.bytes = twb::lane_bytes(c, bmax);
   st = twh::refresh_dd_factor(c, 0);
   if (st != TW_OK) return st;
   // (rows of F_q that are not loaded yet get theirs in tw_set_block_column)
