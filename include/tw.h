@@ -424,8 +424,9 @@ tw_status tw_infer_batch(tw_ctx *ctx, tw_prec prec, int nrhs, const int *nt_wind
  * Tiles of the batched per-frequency products.  tw_reserve_batch times the
  * legal candidates on the context's operator and workspaces (CUDA events,
  * one warm-up launch, the mean of two) and keeps the fastest; the choice is
- * cached for the process by shape (Nd, Nq, Nx, Ny, Nt, bmax, keep), so a
- * later context of the same shape takes it without measuring.  The
+ * cached for the process by shape (Nd, Nq, Nx, Ny, Nt, bmax, keep) and whether
+ * the sliced products' tables fit, so a later context of the same shape takes
+ * it without measuring.  The
  * environment variable TW_AUTOTUNE=0 keeps the built-in rules instead.
  *   adj_tile  : right-hand sides per tensor-core tile of the reduced-
  *               precision adjoint (multiple of 8, <= 80, 80 as 72; more tiles re-read

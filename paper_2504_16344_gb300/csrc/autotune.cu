@@ -27,12 +27,13 @@ using namespace tw;
 
 namespace {
 
-using Key = std::array<long, 7>;
+using Key = std::array<long, 8>;
 std::mutex g_mu;
 std::map<Key, tw_tiles> g_cache;
 
+// (a reservation without the sliced products' tables has other candidates)
 Key key_of(const tw_ctx *c, int bmax) {
-  return {c->Nd, c->Nq, c->Nx, c->Ny, c->Nt, bmax, (long)c->keep};
+  return {c->Nd, c->Nq, c->Nx, c->Ny, c->Nt, bmax, (long)c->keep, c->ea64 ? 1L : 0L};
 }
 
 // mean device time of fn over two launches after one warm-up (ms; -1 on error)

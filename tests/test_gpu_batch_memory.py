@@ -27,6 +27,7 @@ class Short:
 
     def __init__(self, ctx):
         import torch
+        ctx.reserve_batch(0)
         torch.cuda.empty_cache()
         f = self.free()
         ctx.reserve_batch(B)
@@ -75,3 +76,17 @@ def test_reservation_without_room_for_the_slices(ctx):
     ctx.infer_batch(tw.PREC_FP64, d, win, m, q)
     ctx.check()
     assert torch.equal(m.cpu(), m0) and torch.equal(q.cpu(), q0)
+
+
+def test_choice_without_the_slices_is_not_kept_for_others(ctx):
+    """The measured tiles of such a reservation are not taken over by one with room,
+    whose products run on the tensor cores (several times faster at this size)."""
+    from paper_2504_16344_gb300 import tw
+    short = Short(ctx)
+    tw.autotune_clear_cache()
+    with short:
+        ctx.reserve_batch(B)
+        tight = ctx.batch_tiles().adj_rw
+        ctx.reserve_batch(0)
+    ctx.reserve_batch(B)
+    assert tight in (1, 2, 4) and ctx.batch_tiles().adj_rw == 0
