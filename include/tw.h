@@ -443,7 +443,8 @@ tw_status tw_infer_batch(tw_ctx *ctx, tw_prec prec, int nrhs, const int *nt_wind
  */
 typedef struct {
   int adj_tile, adj_rw, fwd_lanes;
-  double adj_tile_ms, adj_rw_ms, fwd_lanes_ms;  /* time of each choice; -1 if not measured */
+  double adj_tile_ms, adj_rw_ms, fwd_lanes_ms;  /* time of each choice (adj_rw: adjoint and forecast
+                                                 products together); -1 if not measured */
   int tuned;            /* 1 measured (now or by an earlier context), 0 built-in
                            rules, 2 set by tw_set_batch_tiles                  */
 } tw_tiles;

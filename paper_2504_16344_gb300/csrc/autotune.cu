@@ -4,9 +4,9 @@
 // forecast's forward product F_q X, one matrix product per frequency) have
 // tile parameters whose best value depends on the shapes: the number of
 // right-hand sides per tensor-core tile of the mixed adjoint (how many tiles
-// re-read the operator against the MMA width), the right-hand sides per warp
-// of the FP64-class adjoint, and the lanes per right-hand side of the
-// forward products.  tw_reserve_batch times every legal candidate on the
+// re-read the operator against the MMA width), the form of the FP64-class
+// products (tensor cores, or right-hand sides per warp of the adjoint), and the
+// lanes per right-hand side of the FP32-pipe forward products.  tw_reserve_batch times every legal candidate on the
 // context's own operator and workspaces with CUDA events (one warm-up launch,
 // then the mean of two) and keeps the fastest; the choice is cached for the
 // process by shape, so later contexts of the same shape skip the
@@ -112,7 +112,7 @@ tw_status autotune_lane(tw_ctx *c, tw_lane &L) {
     const void *A = c->opG[fmt] ? c->opG[fmt] : c->op[TW_MAP_F][fmt];
     const int8_t *ea = c->opG[fmt] ? c->eaG[fmt] : c->ea[TW_MAP_F][fmt];
     std::vector<int> cand;
-    for (int P = 8; P <= 80 && P <= (B + 7) / 8 * 8; P += 8) cand.push_back(P);
+    for (int P = 8; P <= 72 && P <= (B + 7) / 8 * 8; P += 8) cand.push_back(P);
     std::vector<double> ms;
     for (int P : cand)
       ms.push_back(time_ms([&] {
@@ -122,25 +122,7 @@ tw_status autotune_lane(tw_ctx *c, tw_lane &L) {
     const int k = tw_autotune_pick((int)ms.size(), ms.data());
     if (k >= 0) { t.adj_tile = cand[k]; t.adj_tile_ms = ms[k]; }
   }
-  // 2) FP64-class adjoint: on the tensor cores (0), or right-hand sides per warp
-  if (c->op[TW_MAP_F][TW_PREC_FP64]) {
-    const void *A = c->opG[0] ? c->opG[0] : c->op[TW_MAP_F][0];
-    const int8_t *ea = c->ea64;
-    const bool tc = ea != nullptr;
-    const int cand[4] = {0, 4, 2, 1};
-    double ms[4];
-    for (int k = 0; k < 4; ++k)
-      ms[k] = k == 0 && !tc ? -1.0 : time_ms([&] {
-        if (k == 0)
-          return launch_gemm_adj_sl64(A, ea, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm, Nf,
-                                      Nd, Nm, B, L.sl64_ws, L.sl64_ws_n, L.sl64_eb, L.sl64_eb_n, c->d_err, 0);
-        return launch_gemm_adj_dd(A, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm, Nf, Nd, Nm,
-                                  B, 0, cand[k]);
-      });
-    const int k = tw_autotune_pick(4, ms);
-    if (k >= 0) { t.adj_rw = cand[k]; t.adj_rw_ms = ms[k]; }
-  }
-  // 3) forward products (the forecast's F_q X): lanes per right-hand side
+  // 2) forward products on the FP32 pipes (the forecast's F_q X): lanes per right-hand side
   {
     const int cand[2] = {1, 2};
     double ms[2];
@@ -156,6 +138,29 @@ tw_status autotune_lane(tw_ctx *c, tw_lane &L) {
       });
     const int k = tw_autotune_pick(2, ms);
     if (k >= 0) { t.fwd_lanes = cand[k]; t.fwd_lanes_ms = ms[k]; }
+  }
+  // 3) FP64-class products: on the tensor cores (0), or right-hand sides per warp of
+  // the adjoint.  The choice holds for the forward product as well, so both are
+  // timed: with two sensors and 40 forecast points the FP32-pipe adjoint is faster
+  // by 0.01 ms, the forward product slower by 1.1
+  if (c->op[TW_MAP_F][TW_PREC_FP64]) {
+    const void *A = c->opG[0] ? c->opG[0] : c->op[TW_MAP_F][0];
+    const int cand[4] = {0, 4, 2, 1};
+    double ms[4];
+    L.fwd_lpb = t.fwd_lanes;
+    for (int k = 0; k < 4; ++k) {
+      L.adj_rw = cand[k];
+      ms[k] = k == 0 && !c->ea64 ? -1.0 : time_ms([&] {
+        cudaError_t e = k == 0
+            ? launch_gemm_adj_sl64(A, c->ea64, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm, Nf, Nd,
+                                   Nm, B, L.sl64_ws, L.sl64_ws_n, L.sl64_eb, L.sl64_eb_n, c->d_err, 0)
+            : launch_gemm_adj_dd(A, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm, Nf, Nd, Nm, B, 0,
+                                 cand[k]);
+        return e == cudaSuccess ? forward_dd(c, L, TW_MAP_FQ, B, 0) : e;
+      });
+    }
+    const int k = tw_autotune_pick(4, ms);
+    if (k >= 0) { t.adj_rw = cand[k]; t.adj_rw_ms = ms[k]; }
   }
   TW_CUDA(c, cudaDeviceSynchronize());
   tw_status st = tw_check(c, 0);

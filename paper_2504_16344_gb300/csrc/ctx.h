@@ -172,6 +172,8 @@ tw_status refresh_dd_factor(tw_ctx *c, cudaStream_t s);
 
 // host-window calls routed to the batched path (tw_batch.cu)
 namespace twb {
+// y^ = F^ x^ of a map in the FP64 class, in the lane's buffers
+cudaError_t forward_dd(tw_ctx *c, tw_lane &L, int which, int B, cudaStream_t s);
 // allocate / free a lane's workspaces (bmax right-hand sides)
 tw_status alloc_lane(tw_ctx *c, tw_lane &L, int bmax);
 void free_lane(tw_ctx *c, tw_lane &L);

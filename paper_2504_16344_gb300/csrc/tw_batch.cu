@@ -78,7 +78,7 @@ static cudaError_t sweep(tw_ctx *c, tw_lane &L, tw_prec prec, bool fwd, const vo
 
 // y^ = F^ x^ of a map in the FP64 class (x^ in L.bxh, y^ to L.byh): on the
 // tensor cores unless SIMT tiles were chosen or their tables did not fit
-static cudaError_t forward_dd(tw_ctx *c, tw_lane &L, int which, int B, cudaStream_t s) {
+cudaError_t forward_dd(tw_ctx *c, tw_lane &L, int which, int B, cudaStream_t s) {
   const int Nf = c->Nf, Nr = which == TW_MAP_F ? c->Nd : c->Nq, Nm = c->Nm;
   const void *A = c->op[which][TW_PREC_FP64];
   const cdd *x = (const cdd *)L.bxh;
