@@ -432,10 +432,12 @@ tw_status tw_infer_batch(tw_ctx *ctx, tw_prec prec, int nrhs, const int *nt_wind
  *               precision adjoint (multiple of 8, <= 80, 80 as 72; more tiles re-read
  *               the operator, fewer leave the MMA narrow)
  *   adj_rw    : right-hand sides per warp of the FP64-class adjoint on the
- *               FP32 pipes (1, 2, 4), the forward product there too; 0 = both
- *               on the tensor cores (on the FP32 pipes by batch size if their
- *               workspaces did not fit): exact fixed-point slices, 56 bits below
- *               the largest entry of an operator row and of a data column
+ *               FP32 pipes (1, 2, 4); 0 = on the tensor cores (on the FP32 pipes by
+ *               batch size if their workspaces did not fit), where exact
+ *               fixed-point slices are multiplied and sums that these would leave
+ *               fewer digits than double-float are formed in double-float.  The
+ *               forward products take the form measured as faster for each map;
+ *               tw_set_batch_tiles puts them where it puts the adjoint.
  *   fwd_lanes : lanes per right-hand side of the forward products (1, 2)
  * A column's result never depends on its batch mates for any choice; it
  * can differ in the last bits between choices (fwd_lanes changes the order
@@ -443,8 +445,7 @@ tw_status tw_infer_batch(tw_ctx *ctx, tw_prec prec, int nrhs, const int *nt_wind
  */
 typedef struct {
   int adj_tile, adj_rw, fwd_lanes;
-  double adj_tile_ms, adj_rw_ms, fwd_lanes_ms;  /* time of each choice (adj_rw: adjoint and forecast
-                                                 products together); -1 if not measured */
+  double adj_tile_ms, adj_rw_ms, fwd_lanes_ms;  /* time of each choice; -1 if not measured */
   int tuned;            /* 1 measured (now or by an earlier context), 0 built-in
                            rules, 2 set by tw_set_batch_tiles                  */
 } tw_tiles;

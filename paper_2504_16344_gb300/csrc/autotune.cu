@@ -4,9 +4,10 @@
 // forecast's forward product F_q X, one matrix product per frequency) have
 // tile parameters whose best value depends on the shapes: the number of
 // right-hand sides per tensor-core tile of the mixed adjoint (how many tiles
-// re-read the operator against the MMA width), the form of the FP64-class
-// products (tensor cores, or right-hand sides per warp of the adjoint), and the
-// lanes per right-hand side of the FP32-pipe forward products.  tw_reserve_batch times every legal candidate on the
+// re-read the operator against the MMA width), the form of each FP64-class
+// product (tensor cores, or FP32 pipes: for the adjoint with how many right-hand
+// sides per warp), and the lanes per right-hand side of the FP32-pipe forward
+// products.  tw_reserve_batch times every legal candidate on the
 // context's own operator and workspaces with CUDA events (one warm-up launch,
 // then the mean of two) and keeps the fastest; the choice is cached for the
 // process by shape, so later contexts of the same shape skip the
@@ -29,7 +30,11 @@ namespace {
 
 using Key = std::array<long, 8>;
 std::mutex g_mu;
-std::map<Key, tw_tiles> g_cache;
+struct Choice {
+  tw_tiles t{};
+  bool fwd_tc[2] = {true, true};     // FP64-class forward products with F, F_q on the tensor cores
+};
+std::map<Key, Choice> g_cache;
 
 // (a reservation without the sliced products' tables has other candidates)
 Key key_of(const tw_ctx *c, int bmax) {
@@ -56,20 +61,34 @@ double time_ms(F fn) {
   return ms;
 }
 
-void apply(tw_lane &L, const tw_tiles &t) {
-  L.sl_tile = t.adj_tile;
-  L.adj_rw = t.adj_rw;
-  L.fwd_lpb = t.fwd_lanes;
+void apply(tw_ctx *c, tw_lane &L, const Choice &v) {
+  L.sl_tile = v.t.adj_tile;
+  L.adj_rw = v.t.adj_rw;
+  L.fwd_lpb = v.t.fwd_lanes;
+  for (int which = 0; which < 2; ++which) L.fwd_tc[which] = v.fwd_tc[which];
+  c->tiles = v.t;
 }
 
-tw_tiles rule_tiles(const tw_lane &L) {
-  tw_tiles t{};
+// The choice without measuring.  FP64-class products on the tensor cores where that
+// was the faster form (60 and 40 steps of 12,500 and 600 points, 1 to 32 right-hand
+// sides; us, SIMT less tensor cores): the adjoint from eight sensors on (2: -45, 8: 41,
+// 27: 250, 100: 1,090) if it is worth the launches (600 points: 8 sensors -12, 27: 0,
+// 100: 35), the forward product from 17 rows on (10: -270, 40: 1,240), with more than
+// 16 right-hand sides from three on (1: -370, 3: 40, 10: 300).
+Choice rule_tiles(const tw_ctx *c, const tw_lane &L) {
+  Choice v;
+  tw_tiles &t = v.t;
   t.adj_tile = sl_pick_tile(L.bmax);
-  t.adj_rw = 0;
+  const double work = (double)c->Nd * c->Nm * c->Nf * ((L.bmax + 7) / 8 * 8);
+  t.adj_rw = c->Nd >= 8 && work >= 6e6 ? 0 : (L.bmax > 16 ? 4 : (L.bmax > 8 ? 2 : 1));
+  for (int which = 0; which < 2; ++which) {
+    const int Nr = which == TW_MAP_F ? c->Nd : c->Nq;
+    v.fwd_tc[which] = Nr > 16 || (L.bmax > 16 && Nr >= 3);
+  }
   t.fwd_lanes = L.bmax <= 16 ? 2 : 1;
   t.adj_tile_ms = t.adj_rw_ms = t.fwd_lanes_ms = -1.0;
   t.tuned = 0;
-  return t;
+  return v;
 }
 
 }  // namespace
@@ -80,14 +99,15 @@ void copy_tiles(tw_lane &dst, const tw_lane &src) {
   dst.sl_tile = src.sl_tile;
   dst.adj_rw = src.adj_rw;
   dst.fwd_lpb = src.fwd_lpb;
+  for (int which = 0; which < 2; ++which) dst.fwd_tc[which] = src.fwd_tc[which];
 }
 
 tw_status autotune_lane(tw_ctx *c, tw_lane &L) {
-  tw_tiles t = rule_tiles(L);
+  Choice v = rule_tiles(c, L);
+  tw_tiles &t = v.t;
   const char *env = getenv("TW_AUTOTUNE");
   if (env && strcmp(env, "0") == 0) {
-    apply(L, t);
-    c->tiles = t;
+    apply(c, L, v);
     return TW_OK;
   }
   const Key key = key_of(c, L.bmax);
@@ -95,8 +115,7 @@ tw_status autotune_lane(tw_ctx *c, tw_lane &L) {
     std::lock_guard<std::mutex> g(g_mu);
     auto it = g_cache.find(key);
     if (it != g_cache.end()) {
-      apply(L, it->second);
-      c->tiles = it->second;
+      apply(c, L, it->second);
       return TW_OK;
     }
   }
@@ -139,37 +158,42 @@ tw_status autotune_lane(tw_ctx *c, tw_lane &L) {
     const int k = tw_autotune_pick(2, ms);
     if (k >= 0) { t.fwd_lanes = cand[k]; t.fwd_lanes_ms = ms[k]; }
   }
-  // 3) FP64-class products: on the tensor cores (0), or right-hand sides per warp of
-  // the adjoint.  The choice holds for the forward product as well, so both are
-  // timed: with two sensors and 40 forecast points the FP32-pipe adjoint is faster
-  // by 0.01 ms, the forward product slower by 1.1
+  // 3) FP64-class adjoint: on the tensor cores (0), or right-hand sides per warp
   if (c->op[TW_MAP_F][TW_PREC_FP64]) {
     const void *A = c->opG[0] ? c->opG[0] : c->op[TW_MAP_F][0];
     const int cand[4] = {0, 4, 2, 1};
     double ms[4];
-    L.fwd_lpb = t.fwd_lanes;
-    for (int k = 0; k < 4; ++k) {
-      L.adj_rw = cand[k];
+    for (int k = 0; k < 4; ++k)
       ms[k] = k == 0 && !c->ea64 ? -1.0 : time_ms([&] {
-        cudaError_t e = k == 0
-            ? launch_gemm_adj_sl64(A, c->ea64, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm, Nf, Nd,
-                                   Nm, B, L.sl64_ws, L.sl64_ws_n, L.sl64_eb, L.sl64_eb_n, c->d_err, 0)
-            : launch_gemm_adj_dd(A, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm, Nf, Nd, Nm, B, 0,
-                                 cand[k]);
-        return e == cudaSuccess ? forward_dd(c, L, TW_MAP_FQ, B, 0) : e;
+        if (k == 0)
+          return launch_gemm_adj_sl64(A, c->ea64, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm, Nf,
+                                      Nd, Nm, B, L.sl64_ws, L.sl64_ws_n, L.sl64_eb, L.sl64_eb_n, c->d_err, 0);
+        return launch_gemm_adj_dd(A, (const cdd *)L.byh, (long)Nf * Nd, (cdd *)L.bxh, (long)Nf * Nm, Nf, Nd, Nm,
+                                  B, 0, cand[k]);
       });
-    }
     const int k = tw_autotune_pick(4, ms);
     if (k >= 0) { t.adj_rw = cand[k]; t.adj_rw_ms = ms[k]; }
+    // 4) FP64-class forward products: the adjoint's choice would not do for them (two
+    // sensors and 40 forecast points: FP32 pipes faster by 45 us there, slower by 1,240
+    // here; 100 sensors and one point: slower by 1,090 there, faster by 600 here)
+    L.fwd_lpb = t.fwd_lanes;
+    for (int which = 0; which < 2; ++which) {
+      double f[2];
+      for (int k = 0; k < 2; ++k) {
+        L.fwd_tc[which] = k == 0;
+        f[k] = k == 0 && !c->ea64 ? -1.0 : time_ms([&] { return forward_dd(c, L, which, B, 0); });
+      }
+      const int k2 = tw_autotune_pick(2, f);
+      if (k2 >= 0) v.fwd_tc[which] = k2 == 0;
+    }
   }
   TW_CUDA(c, cudaDeviceSynchronize());
   tw_status st = tw_check(c, 0);
   if (st != TW_OK) return st;
   t.tuned = 1;
-  apply(L, t);
-  c->tiles = t;
+  apply(c, L, v);
   std::lock_guard<std::mutex> g(g_mu);
-  g_cache[key] = t;
+  g_cache[key] = v;
   return TW_OK;
 }
 
@@ -199,11 +223,12 @@ tw_status tw_set_batch_tiles(tw_ctx *c, const tw_tiles *t) {
   if (t->adj_rw != 0 && t->adj_rw != 1 && t->adj_rw != 2 && t->adj_rw != 4)
     return twh::fail(c, TW_ERR_ARG, "adj_rw must be 0, 1, 2 or 4");
   if (t->fwd_lanes != 1 && t->fwd_lanes != 2) return twh::fail(c, TW_ERR_ARG, "fwd_lanes must be 1 or 2");
-  tw_tiles v = *t;
-  v.adj_tile_ms = v.adj_rw_ms = v.fwd_lanes_ms = -1.0;
-  v.tuned = 2;
-  apply(c->lane, v);
-  c->tiles = v;
+  Choice v;
+  v.t = *t;
+  v.t.adj_tile_ms = v.t.adj_rw_ms = v.t.fwd_lanes_ms = -1.0;
+  v.t.tuned = 2;
+  v.fwd_tc[0] = v.fwd_tc[1] = t->adj_rw == 0;
+  apply(c, c->lane, v);
   return TW_OK;
 }
 

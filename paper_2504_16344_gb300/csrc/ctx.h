@@ -41,7 +41,8 @@ struct tw_lane {
   // per right-hand side (forward products); chosen by measurement at
   // tw_reserve_batch, the same for every lane of a context
   int sl_tile = 0;
-  int adj_rw = 0;                    // 0: the FP64-class products run on the tensor cores
+  int adj_rw = 0;                    // 0: the FP64-class adjoint runs on the tensor cores
+  bool fwd_tc[2] = {true, true};     // so does its forward product with F, with F_q
   int fwd_lpb = 1;
   size_t bytes = 0;                  // device bytes of the lane
 };

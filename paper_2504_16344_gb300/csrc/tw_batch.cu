@@ -77,12 +77,12 @@ static cudaError_t sweep(tw_ctx *c, tw_lane &L, tw_prec prec, bool fwd, const vo
 }
 
 // y^ = F^ x^ of a map in the FP64 class (x^ in L.bxh, y^ to L.byh): on the
-// tensor cores unless SIMT tiles were chosen or their tables did not fit
+// tensor cores if that was chosen and their tables fit
 cudaError_t forward_dd(tw_ctx *c, tw_lane &L, int which, int B, cudaStream_t s) {
   const int Nf = c->Nf, Nr = which == TW_MAP_F ? c->Nd : c->Nq, Nm = c->Nm;
   const void *A = c->op[which][TW_PREC_FP64];
   const cdd *x = (const cdd *)L.bxh;
-  if (L.adj_rw != 0 || !c->ea64)
+  if (!L.fwd_tc[which] || !c->ea64)
     return launch_gemm_fwd_dd(A, x, (long)Nf * Nm, (cdd *)L.bpart, (cdd *)L.byh, (long)Nf * Nr, Nf, Nr, Nm, B, s,
                               fwd_lpb(L));
   return launch_gemm_fwd_sl64(A, c->ef[which], x, (long)Nf * Nm, L.sl64_fx, L.sl64_fx_n, (cdd *)L.bpart, (cdd *)L.byh,
