@@ -350,3 +350,24 @@ def test_every_tile_candidate_matches_oracle(case):
                 assert em < 1e-11 and eq < 1e-11, (rw, lanes)
     finally:
         ctx.set_batch_tiles(t0.adj_tile, t0.adj_rw, t0.fwd_lanes)
+
+
+def test_tensor_core_products_match_oracle(case):
+    """The FP64-class products on the tensor cores (adj_rw = 0), whatever the tuner
+    chose at this size, give the oracle's result with either lane count."""
+    import torch
+    from paper_2504_16344_gb300 import tw
+    ctx, ws = case["ctx"], case["ws"]
+    t0 = ctx.batch_tiles()
+    win = torch.tensor(ws, dtype=torch.int32, device=case["dev"])
+    d = _t(case["d"], case["dev"])
+    try:
+        for lanes in (1, 2):
+            ctx.set_batch_tiles(t0.adj_tile, 0, lanes)
+            m, q = ctx.infer_batch(tw.PREC_FP64, d, win)
+            ctx.check()
+            m, q = m.cpu().numpy(), q.cpu().numpy()
+            assert max(rel(m[e], case["m_ref"][e]) for e in range(NEV)) < 1e-11
+            assert max(rel(q[e], case["q_ref"][e]) for e in range(NEV)) < 1e-11
+    finally:
+        ctx.set_batch_tiles(t0.adj_tile, t0.adj_rw, t0.fwd_lanes)
