@@ -890,7 +890,7 @@ int cholesky_tc_width() { return CHOL_SW; }
 
 cudaError_t launch_cholesky_d(double *K, long ldk, int NB, double *inv, int *err, uint8_t *ws,
                               size_t ws_bytes, int *eg, cudaStream_t s) {
-  if (!ws) return cholesky_t<double>(K, ldk, NB, inv, err, s);
+  if (!ws) return cudaErrorInvalidValue;
   const size_t sm_inv = 2 * NB_ * (NB_ + 1) * sizeof(double);
   const size_t sm_trsm = 2 * NB_ * (NB_ + 1) * sizeof(double);
   smem_attr(k_inv_diag_d, sm_inv);

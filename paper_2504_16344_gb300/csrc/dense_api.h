@@ -79,10 +79,10 @@ cudaError_t launch_trsm_d(const double *Lp, const double *Linv, const double *Lc
                           const void *rhs, int rhs_kind, long rhs_bstride, double *out,
                           long out_bstride, const int *win, int Nd, int Nt, int B, int NB,
                           int *prog, bool fwd, int *err, int *abort_flag, cudaStream_t s);
-// split: two right-hand sides per column slice, a row's sum split over four
-// threads (faster hand-offs, other rounding)
 // the same sweeps with the single-vector solve's pre-multiplied blocks: Lx =
-// Lf (Linv_I L_IJ, forward) or Lb (L_IJ Linv_J, backward), packed like L
+// Lf (Linv_I L_IJ, forward) or Lb (L_IJ Linv_J, backward), packed like L; split: two
+// right-hand sides per column slice, a row's sum split over four threads (faster
+// hand-offs, other rounding)
 cudaError_t launch_trsm_dd_scaled(const dd *Lx, const dd *Linv, const void *rhs, int rhs_kind,
                                   long rhs_bstride, dd *out, long out_bstride, const int *win, int Nd,
                                   int Nt, int B, int NB, int *prog, bool fwd, bool split, int *err,

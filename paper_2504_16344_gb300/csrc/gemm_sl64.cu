@@ -36,7 +36,7 @@
 // are double-buffered as well.
 // Measured (64 right-hand sides, 100 rows, 50,000 grid points, 401 frequencies):
 // 25.1 ms (28.2 ms with scalar instead of packed slicing), against 246 ms for the SIMT product and 4.8 ms to read the operator;
-// a stage takes 2,100 cycles where its MMAs need 900 (the accumulators are
+// a stage takes 1,900 cycles where its MMAs need 900 (the accumulators are
 // single-buffered at N = 64, so the MMAs of a tile wait for the drain of the
 // one before).  Issuing the MMAs from one lane's branch instead of an elected
 // lane of a converged warp: 43 ms.
