@@ -153,3 +153,42 @@ def test_sweeps_of_wide_range(B, spread):
     assert torch.equal(one[0], m[B - 1])
     keep = [b for b in range(B) if b != 1]
     assert torch.equal(mates[keep], m[keep])
+
+
+# several (frequency, range, tile) items per CTA: 81 x 2 of X^ on the MMA rows, 81 x 2
+# x 2 of F^ on them
+@pytest.mark.parametrize("Nq,B", [(20, 40), (100, 33)])
+def test_forward_over_several_items_per_cta(Nq, B):
+    import torch
+    Nd, Nx, Ny, Nt = 2, 65, 64, 80
+    F, Fq, m = _randn(1, Nt, Nd, Nx * Ny), _randn(2, Nt, Nq, Nx * Ny), _randn(3, B, Nt, Nx * Ny)
+    tw, ctx = _context(Nd, Nx, Ny, Nt, B, F, Fq, 1e6 * Nx * Ny)
+    q = {}
+    for rw in (0, 4):
+        ctx.set_batch_tiles(8, rw, 1)
+        q[rw] = ctx.forecast_batch(tw.PREC_FP64, m)
+    ctx.check()
+    ctx.close()
+    tol = 8 * 2.0 ** -48 * (2 * Nx * Ny) ** 0.5        # as above
+    for b in range(B):
+        e = ((q[0][b] - q[4][b]).norm(dim=0) / q[4][b].norm(dim=0)).max()
+        assert e < tol, (b, float(e))
+
+
+# more row and column tiles in the first panels' updates (85 x 2) than SMs
+def test_sweeps_over_several_tiles_per_cta():
+    import torch
+    Nd, Nx, Ny, Nt, B = 200, 6, 5, 58, 65
+    F, Fq = _randn(1, Nt, Nd, Nx * Ny), _randn(2, Nt, 2, Nx * Ny)
+    tw, ctx = _context(Nd, Nx, Ny, Nt, 1, F, Fq, 1.0 * Nx * Ny * Nt)
+    d = _randn(3, B, Nt, Nd)
+    win = [1 + (7 * b + Nt - 1) % Nt for b in range(B)]
+    ctx.reserve_batch(0)                               # single-vector solves
+    ref = ctx.infer(tw.PREC_FP64, d, windows=win)
+    ctx.reserve_batch(B)
+    m, _ = ctx.infer_batch(tw.PREC_FP64, d, torch.tensor(win, dtype=torch.int32, device="cuda"))
+    ctx.check()
+    ctx.close()
+    for b in range(B):
+        e = (m[b] - ref[b]).norm() / ref[b].norm()
+        assert e < 1e-11, (b, float(e))                # as above
