@@ -654,15 +654,14 @@ int tile_count(int B) { return (B + tile_cols(B) - 1) / tile_cols(B); }
 // ------------------------------------------------------------------ host side
 // Panels against one sweep on the FP32 pipes split over threads (trsm.cu), for
 // the reserved batch (not the call's, so that a column's rounding does not
-// depend on its batch).  Both pay the chain from row to row; the panels add some 8 us
-// a row (five launches and a wave of tiles per 12 rows), the sweep its products,
-// NB / 2 blocks a row for every slice of two right-hand sides.  Measured (us a
-// sweep, panels / split): at slices x NB of 2,100-2,300 they meet (188 block rows, 24
-// right-hand sides 1,541 / 1,537; 260, 16 2,042 / 1,869; 132, 32 1,084 / 1,024), above
-// the panels win (313, 16 (2,504) 2,509 / 2,795; 132, 48 (3,168) 1,250 / 1,462; 260,
-// 24 (3,120) 2,165 / 2,731; 625, 16 (5,000) 6,263 / 10,022; 625, 64 (20,000) 8,805 /
-// 38,628), below they lose (625, 8 (2,500) 6,148 / 5,360; 400, 8 (1,600) 3,408 / 2,488).
-bool trsm_tc_applies(int NB, int bmax) { return NB > 2 * PW && (long)((bmax + 1) / 2) * NB > 2500; }
+// depend on its batch).  Both pay the chain, about 3 us a row; the panels add
+// about 5 us a row (three launches and a wave of tiles per 12 rows), the sweep
+// its products, about 3.2 ns per block and slice of two on 152 SMs (NB / 2
+// blocks a row).  They meet where slices x NB is near 4,000.  Measured (us a
+// sweep): NB 625, 64 right-hand sides (20,000): panels 7,600, one sweep 27,700;
+// NB 188, 16 (1,504): panels 1,240, split sweep 760; NB 118, 11 (708): panels
+// 760, split sweep 350.
+bool trsm_tc_applies(int NB, int bmax) { return NB > 2 * PW && (long)((bmax + 1) / 2) * NB > 4096; }
 
 static int exp_chunks(int NB) { return (NB + PW - 1) / PW * NCH; }   // whole panels
 size_t trsm_tc_exp_bytes(int NB) { return (size_t)exp_chunks(NB) * NB * NB_; }
