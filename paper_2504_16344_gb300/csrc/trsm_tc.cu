@@ -654,13 +654,16 @@ int tile_count(int B) { return (B + tile_cols(B) - 1) / tile_cols(B); }
 // ------------------------------------------------------------------ host side
 // Panels against one sweep on the FP32 pipes split over threads (trsm.cu), for
 // the reserved batch (not the call's, so that a column's rounding does not
-// depend on its batch).  Both pay the chain, about 3 us a row; the panels add
-// about 5 us a row (three launches and a wave of tiles per 12 rows), the sweep
-// its products, about 3.2 ns per block and slice of two on 152 SMs (NB / 2
-// blocks a row).  They meet where slices x NB is near 4,000.  Measured (us a
-// sweep): NB 625, 64 right-hand sides (20,000): panels 7,600, one sweep 27,700;
-// NB 188, 16 (1,504): panels 1,240, split sweep 760; NB 118, 11 (708): panels
-// 760, split sweep 350.
+// depend on its batch).  Both pay the chain from row to row; the panels add some 8 us
+// a row (five launches and a wave of tiles per 12 rows) up to the largest window, the
+// sweep its products, NB / 2 blocks a row for every slice of two right-hand sides,
+// up to their own windows.  Measured (us a sweep, panels / split), windows of a quarter
+// to the whole: they meet at slices x NB near 4,000 (313 block rows, 24 right-hand
+// sides (3,756) 2,525 / 2,489; 132, 64 (4,224) 1,266 / 1,207; 260, 32 (4,160) 2,146 /
+// 2,242), above the panels win (188, 48 (4,512) 1,739 / 1,973; 400, 32 (6,400) 3,641 /
+// 5,394; 625, 64 (20,000) 8,245 / 22,233), below they lose (260, 24 (3,120) 2,016 /
+// 1,671; 188, 24 (2,256) 1,494 / 981).  Windows that are all whole would put the line at
+// 2,200 (260, 24 2,165 / 2,731).
 bool trsm_tc_applies(int NB, int bmax) { return NB > 2 * PW && (long)((bmax + 1) / 2) * NB > 4096; }
 
 static int exp_chunks(int NB) { return (NB + PW - 1) / PW * NCH; }   // whole panels
