@@ -14,6 +14,7 @@
 // transform runs as rows (contiguous), columns (strided, with the lambda
 // scaling and the inverse column transform fused), inverse rows.
 #include <algorithm>
+#include <type_traits>
 
 #include "kernels.h"
 
@@ -119,8 +120,8 @@ __device__ __forceinline__ void stage_cols(typename P::mem *buf, const typename 
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
 }
 
-template <class P, bool BIG>
-__global__ void __launch_bounds__(256, BIG ? P::occ_big : P::occ)
+template <class P, int LEVEL>
+__global__ void __launch_bounds__(256, LEVEL == 2 ? P::occ_big : P::occ)
 k_rfft_time(const void *__restrict__ in, int in_kind, long in_ld, int n_in,
             typename P::mem *__restrict__ out, long out_ld, int N, FftPlan pl,
             const typename P::cx *__restrict__ twM, const typename P::cx *__restrict__ twL,
@@ -149,7 +150,7 @@ k_rfft_time(const void *__restrict__ in, int in_kind, long in_ld, int n_in,
     buf0[j * B + b] = P::make(r, im);
   }
   __syncthreads();
-  cx *Z = fft_run<P, false, BIG>(buf0, buf1, twM, pl, B, B, 1, true);
+  cx *Z = fft_run<P, false, LEVEL>(buf0, buf1, twM, pl, B, B, 1, true);
   // X_k = (Z_k + conj Z_{M-k})/2 + W_L^k (Z_k - conj Z_{M-k})/(2i)
   for (int idx = threadIdx.x; idx < (M + 1) * B; idx += blockDim.x) {
     const int b = idx & (B - 1), k = idx >> lgB;
@@ -164,8 +165,8 @@ k_rfft_time(const void *__restrict__ in, int in_kind, long in_ld, int n_in,
   }
 }
 
-template <class P, bool BIG>
-__global__ void __launch_bounds__(256, BIG ? P::occ_big : P::occ)
+template <class P, int LEVEL>
+__global__ void __launch_bounds__(256, LEVEL == 2 ? P::occ_big : P::occ)
 k_irfft_time(const typename P::mem *__restrict__ in, long in_ld, void *__restrict__ out,
              int out_kind, long out_ld, int N, int n_keep, FftPlan pl,
              const typename P::cx *__restrict__ twM, const typename P::cx *__restrict__ twL,
@@ -194,7 +195,7 @@ k_irfft_time(const typename P::mem *__restrict__ in, long in_ld, void *__restric
     buf1[k * B + b] = P::add(E, P::mul_i(O));
   }
   __syncthreads();
-  cx *z = fft_run<P, true, BIG>(buf1, buf0, twM, pl, B, B, 1, true);
+  cx *z = fft_run<P, true, LEVEL>(buf1, buf0, twM, pl, B, B, 1, true);
   for (int idx = threadIdx.x; idx < M * B; idx += blockDim.x) {
     const int b = idx & (B - 1), t = idx >> lgB;
     const long n = n0 + b;
@@ -213,8 +214,8 @@ k_irfft_time(const typename P::mem *__restrict__ in, long in_ld, void *__restric
 // transform of m (-> m^ into `spec`, which may be `in`: a CTA reads all of its
 // columns before it writes them).  The forecast's time FFT of m then needs no
 // second pass over m in HBM and no conversion of m back from its stored type.
-template <class P, bool BIG>
-__global__ void __launch_bounds__(256, BIG ? P::occ_big : P::occ)
+template <class P, int LEVEL>
+__global__ void __launch_bounds__(256, LEVEL == 2 ? P::occ_big : P::occ)
 k_irfft_rfft_time(const typename P::mem *in, long in_ld, void *__restrict__ out, int out_kind,
                   long out_ld, typename P::mem *spec, long spec_ld, int N, int n_keep_all, FftPlan pl,
                   const typename P::cx *__restrict__ twM, const typename P::cx *__restrict__ twL,
@@ -246,7 +247,7 @@ k_irfft_rfft_time(const typename P::mem *in, long in_ld, void *__restrict__ out,
     buf1[k * B + b] = P::add(E, P::mul_i(O));
   }
   __syncthreads();
-  cx *z = fft_run<P, true, BIG>(buf1, buf0, twM, pl, B, B, 1, true);
+  cx *z = fft_run<P, true, LEVEL>(buf1, buf0, twM, pl, B, B, 1, true);
   cx *w = z == buf0 ? buf1 : buf0;
   // m_t = invM (Re, Im) z_{t/2} for t < n_keep, else 0: written out, and
   // packed again as the forward transform's input m_{2j} + i m_{2j+1}
@@ -266,7 +267,7 @@ k_irfft_rfft_time(const typename P::mem *in, long in_ld, void *__restrict__ out,
     w[j * B + b] = P::make(t0 < M ? r0 : P::re_zero(), t1 < M ? r1 : P::re_zero());
   }
   __syncthreads();
-  cx *Z = fft_run<P, false, BIG>(w, z, twM, pl, B, B, 1, true);
+  cx *Z = fft_run<P, false, LEVEL>(w, z, twM, pl, B, B, 1, true);
   // X_k = (Z_k + conj Z_{M-k})/2 + W_L^k (Z_k - conj Z_{M-k})/(2i)  (as in k_rfft_time)
   for (int idx = threadIdx.x; idx < (M + 1) * B; idx += blockDim.x) {
     const int b = idx & (B - 1), k = idx >> lgB;
@@ -290,7 +291,7 @@ struct FieldMap {
 };
 
 // rows pass: pair tp holds z = x_{2tp} + i x_{2tp+1}; FFT along b (length Ny)
-template <class P, bool INV>
+template <class P, bool INV, int LEVEL>
 __global__ void __launch_bounds__(256, P::occ_prior)
 k_prior_rows(const void *__restrict__ x, int in_kind, void *__restrict__ y, int out_kind,
              typename P::cx *__restrict__ work, int nt, int Nx, int Ny, FftPlan ply,
@@ -339,7 +340,7 @@ k_prior_rows(const void *__restrict__ x, int in_kind, void *__restrict__ y, int 
     buf0[b * Ny + j] = v;
   }
   __syncthreads();
-  cx *Z = fft_run<P, INV, true>(buf0, buf1, twy, ply, BR, 1, Ny, false);
+  cx *Z = fft_run<P, INV, LEVEL>(buf0, buf1, twy, ply, BR, 1, Ny, false);
   for (int idx = threadIdx.x; idx < BR * Ny; idx += blockDim.x) {
     unsigned jq, jr;
     fdivmod((unsigned)idx, (unsigned)Ny, mag, jq, jr);
@@ -364,7 +365,7 @@ k_prior_rows(const void *__restrict__ x, int in_kind, void *__restrict__ y, int 
 
 // columns pass: forward FFT along a (length Nx, stride Ny), scale by lambda,
 // inverse FFT along a, in place in `work`.
-template <class P>
+template <class P, int LEVEL>
 __global__ void __launch_bounds__(256, P::occ_prior)
 k_prior_cols(typename P::cx *__restrict__ work, const typename P::re *__restrict__ lam, int Nx,
              int Ny, FftPlan plx, const typename P::cx *__restrict__ twx, int BC, int nt,
@@ -384,14 +385,14 @@ k_prior_cols(typename P::cx *__restrict__ work, const typename P::re *__restrict
     buf0[a * BC + b] = (j < Ny) ? wp[(long)a * Ny + j] : P::zero();
   }
   __syncthreads();
-  cx *Z = fft_run<P, false, true>(buf0, buf1, twx, plx, BC, BC, 1, true);
+  cx *Z = fft_run<P, false, LEVEL>(buf0, buf1, twx, plx, BC, BC, 1, true);
   cx *O = (Z == buf0) ? buf1 : buf0;
   for (int idx = threadIdx.x; idx < Nx * BC; idx += blockDim.x) {
     const int b = idx & (BC - 1), p = idx >> lgB, j = j0 + b;
     if (j < Ny) Z[p * BC + b] = P::scale_re(Z[p * BC + b], lam[(long)p * Ny + j]);
   }
   __syncthreads();
-  cx *Y = fft_run<P, true, true>(Z, O, twx, plx, BC, BC, 1, true);
+  cx *Y = fft_run<P, true, LEVEL>(Z, O, twx, plx, BC, BC, 1, true);
   for (int idx = threadIdx.x; idx < Nx * BC; idx += blockDim.x) {
     const int b = idx & (BC - 1), a = idx >> lgB, j = j0 + b;
     if (j < Ny) wp[(long)a * Ny + j] = Y[a * BC + b];
@@ -427,7 +428,7 @@ k_cfield_rows(cdd *__restrict__ x, cd *__restrict__ work, int Nx, int Ny, FftPla
     buf0[b * Ny + j] = v;
   }
   __syncthreads();
-  cd *Z = fft_run<PolD, INV, true>(buf0, buf1, twy, ply, BR, 1, Ny, false);
+  cd *Z = fft_run<PolD, INV, 0>(buf0, buf1, twy, ply, BR, 1, Ny, false);
   for (int idx = threadIdx.x; idx < BR * Ny; idx += blockDim.x) {
     unsigned jq, jr;
     fdivmod((unsigned)idx, (unsigned)Ny, mag, jq, jr);
@@ -457,6 +458,17 @@ int pick_batch(int len, size_t elem, int cap, size_t budget) {
   return B;
 }
 
+// launch(integral_constant<int, level>) of a plan for B series a CTA
+template <class P, class F>
+void at_level(const FftPlan &pl, int B, int least, const F &launch) {
+  if constexpr (P::fused) {
+    const int level = fft_level(pl, B, least);
+    if (level == 2) return launch(std::integral_constant<int, 2>{});
+    if (level == 1) return launch(std::integral_constant<int, 1>{});
+  }
+  launch(std::integral_constant<int, 0>{});
+}
+
 template <class P>
 cudaError_t rfft_time(const void *in, int in_kind, long in_ld, int n_in, typename P::mem *out,
                       long out_ld, int N, const FftPlan &pl, const typename P::cx *twM,
@@ -465,19 +477,11 @@ cudaError_t rfft_time(const void *in, int in_kind, long in_ld, int n_in, typenam
   const int B = pick_batch(pl.M + 1, sizeof(typename P::cx), 32, P::smem);
   const size_t sm = (size_t)2 * (pl.M + 1) * B * sizeof(typename P::cx);
   const dim3 grid((unsigned)((N + B - 1) / B), (unsigned)ba.count);
-  const bool big = P::fused && fft_big(pl);
-  if constexpr (P::fused) {
-    if (big) {
-      ensure_smem(k_rfft_time<P, true>, sm);
-      k_rfft_time<P, true><<<grid, 256, sm, s>>>(in, in_kind, in_ld, n_in, out, out_ld, N, pl, twM, twL, B,
-                                       ba);
-    }
-  }
-  if (!big) {
-    ensure_smem(k_rfft_time<P, false>, sm);
-    k_rfft_time<P, false><<<grid, 256, sm, s>>>(in, in_kind, in_ld, n_in, out, out_ld, N, pl, twM, twL, B,
-                                       ba);
-  }
+  at_level<P>(pl, B, FFT_LEAST_TIME, [&](auto level) {
+    constexpr int LV = decltype(level)::value;
+    ensure_smem(k_rfft_time<P, LV>, sm);
+    k_rfft_time<P, LV><<<grid, 256, sm, s>>>(in, in_kind, in_ld, n_in, out, out_ld, N, pl, twM, twL, B, ba);
+  });
   count_launches(1);
   return cudaGetLastError();
 }
@@ -491,19 +495,11 @@ cudaError_t irfft_time(const typename P::mem *in, long in_ld, void *out, int out
   const int B = pick_batch(pl.M + 1, sizeof(typename P::cx), 32, P::smem);
   const size_t sm = (size_t)2 * (pl.M + 1) * B * sizeof(typename P::cx);
   const dim3 grid((unsigned)((N + B - 1) / B), (unsigned)ba.count);
-  const bool big = P::fused && fft_big(pl);
-  if constexpr (P::fused) {
-    if (big) {
-      ensure_smem(k_irfft_time<P, true>, sm);
-      k_irfft_time<P, true><<<grid, 256, sm, s>>>(in, in_ld, out, out_kind, out_ld, N, n_keep, pl, twM, twL,
-                                        invM, B, ba);
-    }
-  }
-  if (!big) {
-    ensure_smem(k_irfft_time<P, false>, sm);
-    k_irfft_time<P, false><<<grid, 256, sm, s>>>(in, in_ld, out, out_kind, out_ld, N, n_keep, pl, twM, twL,
-                                        invM, B, ba);
-  }
+  at_level<P>(pl, B, FFT_LEAST_TIME, [&](auto level) {
+    constexpr int LV = decltype(level)::value;
+    ensure_smem(k_irfft_time<P, LV>, sm);
+    k_irfft_time<P, LV><<<grid, 256, sm, s>>>(in, in_ld, out, out_kind, out_ld, N, n_keep, pl, twM, twL, invM, B, ba);
+  });
   count_launches(1);
   return cudaGetLastError();
 }
@@ -523,18 +519,24 @@ cudaError_t prior(const void *x, int in_kind, void *y, int out_kind, int nt, int
   while (BC * 2 <= 16 && (size_t)2 * (BC * 2) * Nx * sizeof(cx) <= (size_t)P::smem) BC *= 2;
   const size_t smr = (size_t)2 * BR * Ny * sizeof(cx);
   const size_t smc = (size_t)2 * BC * Nx * sizeof(cx);
-  ensure_smem(k_prior_rows<P, false>, smr);
-  ensure_smem(k_prior_rows<P, true>, smr);
-  ensure_smem(k_prior_cols<P>, smc);
-  dim3 gr((Nx + BR - 1) / BR, np, ba.count), gc((Ny + BC - 1) / BC, np, ba.count);
-  k_prior_rows<P, false><<<gr, 256, smr, s>>>(x, in_kind, nullptr, 0, work, nt, Nx, Ny, ply, twy, BR,
-                                              fm, ba, 0);
-  count_launches(1);
-  k_prior_cols<P><<<gc, 256, smc, s>>>(work, lam, Nx, Ny, plx, twx, BC, nt, ba);
-  count_launches(1);
-  k_prior_rows<P, true><<<gr, 256, smr, s>>>(nullptr, 0, y, out_kind, work, nt, Nx, Ny, ply, twy, BR,
-                                             fm, ba, accum);
-  count_launches(1);
+  const dim3 gr((Nx + BR - 1) / BR, np, ba.count), gc((Ny + BC - 1) / BC, np, ba.count);
+  at_level<P>(ply, BR, FFT_LEAST_PRIOR, [&](auto level) {
+    constexpr int LV = decltype(level)::value;
+    ensure_smem(k_prior_rows<P, false, LV>, smr);
+    k_prior_rows<P, false, LV><<<gr, 256, smr, s>>>(x, in_kind, nullptr, 0, work, nt, Nx, Ny, ply, twy, BR, fm, ba, 0);
+  });
+  at_level<P>(plx, BC, FFT_LEAST_PRIOR, [&](auto level) {
+    constexpr int LV = decltype(level)::value;
+    ensure_smem(k_prior_cols<P, LV>, smc);
+    k_prior_cols<P, LV><<<gc, 256, smc, s>>>(work, lam, Nx, Ny, plx, twx, BC, nt, ba);
+  });
+  at_level<P>(ply, BR, FFT_LEAST_PRIOR, [&](auto level) {
+    constexpr int LV = decltype(level)::value;
+    ensure_smem(k_prior_rows<P, true, LV>, smr);
+    k_prior_rows<P, true, LV><<<gr, 256, smr, s>>>(nullptr, 0, y, out_kind, work, nt, Nx, Ny, ply, twy, BR, fm, ba,
+                                                   accum);
+  });
+  count_launches(3);
   return cudaGetLastError();
 }
 
@@ -562,19 +564,11 @@ cudaError_t irfft_rfft_time(const typename P::mem *in, long in_ld, void *out, in
   const int B = pick_batch(pl.M + 1, sizeof(typename P::cx), 32, P::smem);
   const size_t sm = (size_t)2 * (pl.M + 1) * B * sizeof(typename P::cx);
   const dim3 grid((unsigned)((N + B - 1) / B), (unsigned)ba.count);
-  const bool big = P::fused && fft_big(pl);
-  if constexpr (P::fused) {
-    if (big) {
-      ensure_smem(k_irfft_rfft_time<P, true>, sm);
-      k_irfft_rfft_time<P, true><<<grid, 256, sm, s>>>(in, in_ld, out, out_kind, out_ld, spec, spec_ld, N, n_keep, pl,
-                                             twM, twL, invM, B, ba);
-    }
-  }
-  if (!big) {
-    ensure_smem(k_irfft_rfft_time<P, false>, sm);
-    k_irfft_rfft_time<P, false><<<grid, 256, sm, s>>>(in, in_ld, out, out_kind, out_ld, spec, spec_ld, N, n_keep, pl,
-                                             twM, twL, invM, B, ba);
-  }
+  at_level<P>(pl, B, FFT_LEAST_TIME, [&](auto level) {
+    constexpr int LV = decltype(level)::value;
+    ensure_smem(k_irfft_rfft_time<P, LV>, sm);
+    k_irfft_rfft_time<P, LV><<<grid, 256, sm, s>>>(in, in_ld, out, out_kind, out_ld, spec, spec_ld, N, n_keep, pl, twM, twL, invM, B, ba);
+  });
   count_launches(1);
   return cudaGetLastError();
 }
@@ -639,13 +633,13 @@ cudaError_t launch_prior_cfields_d(cdd *x, long nf, int Nx, int Ny, cd *work, lo
   const size_t smr = (size_t)2 * BR * Ny * sizeof(cd), smc = (size_t)2 * BC * Nx * sizeof(cd);
   ensure_smem(k_cfield_rows<false>, smr);
   ensure_smem(k_cfield_rows<true>, smr);
-  ensure_smem(k_prior_cols<PolD>, smc);
+  ensure_smem(k_prior_cols<PolD, 0>, smc);
   for (long f0 = 0; f0 < nf; f0 += nf_chunk) {
     const int nc = (int)std::min<long>(nf_chunk, nf - f0);
     cdd *xc = x + f0 * Nx * Ny;
     dim3 gr((Nx + BR - 1) / BR, nc), gc((Ny + BC - 1) / BC, nc);
     k_cfield_rows<false><<<gr, 256, smr, s>>>(xc, work, Nx, Ny, ply, twy, BR);
-    k_prior_cols<PolD><<<gc, 256, smc, s>>>(work, lam, Nx, Ny, plx, twx, BC, 2 * nc, BatchArg{});
+    k_prior_cols<PolD, 0><<<gc, 256, smc, s>>>(work, lam, Nx, Ny, plx, twx, BC, 2 * nc, BatchArg{});
     k_cfield_rows<true><<<gr, 256, smr, s>>>(xc, work, Nx, Ny, ply, twy, BR);
     count_launches(3);
     cudaError_t e = cudaGetLastError();

@@ -40,12 +40,26 @@ struct FftPlan {
   int M;
   FftStages st, fst;
 };
-// whether the fused sequence has the 25-point pass
-inline bool fft_big(const FftPlan &pl) {
+// The sequence for B series a CTA: 0 the single passes, 1 the fused ones, 2 those with
+// the 25-point pass.  A fused pass has a thread do what 4 to 25 did, so it is taken
+// where at least `least` threads get one.  Plans without a fused pass run kernels
+// without their registers and code (complex64 prior filter of 21 x 76 and of 8 batches
+// of 44 x 52: 31.2 -> 28.5 and 98 -> 83 us).
+inline int fft_level(const FftPlan &pl, int B, int least) {
+  int level = 0;
   for (int i = 0; i < pl.fst.nst; ++i)
-    if (pl.fst.R2[i] == 5 && pl.fst.R[i] == 5) return true;
-  return false;
+    if (pl.fst.R2[i] > 1) {
+      const int R = pl.fst.R[i] * pl.fst.R2[i];
+      if (pl.M / R * B < least) return 0;
+      level = R == 25 ? 2 : (level ? level : 1);
+    }
+  return level;
 }
+// time transforms: those of 32 steps and 32 series, 64 threads, 9.7 us single and 8.3 fused
+constexpr int FFT_LEAST_TIME = 32;
+// prior filter, three transforms of up to 16 series a CTA: 64 x 25 (64 threads) 22.4 us
+// single and 25.3 fused, 128 x 128 (128) 45.1 and 41.6
+constexpr int FFT_LEAST_PRIOR = 96;
 
 // floor(2^32 / x) for a divisor x >= 2 (x = 1: any value)
 __device__ __forceinline__ unsigned fdiv_mag(unsigned x) {
@@ -368,26 +382,26 @@ __device__ void fft_pass_generic(typename P::cx *src, typename P::cx *dst,
 }
 
 // Full transform.  Returns the buffer that holds the result (buf0 or buf1).
-// BIG: the plan may hold the 25-point pass (fft_big), which needs more registers.
-template <class P, bool INV, bool BIG>
+// LEVEL as fft_level chose (double-float and FP64: 0); the 25-point pass needs more registers.
+template <class P, bool INV, int LEVEL>
 __device__ typename P::cx *fft_run(typename P::cx *buf0, typename P::cx *buf1,
                                    const typename P::cx *tab, const FftPlan &pl, int B,
                                    int es, int ss, bool series_fast) {
   typedef typename P::cx cx;
   cx *src = buf0, *dst = buf1;
-  const FftStages &fs = P::fused ? pl.fst : pl.st;
+  const FftStages &fs = LEVEL > 0 ? pl.fst : pl.st;
   int p = 1;
   for (int st = 0; st < fs.nst; ++st) {
     const int R = fs.R[st], R2 = fs.R2[st];
     const unsigned pm = fs.pmag[st], sm = fs.smag[st];
-    if constexpr (P::fused) {
+    if constexpr (LEVEL > 0) {
       if (R2 > 1) {
         switch (R * 8 + R2) {
 #define TW_FFT_PASS2(A, C) case A * 8 + C: fft_pass2<P, INV, A, C>(src, dst, tab, pl.M, p, B, es, ss, series_fast, pm, sm); break;
           TW_FFT_PAIRS(TW_FFT_PASS2)
 #undef TW_FFT_PASS2
           default:
-            if constexpr (BIG)
+            if constexpr (LEVEL == 2)
               fft_pass2<P, INV, 5, 5>(src, dst, tab, pl.M, p, B, es, ss, series_fast, pm, sm);
         }
         __syncthreads();
