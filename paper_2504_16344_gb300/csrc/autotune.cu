@@ -175,9 +175,12 @@ tw_status autotune_lane(tw_ctx *c, tw_lane &L) {
     if (k >= 0) { t.adj_rw = cand[k]; t.adj_rw_ms = ms[k]; }
     // 4) FP64-class forward products: the adjoint's choice would not do for them (two
     // sensors and 40 forecast points: FP32 pipes faster by 45 us there, slower by 1,240
-    // here; 100 sensors and one point: slower by 1,090 there, faster by 600 here)
+    // here; 100 sensors and one point: slower by 1,090 there, faster by 600 here).  Above
+    // 16 rows the rule holds at every size measured; there the FP32-pipe form alone would
+    // take most of the reservation's time (0.9 s for 100 rows and 64 right-hand sides)
     L.fwd_lpb = t.fwd_lanes;
     for (int which = 0; which < 2; ++which) {
+      if ((which == TW_MAP_F ? Nd : Nq) > 16) continue;
       double f[2];
       for (int k = 0; k < 2; ++k) {
         L.fwd_tc[which] = k == 0;
