@@ -438,7 +438,8 @@ tw_status tw_infer_batch(tw_ctx *ctx, tw_prec prec, int nrhs, const int *nt_wind
  *               fewer digits than double-float are formed in double-float.  The
  *               forward products take the form that is faster for each map (measured
  *               up to 16 rows); tw_set_batch_tiles puts them where it puts the
- *               adjoint.
+ *               adjoint, and with 1, 2 or 4 keeps the products within large batches'
+ *               solves off the tensor cores as well.
  *   fwd_lanes : lanes per right-hand side of the forward products (1, 2)
  * A column's result never depends on its batch mates for any choice; it
  * can differ in the last bits between choices (fwd_lanes changes the order

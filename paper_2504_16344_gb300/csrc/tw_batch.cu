@@ -60,14 +60,16 @@ namespace twb {
 
 // one batched sweep with K's factor in double-float.  FP64-class results: in
 // panels with the products between them on the tensor cores where their tables
-// are kept, else split over threads.  The reduced paths keep the plain sweep: a
+// are kept and the caller has not put the products on the FP32 pipes
+// (tw_set_batch_tiles), else split over threads.  The reduced paths keep the plain sweep: a
 // last-bit change of y moves the FP32 roundings after it, and with them their
 // results by a few of FP32's last bits.
 static cudaError_t sweep(tw_ctx *c, tw_lane &L, tw_prec prec, bool fwd, const void *rhs, int rhs_kind,
                          long rhs_bstride, dd *out, const int *win, int B, cudaStream_t s) {
   const dd *Lx = fwd ? c->Lfs : c->Lbs;
   int *prog = L.trsm_prog + (fwd ? 0 : trsm_prog_ints(L.bmax));
-  const bool f64 = prec == TW_PREC_FP64, panels = trsm_tc_applies(c->NB, c->lane.bmax);
+  const bool f64 = prec == TW_PREC_FP64, refused = c->tiles.tuned == 2 && L.adj_rw != 0;
+  const bool panels = trsm_tc_applies(c->NB, c->lane.bmax) && !refused;
   if (f64 && panels && c->trsm_eb)
     return launch_trsm_dd_tc(Lx, fwd ? c->trsm_ef : c->trsm_eb, c->inv_dd, rhs, rhs_kind, rhs_bstride, out,
                              c->n_pad, win, c->Nd, c->Nt, B, c->NB, prog, fwd, L.trsm_ws, L.trsm_ws_n, c->d_err,

@@ -75,7 +75,8 @@ def test_reservation_without_room_for_the_slices(ctx):
     ctx.set_batch_tiles(tiles.adj_tile, tiles.adj_rw, tiles.fwd_lanes)
     ctx.infer_batch(tw.PREC_FP64, d, win, m, q)
     ctx.check()
-    assert torch.equal(m.cpu(), m0) and torch.equal(q.cpu(), q0)
+    # (set by hand, these tiles take the sweeps off the tensor cores too: the solves' bound)
+    assert (m.cpu() - m0).norm() / m0.norm() < 1e-11 and (q.cpu() - q0).norm() / q0.norm() < 1e-11
 
 
 def test_choice_without_the_slices_is_not_kept_for_others(ctx):

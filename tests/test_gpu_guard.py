@@ -192,3 +192,32 @@ def test_sweeps_over_several_tiles_per_cta():
     for b in range(B):
         e = (m[b] - ref[b]).norm() / ref[b].norm()
         assert e < 1e-11, (b, float(e))                # as above
+
+
+def test_sweeps_can_be_kept_off_the_tensor_cores():
+    """adj_rw 1, 2 or 4 set by the caller: one launch a sweep instead of panels, the same
+    results within the solves' bound."""
+    import torch
+    Nd, Nx, Ny, Nt, B = 200, 6, 5, 42, 64
+    F, Fq = _randn(1, Nt, Nd, Nx * Ny), _randn(2, Nt, 2, Nx * Ny)
+    tw, ctx = _context(Nd, Nx, Ny, Nt, B, F, Fq, 1.0 * Nx * Ny * Nt)
+    d = _randn(3, B, Nt, Nd)
+    win = torch.full((B,), Nt, dtype=torch.int32, device="cuda")
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    m, q, count = {}, torch.empty((B, Nt, 2), dtype=torch.float64, device="cuda"), {}
+    for rw in (0, 4):
+        ctx.set_batch_tiles(8, rw, 1)
+        m[rw] = torch.empty((B, Nt, Nx * Ny), dtype=torch.float64, device="cuda")
+        with torch.cuda.stream(stream):
+            ctx.infer_batch(tw.PREC_FP64, d, win, m[rw], q, stream=stream)
+            stream.synchronize()
+            with ctx.capture(stream) as cap:
+                ctx.infer_batch(tw.PREC_FP64, d, win, m[rw], q, stream=stream)
+            count[rw] = cap.graph.kernel_count()
+            cap.graph.close()
+    ctx.check()
+    ctx.close()
+    # eleven panels a sweep, five kernels each, against one
+    assert count[4] < 30 and count[0] > count[4] + 80, count
+    assert (m[0] - m[4]).norm() / m[4].norm() < 1e-11
