@@ -232,8 +232,12 @@ k_trsm_mag(const dd *__restrict__ Lx, const int8_t *__restrict__ ea, const uint1
         int top = -1000;
 #pragma unroll
         for (int q = 0; q < NCH; ++q) top = max(top, er[h][q] + ec[i][q]);
-        // four chunks of 192: at most 2 sqrt(192) times the largest T; added in quadrature, rounded up
-        const float t = top > 120 ? __int_as_float(0x7f800000) : 2.f * 13.8565f * tc_pow2f(max(top, -126));
+        // four chunks of 192, added in quadrature: sqrt(192 v) 2^top with v = sum of 4^(e - top),
+        // 1 to 4; sqrt(v) <= (v + 2) / sqrt(8), 6% at most above
+        float v = 0.f;
+#pragma unroll
+        for (int q = 0; q < NCH; ++q) v += tc_pow2f(2 * max(er[h][q] + ec[i][q] - top, -60));
+        const float t = top > 120 ? __int_as_float(0x7f800000) : 4.899f * (v + 2.f) * tc_pow2f(max(top, -126));
         float &E = i ? o.w : o.y;
         const float hi = fmaxf(E, t), r = __fdividef(fminf(E, t), hi);
         E = hi * (1.f + 0.5f * r * r);
