@@ -250,7 +250,7 @@ k_trsm_mag(const dd *__restrict__ Lx, const int8_t *__restrict__ ea, const uint1
 // before panel I0 .. I1-1 is solved: its rows' sums that fail are formed in double-float
 // over all k before the panel (FWD: below I0, else from I1 up), a CTA each.  Of 64
 // events of the benchmark about one sum in a thousand does, in the first three panels
-// forward and in half of the panels backward; with k_trsm_mag 1.7 ms a sweep.
+// forward and in half of the panels backward; with k_trsm_mag 1.9 ms a sweep.
 template <bool FWD>
 __global__ void __launch_bounds__(256)
 k_trsm_redo(const dd *__restrict__ Lx, const float2 *__restrict__ se, dd *__restrict__ out, long zs,
