@@ -134,7 +134,8 @@ __device__ __forceinline__ float guard_scale(int Nm, int nrange, const int8_t *e
 // blocks in turn
 __global__ void __launch_bounds__(256)
 k_fwd_check(const int8_t *__restrict__ ef, const uint16_t *__restrict__ low, const int8_t *__restrict__ ex,
-            const uint16_t *__restrict__ xsum, int nbp, int nrange, int Nr, int Nm, int B, int *__restrict__ open) {
+            const uint16_t *__restrict__ xsum, int nbp, int nrange, int Nr, int Nm, int B, int *__restrict__ open,
+            unsigned long long *__restrict__ Sq) {
   __shared__ float sS[8][16][65], sM[8][64];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
   const int w = blockIdx.y, col0 = blockIdx.z * 64, r0 = blockIdx.x * 16, nf = min(8, (B - col0 + 7) / 8);
@@ -165,6 +166,7 @@ k_fwd_check(const int8_t *__restrict__ ef, const uint16_t *__restrict__ low, con
   for (int t = threadIdx.x; t < 1024; t += 256) {
     const int rl = t >> 6, bl = t & 63, r = r0 + rl, b = col0 + bl;
     if (r >= Nr || b >= B) continue;
+    Sq[((size_t)w * Nr + r) * B + b] = 0;                  // k_fwd_mag's sum
     float v = 0.f, m = 0.f;
     for (int k = 0; k < 8; ++k) { v += sS[k][rl][bl]; m += sM[k][bl]; }
     if (m != 0.f && (v == 0.f || tc_guard_fails(v, guard_scale(Nm, nrange, ef + (size_t)w * nrange * Nr + r, Nr,
@@ -173,20 +175,26 @@ k_fwd_check(const int8_t *__restrict__ ef, const uint16_t *__restrict__ low, con
   }
 }
 
-// Sp[w][range][r][b] = sum_k |F^[r][k]| |X^[b][k]| over a range of grid points, of
-// the open frequencies: 32 rows and 32 columns a CTA, whose warps take 16 points
-// in turn, straight from both operands.  Bound by their second reading.
+// Sq[w][r][b] += sum_k |F^[r][k]| |X^[b][k]| over SUB grid points, of the open
+// frequencies: 32 rows and 32 columns a CTA, whose warps take 16 points in turn,
+// straight from both operands.  The pieces are added as integers, in units of
+// 2^-24 sqrt(n) T, so that their order does not matter (a sum that fails is below
+// 2^15); bit 63: not finite.  Bound by the operands' second reading, and for a few open
+// frequencies by a CTA's own latency, hence the short pieces (whole ranges: 70 us).
+constexpr int SUB = 688;                 // 43 steps of 16
+constexpr unsigned long long S_BAD = 1ull << 63;
 __global__ void __launch_bounds__(256, 2)
-k_fwd_mag(const float4 *__restrict__ F, const float4 *__restrict__ X, long xs, const int *__restrict__ open, int nrt,
-          int nbt, int nrange, int Nr, int Nm, int B, float *__restrict__ Sp) {
+k_fwd_mag(const float4 *__restrict__ F, const float4 *__restrict__ X, long xs, const int8_t *__restrict__ ef,
+          const int8_t *__restrict__ ex, const int *__restrict__ open, int nrt, int nbt, int nrange, int Nr, int Nm,
+          int B, unsigned long long *__restrict__ Sq) {
   const int w = blockIdx.y;
   if (!open[w]) return;
   __shared__ float sh[8][32][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
-  const int r0 = blockIdx.x % nrt * 32, b0 = blockIdx.x / nrt % nbt * 32, rg = blockIdx.x / (nrt * nbt);
-  const int kend = min(Nm, (rg + 1) * RANGE);
+  const int r0 = blockIdx.x % nrt * 32, b0 = blockIdx.x / nrt % nbt * 32, kb = blockIdx.x / (nrt * nbt) * SUB;
+  const int kend = min(Nm, kb + SUB);
   float d[2][4][4] = {};
-  for (int k = rg * RANGE + 16 * warp + c; k - c < kend; k += 128) {
+  for (int k = kb + 16 * warp + c; k - c < kend; k += 128) {
     // four entries' magnitudes, zero past the range (a lane's k are c, c + 4, .. on
     // both sides: a load instruction takes 64 bytes in a row)
     auto quad = [&](const float4 *row, uint32_t *o) {
@@ -224,16 +232,24 @@ k_fwd_mag(const float4 *__restrict__ F, const float4 *__restrict__ X, long xs, c
     if (r0 + r >= Nr || b0 + b >= B) continue;
     float S = 0.f;
     for (int v = 0; v < 8; ++v) S += sh[v][r][b];
-    Sp[(((size_t)w * nrange + rg) * Nr + r0 + r) * B + b0 + b] = S;
+    unsigned long long *o = Sq + ((size_t)w * Nr + r0 + r) * B + b0 + b;
+    if (!(S < __int_as_float(0x7f800000))) {
+      atomicOr(o, S_BAD);
+    } else if (S > 0.f) {
+      const float gs = guard_scale(Nm, nrange, ef + (size_t)w * nrange * Nr + r0 + r, Nr,
+                                   ex + (size_t)w * nrange * B + b0 + b, B);
+      // at least one unit: a sum that is not zero stays so; at most 2^40 a piece
+      const float u = fminf(S / gs * 16777216.f, 1.0995116e12f);
+      atomicAdd(o, u >= 1.f ? (unsigned long long)u : 1ull);
+    }
   }
 }
 
 // Yo[b][w][r]: the ranges' partial sums in order; the sums of open frequencies that
 // fail the guard go on the list todo[1 ..], todo[0] of them
 __global__ void __launch_bounds__(256)
-k_fwd_join(const cdd *__restrict__ part, const int8_t *__restrict__ ef, const int8_t *__restrict__ ex,
-           const int *__restrict__ open, const float *__restrict__ Sp, cdd *__restrict__ Yo, long y_bstride,
-           int nrange, int Nf, int Nr, int Nm, int B, int *__restrict__ todo) {
+k_fwd_join(const cdd *__restrict__ part, const int *__restrict__ open, const unsigned long long *__restrict__ Sq,
+           cdd *__restrict__ Yo, long y_bstride, int nrange, int Nf, int Nr, int B, int *__restrict__ todo) {
   const long i = (long)blockIdx.x * 256 + threadIdx.x;
   if (i >= (long)B * Nf * Nr) return;
   const int r = (int)(i % Nr), w = (int)(i / Nr % Nf), b = (int)(i / Nr / Nf);
@@ -242,10 +258,8 @@ k_fwd_join(const cdd *__restrict__ part, const int8_t *__restrict__ ef, const in
   for (int c = 0; c < nrange; ++c) acc = cdd_add(acc, ld_cdd(p + (size_t)c * Nr));
   st_cdd(Yo + (size_t)b * y_bstride + (size_t)w * Nr + r, acc);
   if (!open[w]) return;
-  float S = 0.f;
-  for (int c = 0; c < nrange; ++c) S += Sp[(((size_t)w * nrange + c) * Nr + r) * B + b];
-  if (tc_guard_fails(S, guard_scale(Nm, nrange, ef + (size_t)w * nrange * Nr + r, Nr,
-                                    ex + (size_t)w * nrange * B + b, B)))
+  const unsigned long long S = Sq[((size_t)w * Nr + r) * B + b];
+  if ((S & S_BAD) || (S != 0 && S < (1ull << 15)))         // as tc_guard_fails: 512 S < sqrt(n) T
     todo[1 + atomicAdd(todo, 1)] = (int)i;
 }
 
@@ -728,7 +742,7 @@ cudaError_t launch_fwd_exp64(const void *F, int8_t *ef, int Nf, int Nr, int Nm, 
 size_t gemm_fwd_sl64_ws_bytes(int Nf, int Nr, int Nm, int B) {
   const size_t nr = gemm_fwd_sl64_nrange(Nm);
   return up16((size_t)Nf * sizeof(int)) + up16(Nf * nr * B) + (size_t)Nf * B * fwd_nbp(Nm) * sizeof(uint16_t) +
-         Nf * nr * Nr * B * sizeof(float) + (1 + (size_t)Nf * Nr * B) * sizeof(int);
+         (size_t)Nf * Nr * B * sizeof(unsigned long long) + (1 + (size_t)Nf * Nr * B) * sizeof(int);
 }
 
 // Yo[b][w][r] for b < B; ef: launch_fwd_exp64; ws: gemm_fwd_sl64_ws_bytes(B).
@@ -745,14 +759,14 @@ cudaError_t launch_gemm_fwd_sl64(const void *F, const int8_t *ef, const cdd *X, 
   int *open = reinterpret_cast<int *>(wp);
   int8_t *ex = reinterpret_cast<int8_t *>(wp += up16((size_t)Nf * sizeof(int)));
   uint16_t *xsum = reinterpret_cast<uint16_t *>(wp += up16((size_t)Nf * nr * B));
-  float *Sp = reinterpret_cast<float *>(wp += (size_t)Nf * B * nbp * sizeof(uint16_t));
-  int *todo = reinterpret_cast<int *>(wp + (size_t)Nf * nr * Nr * B * sizeof(float));
+  unsigned long long *Sq = reinterpret_cast<unsigned long long *>(wp += (size_t)Nf * B * nbp * sizeof(uint16_t));
+  int *todo = reinterpret_cast<int *>(wp + (size_t)Nf * Nr * B * sizeof(unsigned long long));
   cudaError_t e = cudaMemsetAsync(open, 0, (size_t)Nf * sizeof(int), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(todo, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   k_row_scan<false><<<dim3(Nf, B, nr), 256, 0, s>>>(Xp, Nm, x_bstride, Nm, ex, B, xsum, nbp);
   k_fwd_check<<<dim3((Nr + 15) / 16, Nf, (B + 63) / 64), 256, 0, s>>>(ef, fwd_low(ef, Nf, Nr, Nm), ex, xsum, nbp, nr, Nr,
-                                                                     Nm, B, open);
+                                                                     Nm, B, open, Sq);
   count_launches(2);
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
@@ -789,9 +803,10 @@ cudaError_t launch_gemm_fwd_sl64(const void *F, const int8_t *ef, const cdd *X, 
   if (xm) pick(std::true_type{});
   else pick(std::false_type{});
   const int nrt = (Nr + 31) / 32, nbt = (B + 31) / 32;
-  k_fwd_mag<<<dim3(nrt * nbt * nr, Nf), 256, 0, s>>>(Fp, Xp, x_bstride, open, nrt, nbt, nr, Nr, Nm, B, Sp);
-  k_fwd_join<<<(unsigned)(((long)B * Nf * Nr + 255) / 256), 256, 0, s>>>(part, ef, ex, open, Sp, Yo, y_bstride, nr, Nf,
-                                                                        Nr, Nm, B, todo);
+  k_fwd_mag<<<dim3(nrt * nbt * ((Nm + SUB - 1) / SUB), Nf), 256, 0, s>>>(Fp, Xp, x_bstride, ef, ex, open, nrt, nbt, nr,
+                                                                        Nr, Nm, B, Sq);
+  k_fwd_join<<<(unsigned)(((long)B * Nf * Nr + 255) / 256), 256, 0, s>>>(part, open, Sq, Yo, y_bstride, nr, Nf, Nr, B,
+                                                                        todo);
   k_fwd_redo<<<(unsigned)std::max(1, 4 * nsm), 256, 0, s>>>(reinterpret_cast<const cdd *>(F), X, x_bstride, todo, Yo,
                                                            y_bstride, Nf, Nr, Nm);
   count_launches(4);
