@@ -74,10 +74,11 @@ __device__ __forceinline__ void note(int *err, volatile int *fail, int info) {
 template <bool LOW>
 __global__ void __launch_bounds__(256)
 k_row_scan(const float4 *__restrict__ A, long ws, long rs, int Nm, int8_t *__restrict__ e, int es,
-           uint16_t *__restrict__ blk, int nbp) {
+           uint16_t *__restrict__ blk, int nbp, int *__restrict__ open) {
   __shared__ float red[8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rg = blockIdx.z;
   const int kb = rg * RANGE, kend = min(Nm, kb + RANGE);
+  if (!LOW && blockIdx.y == 0 && rg == 0 && threadIdx.x == 0) open[blockIdx.x] = 0;    // for k_fwd_check
   const float4 *p = A + (long)blockIdx.x * ws + (long)blockIdx.y * rs;
   uint16_t *out = blk + ((size_t)blockIdx.x * es + blockIdx.y) * nbp;
   float mx = 0.f;
@@ -245,32 +246,36 @@ k_fwd_mag(const float4 *__restrict__ F, const float4 *__restrict__ X, long xs, c
   }
 }
 
-// Yo[b][w][r]: the ranges' partial sums in order; the sums of open frequencies that
-// fail the guard go on the list todo[1 ..], todo[0] of them
+// Yo[b][w][r]: the ranges' partial sums in order; then the sums of open frequencies
+// that fail the guard again in double-float, by all of the CTA's threads.  (A CTA's
+// outputs are gridDim.x apart: those of one frequency, which fail together, go to
+// different CTAs.)
 __global__ void __launch_bounds__(256)
-k_fwd_join(const cdd *__restrict__ part, const int *__restrict__ open, const unsigned long long *__restrict__ Sq,
-           cdd *__restrict__ Yo, long y_bstride, int nrange, int Nf, int Nr, int B, int *__restrict__ todo) {
-  const long i = (long)blockIdx.x * 256 + threadIdx.x;
-  if (i >= (long)B * Nf * Nr) return;
-  const int r = (int)(i % Nr), w = (int)(i / Nr % Nf), b = (int)(i / Nr / Nf);
-  const cdd *p = part + (size_t)(i / Nr) * nrange * Nr + r;
-  cdd acc = cdd_zero();
-  for (int c = 0; c < nrange; ++c) acc = cdd_add(acc, ld_cdd(p + (size_t)c * Nr));
-  st_cdd(Yo + (size_t)b * y_bstride + (size_t)w * Nr + r, acc);
-  if (!open[w]) return;
-  const unsigned long long S = Sq[((size_t)w * Nr + r) * B + b];
-  if ((S & S_BAD) || (S != 0 && S < (1ull << 15)))         // as tc_guard_fails: 512 S < sqrt(n) T
-    todo[1 + atomicAdd(todo, 1)] = (int)i;
-}
-
-// the listed sums in double-float, one CTA each
-__global__ void __launch_bounds__(256)
-k_fwd_redo(const cdd *__restrict__ F, const cdd *__restrict__ X, long xs, const int *__restrict__ todo,
-           cdd *__restrict__ Yo, long y_bstride, int Nf, int Nr, int Nm) {
+k_fwd_join(const cdd *__restrict__ part, const cdd *__restrict__ F, const cdd *__restrict__ X, long xs,
+           const int *__restrict__ open, const unsigned long long *__restrict__ Sq, cdd *__restrict__ Yo,
+           long y_bstride, int nrange, int Nf, int Nr, int Nm, int B) {
+  __shared__ int list[256], count;
   __shared__ cdd sh[8];
-  const int lane = threadIdx.x & 31, ntodo = todo[0];
-  for (int it = blockIdx.x; it < ntodo; it += gridDim.x) {
-    const int i = todo[1 + it], r = i % Nr, w = i / Nr % Nf, b = i / Nr / Nf;
+  const int lane = threadIdx.x & 31;
+  const long i = blockIdx.x + (long)gridDim.x * threadIdx.x;
+  if (threadIdx.x == 0) count = 0;
+  __syncthreads();
+  if (i < (long)B * Nf * Nr) {
+    const int r = (int)(i % Nr), w = (int)(i / Nr % Nf), b = (int)(i / Nr / Nf);
+    const cdd *p = part + (size_t)(i / Nr) * nrange * Nr + r;
+    cdd acc = cdd_zero();
+    for (int c = 0; c < nrange; ++c) acc = cdd_add(acc, ld_cdd(p + (size_t)c * Nr));
+    st_cdd(Yo + (size_t)b * y_bstride + (size_t)w * Nr + r, acc);
+    if (open[w]) {
+      const unsigned long long S = Sq[((size_t)w * Nr + r) * B + b];
+      if ((S & S_BAD) || (S != 0 && S < (1ull << 15)))     // as tc_guard_fails: 512 S < sqrt(n) T
+        list[atomicAdd(&count, 1)] = threadIdx.x;
+    }
+  }
+  __syncthreads();
+  for (int it = 0; it < count; ++it) {
+    const long q = blockIdx.x + (long)gridDim.x * list[it];
+    const int r = (int)(q % Nr), w = (int)(q / Nr % Nf), b = (int)(q / Nr / Nf);
     const cdd *f = F + ((size_t)w * Nr + r) * Nm, *x = X + (long)b * xs + (size_t)w * Nm;
     cdd a[4] = {cdd_zero(), cdd_zero(), cdd_zero(), cdd_zero()};      // four chains in flight
     for (int k = threadIdx.x; k < Nm; k += 1024)
@@ -280,7 +285,7 @@ k_fwd_redo(const cdd *__restrict__ F, const cdd *__restrict__ X, long xs, const 
     cdd y = cdd_add(cdd_add(a[0], a[1]), cdd_add(a[2], a[3]));
     y.re = tc_warp_sum(y.re);
     y.im = tc_warp_sum(y.im);
-    __syncthreads();                     // the item before is read
+    __syncthreads();                     // the sum before is read
     if (lane == 0) sh[threadIdx.x >> 5] = y;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -732,17 +737,17 @@ cudaError_t launch_fwd_exp64(const void *F, int8_t *ef, int Nf, int Nr, int Nm, 
   const int nbp = fwd_nbp(Nm);
   k_row_scan<true><<<dim3(Nf, nrows, gemm_fwd_sl64_nrange(Nm)), 256, 0, s>>>(reinterpret_cast<const float4 *>(F) + (size_t)row0 * Nm,
                                                    (long)Nr * Nm, Nm, Nm, ef + row0, Nr,
-                                                   const_cast<uint16_t *>(fwd_low(ef, Nf, Nr, Nm)) + (size_t)row0 * nbp, nbp);
+                                                   const_cast<uint16_t *>(fwd_low(ef, Nf, Nr, Nm)) + (size_t)row0 * nbp, nbp,
+                                                   nullptr);
   count_launches(1);
   return cudaGetLastError();
 }
 
-// per call: open frequencies and the number of sums on the list, exponents and block
-// sums of X^, magnitude sums, the list
+// per call: open frequencies, exponents and block sums of X^, magnitude sums
 size_t gemm_fwd_sl64_ws_bytes(int Nf, int Nr, int Nm, int B) {
   const size_t nr = gemm_fwd_sl64_nrange(Nm);
   return up16((size_t)Nf * sizeof(int)) + up16(Nf * nr * B) + (size_t)Nf * B * fwd_nbp(Nm) * sizeof(uint16_t) +
-         (size_t)Nf * Nr * B * sizeof(unsigned long long) + (1 + (size_t)Nf * Nr * B) * sizeof(int);
+         (size_t)Nf * Nr * B * sizeof(unsigned long long);
 }
 
 // Yo[b][w][r] for b < B; ef: launch_fwd_exp64; ws: gemm_fwd_sl64_ws_bytes(B).
@@ -759,12 +764,8 @@ cudaError_t launch_gemm_fwd_sl64(const void *F, const int8_t *ef, const cdd *X, 
   int *open = reinterpret_cast<int *>(wp);
   int8_t *ex = reinterpret_cast<int8_t *>(wp += up16((size_t)Nf * sizeof(int)));
   uint16_t *xsum = reinterpret_cast<uint16_t *>(wp += up16((size_t)Nf * nr * B));
-  unsigned long long *Sq = reinterpret_cast<unsigned long long *>(wp += (size_t)Nf * B * nbp * sizeof(uint16_t));
-  int *todo = reinterpret_cast<int *>(wp + (size_t)Nf * Nr * B * sizeof(unsigned long long));
-  cudaError_t e = cudaMemsetAsync(open, 0, (size_t)Nf * sizeof(int), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(todo, 0, sizeof(int), s);
-  if (e != cudaSuccess) return e;
-  k_row_scan<false><<<dim3(Nf, B, nr), 256, 0, s>>>(Xp, Nm, x_bstride, Nm, ex, B, xsum, nbp);
+  unsigned long long *Sq = reinterpret_cast<unsigned long long *>(wp + (size_t)Nf * B * nbp * sizeof(uint16_t));
+  k_row_scan<false><<<dim3(Nf, B, nr), 256, 0, s>>>(Xp, Nm, x_bstride, Nm, ex, B, xsum, nbp, open);
   k_fwd_check<<<dim3((Nr + 15) / 16, Nf, (B + 63) / 64), 256, 0, s>>>(ef, fwd_low(ef, Nf, Nr, Nm), ex, xsum, nbp, nr, Nr,
                                                                      Nm, B, open, Sq);
   count_launches(2);
@@ -805,11 +806,10 @@ cudaError_t launch_gemm_fwd_sl64(const void *F, const int8_t *ef, const cdd *X, 
   const int nrt = (Nr + 31) / 32, nbt = (B + 31) / 32;
   k_fwd_mag<<<dim3(nrt * nbt * ((Nm + SUB - 1) / SUB), Nf), 256, 0, s>>>(Fp, Xp, x_bstride, ef, ex, open, nrt, nbt, nr,
                                                                         Nr, Nm, B, Sq);
-  k_fwd_join<<<(unsigned)(((long)B * Nf * Nr + 255) / 256), 256, 0, s>>>(part, open, Sq, Yo, y_bstride, nr, Nf, Nr, B,
-                                                                        todo);
-  k_fwd_redo<<<(unsigned)std::max(1, 4 * nsm), 256, 0, s>>>(reinterpret_cast<const cdd *>(F), X, x_bstride, todo, Yo,
-                                                           y_bstride, Nf, Nr, Nm);
-  count_launches(4);
+  k_fwd_join<<<(unsigned)(((long)B * Nf * Nr + 255) / 256), 256, 0, s>>>(part, reinterpret_cast<const cdd *>(F), X,
+                                                                        x_bstride, open, Sq, Yo, y_bstride, nr, Nf,
+                                                                        Nr, Nm, B);
+  count_launches(3);
   return cudaGetLastError();
 }
 
